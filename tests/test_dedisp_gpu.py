@@ -305,6 +305,23 @@ def test_corner_turn_then_dedisperse(P, nchan, nsamp):
         np.testing.assert_array_equal(got, oracle.dedisperse(oracle.delay_table(f, 64e-6, dms), want, nsamp))
 
 
+@pytest.mark.parametrize("nchan,nsamp", [(1, 1), (60, 2047), (64, 2049), (65, 1025), (130, 513), (256, 511),
+                                         (257, 255), (513, 1000), (1030, 257)])
+def test_corner_turn_whole_words(P, nchan, nsamp):
+    """Rows of whole 32-bit words (the register transpose) at the edges of its
+    tiles: 4, 8, 16 or 32 lanes across the channels, 256 to 2048 samples per
+    tile, spare words in both strides; the padding of every row is written 0."""
+    import torch
+
+    rng = np.random.default_rng(nchan * 7 + nsamp)
+    ld_tm, ld_cm = (nchan + 15) // 16 * 4 + 8, (nsamp + 15) // 16 * 4 + 12
+    tm = rng.integers(0, 256, size=(nsamp, ld_tm), dtype=np.uint8)
+    out = torch.full((nchan, ld_cm), 0xA5, dtype=torch.uint8, device="cuda")
+    P.corner_turn(torch.from_numpy(tm).cuda(), nchan, nsamp, out)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(out.cpu().numpy(), oracle.corner_turn(tm, nchan, nsamp, ld_cm))
+
+
 def test_autotune_cache_round_trip(P, tmp_path):
     """The tuner writes its choice to the plan's cache file; a new plan of the
     same band, DMs and gulp length reads it back (no timing, 0 ms) and runs
