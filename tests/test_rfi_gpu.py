@@ -63,3 +63,12 @@ def test_bursts_over_13_beams(P):
 @pytest.mark.parametrize("nsamp,nchan,k,m", [(40001, 64, 1, 4), (17, 7, 1, 1), (4096, 130, 0, 13)])
 def test_loose_thresholds_and_ragged_sizes(P, nsamp, nchan, k, m):
     check(P, make_beams(nsamp + nchan, 13, nchan, nsamp, [(0, 3, {0, 1, 2, 3})]), nsamp, k, m)
+
+
+@pytest.mark.parametrize("nchan,nsamp", [(1, 15), (5, 16), (9, 511), (10, 512), (16, 513), (17, 1024), (74, 4100)])
+def test_channel_and_sample_remainders(P, nchan, nsamp):
+    """Channel counts around the five- and ten-channel steps of the zero-DM sum
+    and the 16-channel items of the substitution, lengths around its 512-sample
+    tiles; scattered and adjacent masked words."""
+    events = [(0, 1, {0, 1}), (nsamp // 2, 3, {1, 2}), (max(0, nsamp - 2), 2, {0, 2})]
+    check(P, make_beams(nchan * 31 + nsamp, 3, nchan, nsamp, events), nsamp, 1, 2)
