@@ -11,8 +11,8 @@
 // a product of two bfloat16 values is exact in float, so each step rounds
 // once and the result equals a plain float sum in that order.  Activations
 // after ReLU are rounded to bfloat16 (nearest even); pooling keeps the first
-// maximum.  Gradients are float; each weight gradient is a two-stage sum
-// (fixed chunks of the batch, then the chunks in order), so training is
+// maximum.  Gradients are float; each convolution weight gradient is a two-stage
+// sum (a fixed set of samples per block, then the blocks in order), so training is
 // deterministic.  These are CUDA-core kernels (~12.5 M multiply-adds per
 // snippet): the fixed summation order is what makes the logits reproducible
 // bit for bit, which the tensor cores' internal accumulation order is not.
@@ -21,6 +21,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <vector>
 
@@ -35,7 +36,7 @@ constexpr int kCin[kConvLayers] = {1, 16, 32, 64};
 constexpr int kCout[kConvLayers] = {16, 32, 64, 64};
 constexpr int kHin[kConvLayers] = {64, 32, 16, 8};
 constexpr int kFcIn = 1024, kFcHid = 128;
-constexpr int kChunk = 16;  // samples per first-stage weight-gradient partial
+constexpr int kMaxPartials = 304;  // blocks (= partials) of a convolution's weight gradient: two per SM
 
 struct Layout {
     long long cw[kConvLayers], cb[kConvLayers], f1w, f1b, f2w, f2b, total;
@@ -679,7 +680,7 @@ __global__ void __launch_bounds__(256, (ConvTcCfg<CI, CO, H, TPC>::MINB))
 
 __global__ void __launch_bounds__(1024) bce_kernel(const float *__restrict__ z, const float *__restrict__ y, int N,
                                                    float *__restrict__ dz, float *__restrict__ loss) {
-    __shared__ double s[1024];
+    __shared__ double s[32];
     double acc = 0.0;
     for (int n = threadIdx.x; n < N; n += blockDim.x) {
         const float zn = z[n];
@@ -688,145 +689,487 @@ __global__ void __launch_bounds__(1024) bce_kernel(const float *__restrict__ z, 
         const double zd = zn, yd = y[n];
         acc += (zd > 0 ? zd : 0) - zd * yd + log1p(exp(-fabs(zd)));
     }
-    s[threadIdx.x] = acc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
     __syncthreads();
-    for (int o = 512; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
+    if (threadIdx.x < 32) {
+        acc = threadIdx.x < blockDim.x / 32 ? s[threadIdx.x] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        if (threadIdx.x == 0) *loss = (float)(acc / N);
+    }
+}
+
+// fc2: block 0 sums the weight and bias gradients of fc2 and the bias
+// gradient of fc1 over the batch (8 interleaved slices, joined in order); the
+// other blocks write dh = dz * w2 where the hidden unit was active.
+__global__ void __launch_bounds__(1024) fc2_bwd_kernel(const float *__restrict__ dz, const uint16_t *__restrict__ h1,
+                                                       const uint16_t *__restrict__ w2, int N,
+                                                       float *__restrict__ g_w2, float *__restrict__ g_b2,
+                                                       float *__restrict__ g_b1, float *__restrict__ dh) {
+    const int i = threadIdx.x % kFcHid, sl = threadIdx.x / kFcHid;
+    const float w = bf2f(w2[i]);
+    if (blockIdx.x > 0) {
+        for (long long n = (long long)(blockIdx.x - 1) * 8 + sl; n < N; n += (long long)(gridDim.x - 1) * 8)
+            dh[n * kFcHid + i] = bf2f(h1[n * kFcHid + i]) > 0.0f ? dz[n] * w : 0.0f;
+        return;
+    }
+    __shared__ float s_w[8][kFcHid], s_b[8][kFcHid], s_z[8];
+    float aw = 0.0f, ab = 0.0f, az = 0.0f;
+#pragma unroll 8
+    for (int n = sl; n < N; n += 8) {
+        const float h = bf2f(h1[(long long)n * kFcHid + i]), z = dz[n];
+        aw += z * h;
+        ab += h > 0.0f ? z * w : 0.0f;
+        az += z;
+    }
+    s_w[sl][i] = aw;
+    s_b[sl][i] = ab;
+    if (i == 0) s_z[sl] = az;
+    __syncthreads();
+    if (sl == 0) {
+        for (int k = 1; k < 8; ++k) {
+            aw += s_w[k][i];
+            ab += s_b[k][i];
+            az += s_z[k];
+        }
+        g_w2[i] = aw;
+        g_b1[i] = ab;
+        if (i == 0) *g_b2 = az;
+    }
+}
+
+// fc1 weight gradient: a block owns 16 outputs x 64 inputs, a thread one
+// output x 4 inputs, the batch staged 32 samples at a time.
+__global__ void __launch_bounds__(256) fc1_bwd_w_kernel(const float *__restrict__ dh,
+                                                        const uint16_t *__restrict__ feat, int N,
+                                                        float *__restrict__ g_w1) {
+    __shared__ __align__(16) float s_f[32][64];
+    __shared__ float s_d[32][16];
+    const int tid = threadIdx.x, i0 = blockIdx.x * 64, o0 = blockIdx.y * 16;
+    const int iq = (tid & 15) * 4, o = tid >> 4;
+    // this thread's share of a stage: 8 inputs of one sample, 2 values of dh
+    const int fn = tid >> 3, fi = (tid & 7) * 8;
+    uint4 fv;
+    float d0, d1;
+    auto fetch = [&](int n0) {
+        const int n = n0 + fn, na = n0 + (tid >> 4), nb = na + 16;
+        fv = n < N ? __ldg(reinterpret_cast<const uint4 *>(feat + (long long)n * kFcIn + i0 + fi))
+                   : make_uint4(0, 0, 0, 0);
+        d0 = na < N ? __ldg(dh + (long long)na * kFcHid + o0 + (tid & 15)) : 0.0f;
+        d1 = nb < N ? __ldg(dh + (long long)nb * kFcHid + o0 + (tid & 15)) : 0.0f;
+    };
+    fetch(0);
+    float acc[4] = {};
+    for (int n0 = 0; n0 < N; n0 += 32) {
+        __syncthreads();
+        float4 *f4 = reinterpret_cast<float4 *>(&s_f[fn][fi]);
+        f4[0] = make_float4(__uint_as_float(fv.x << 16), __uint_as_float(fv.x & 0xffff0000u),
+                            __uint_as_float(fv.y << 16), __uint_as_float(fv.y & 0xffff0000u));
+        f4[1] = make_float4(__uint_as_float(fv.z << 16), __uint_as_float(fv.z & 0xffff0000u),
+                            __uint_as_float(fv.w << 16), __uint_as_float(fv.w & 0xffff0000u));
+        s_d[tid >> 4][tid & 15] = d0;
+        s_d[(tid >> 4) + 16][tid & 15] = d1;
+        __syncthreads();
+        if (n0 + 32 < N) fetch(n0 + 32);
+#pragma unroll
+        for (int n = 0; n < 32; ++n) {
+            const float4 f = *reinterpret_cast<const float4 *>(&s_f[n][iq]);
+            const float d = s_d[n][o];
+            acc[0] = fmaf(d, f.x, acc[0]);
+            acc[1] = fmaf(d, f.y, acc[1]);
+            acc[2] = fmaf(d, f.z, acc[2]);
+            acc[3] = fmaf(d, f.w, acc[3]);
+        }
+    }
+    float *dst = g_w1 + (long long)(o0 + o) * kFcIn + i0 + iq;  // 4-byte aligned only: the flat vector is unpadded
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dst[k] = acc[k];
+}
+
+// fc1 input gradient: a block owns 16 samples x 64 inputs.
+__global__ void __launch_bounds__(256) fc1_bwd_x_kernel(const float *__restrict__ dh, const uint16_t *__restrict__ w1,
+                                                        int N, float *__restrict__ dfeat) {
+    __shared__ __align__(16) float s_w[kFcHid][64];
+    __shared__ float s_d[16][kFcHid];
+    const int tid = threadIdx.x, i0 = blockIdx.y * 64, n0 = blockIdx.x * 16;
+#pragma unroll
+    for (int k = 0; k < kFcHid * 8 / 256; ++k) {
+        const int e = tid + 256 * k, o = e >> 3, i8 = (e & 7) * 8;
+        const uint4 q = __ldg(reinterpret_cast<const uint4 *>(w1 + (long long)o * kFcIn + i0 + i8));
+        float4 *f4 = reinterpret_cast<float4 *>(&s_w[o][i8]);
+        f4[0] = make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u),
+                            __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
+        f4[1] = make_float4(__uint_as_float(q.z << 16), __uint_as_float(q.z & 0xffff0000u),
+                            __uint_as_float(q.w << 16), __uint_as_float(q.w & 0xffff0000u));
+    }
+#pragma unroll
+    for (int k = 0; k < 16 * kFcHid / 256; ++k) {
+        const int e = tid + 256 * k, n = n0 + e / kFcHid;
+        s_d[e / kFcHid][e % kFcHid] = n < N ? __ldg(dh + (long long)n * kFcHid + e % kFcHid) : 0.0f;
+    }
+    __syncthreads();
+    const int iq = (tid & 15) * 4, r = tid >> 4;
+    float acc[4] = {};
+#pragma unroll 16
+    for (int o = 0; o < kFcHid; ++o) {
+        const float4 f = *reinterpret_cast<const float4 *>(&s_w[o][iq]);
+        const float d = s_d[r][o];
+        acc[0] = fmaf(d, f.x, acc[0]);
+        acc[1] = fmaf(d, f.y, acc[1]);
+        acc[2] = fmaf(d, f.z, acc[2]);
+        acc[3] = fmaf(d, f.w, acc[3]);
+    }
+    if (n0 + r < N)
+        *reinterpret_cast<float4 *>(dfeat + (long long)(n0 + r) * kFcIn + i0 + iq) =
+            make_float4(acc[0], acc[1], acc[2], acc[3]);
+}
+
+// Gradient of a convolution's pooled output routed to the one position of
+// each 2x2 window that pooling kept (0 elsewhere, and 0 where the ReLU cut).
+__device__ __forceinline__ float live_grad(float d, uint16_t pooled) { return bf2f(pooled) > 0.0f ? d : 0.0f; }
+
+// Input gradient of a 3x3 convolution: din[n][ci] = sum over (co, taps) of the
+// routed output gradient times the flipped weights, a convolution over CO
+// channels whose input is expanded to float as it is staged.  FMA-bound like
+// the forward kernel and tiled like it: a thread owns 8 input channels x a 2x4
+// block of pixels (288 packed FMAs per output channel from a 4x6 patch and 9x8
+// weights), a block 16 input channels of SPB samples, so that the 18-37 KB of
+// weights and two stages of 8 output channels leave room for several blocks
+// per SM.  The next stage's gradients wait in registers.  Sums run over co,
+// then the taps.  The one-thread-per-pixel form this replaces read every
+// gradient 9 CI times: 4290 us for the three layers at 256 snippets, 153 us
+// with this one (3 G multiply-adds: half the packed-FMA rate; 256 blocks leave
+// a third of the SMs with one block instead of two).
+template <int CI, int CO, int H>
+struct ConvBwdXCfg {
+    static constexpr int CIB = 16;                    // input channels per block
+    static constexpr int COC = 8;                     // output channels per stage
+    static constexpr int PT = (H / 2) * (H / 4);      // 2x4 pixel tiles per sample
+    static constexpr int THREADS = PT * 2 >= 128 ? PT * 2 : 128;
+    static constexpr int SPB = THREADS / (PT * 2);    // samples per block
+    // row stride: zeros at H..RS-1 are the right halo and the next row's left
+    // one; 24 for H = 16 puts a quarter-warp's two rows into different banks
+    static constexpr int RS = H == 16 ? 24 : H + 4;
+    static constexpr int CH = (H + 1) * RS;
+    static constexpr int SNIP = 4 + (COC * (H + 1) + 1) * RS;  // staged floats per sample
+    static constexpr int BUF = SPB * SNIP;
+    static constexpr size_t SMEM = (size_t)(CO * 9 * CIB + 2 * BUF) * 4;
+    static constexpr int QUADS = SPB * COC * (H / 2) * (H / 8);  // 4-window groups per stage
+    static constexpr int QPT = QUADS / THREADS;
+    static_assert(QUADS % THREADS == 0 && CO % COC == 0 && CI % CIB == 0 && RS % 4 == 0, "tile shape");
+};
+
+template <int CI, int CO, int H>
+__global__ void __launch_bounds__((ConvBwdXCfg<CI, CO, H>::THREADS))
+    conv_bwd_x_kernel(const float *__restrict__ dpool, const uint16_t *__restrict__ pooled,
+                      const uint8_t *__restrict__ arg, const uint16_t *__restrict__ w, int N,
+                      float *__restrict__ din) {
+    using C = ConvBwdXCfg<CI, CO, H>;
+    constexpr int HO = H / 2, CIB = C::CIB, T = C::THREADS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    float *ws = reinterpret_cast<float *>(smem);  // [co][flipped tap][ci]
+    float *gs = ws + CO * 9 * CIB;
+    const int tid = threadIdx.x;
+    const int ci0 = blockIdx.y * CIB, n0 = blockIdx.x * C::SPB;
+    for (int i = tid; i < 2 * C::BUF / 4; i += T) reinterpret_cast<float4 *>(gs)[i] = make_float4(0, 0, 0, 0);
+    for (int e = tid; e < CO * CIB * 9; e += T) {
+        const int k = e % 9, c = (e / 9) % CIB, co = e / (9 * CIB);
+        ws[(co * 9 + 8 - k) * CIB + c] = bf2f(__ldg(w + ((long long)co * CI + ci0 + c) * 9 + k));
+    }
+    // a stage's 4-window groups: sample j, channel cl, window row yo, windows 4 xq .. 4 xq + 3
+    float4 d4[C::QPT];
+    uint2 p4[C::QPT];
+    uint32_t a4[C::QPT];
+    auto fetch = [&](int s) {
+#pragma unroll
+        for (int k = 0; k < C::QPT; ++k) {
+            const int e = tid + k * T;
+            const int xq = e % (HO / 4), yo = (e / (HO / 4)) % HO, cl = (e / (HO / 4 * HO)) % C::COC;
+            const int n = n0 + e / (HO / 4 * HO * C::COC);
+            const long long o = (((long long)n * CO + s * C::COC + cl) * HO + yo) * HO + 4 * xq;
+            const bool ok = n < N;
+            d4[k] = ok ? __ldg(reinterpret_cast<const float4 *>(dpool + o)) : make_float4(0, 0, 0, 0);
+            p4[k] = ok ? __ldg(reinterpret_cast<const uint2 *>(pooled + o)) : make_uint2(0, 0);
+            a4[k] = ok ? __ldg(reinterpret_cast<const uint32_t *>(arg + o)) : 0u;
+        }
+    };
+    auto expand = [&](int s) {
+#pragma unroll
+        for (int k = 0; k < C::QPT; ++k) {
+            const int e = tid + k * T;
+            const int xq = e % (HO / 4), yo = (e / (HO / 4)) % HO, cl = (e / (HO / 4 * HO)) % C::COC;
+            const int j = e / (HO / 4 * HO * C::COC);
+            const float g[4] = {live_grad(d4[k].x, (uint16_t)p4[k].x), live_grad(d4[k].y, (uint16_t)(p4[k].x >> 16)),
+                                live_grad(d4[k].z, (uint16_t)p4[k].y), live_grad(d4[k].w, (uint16_t)(p4[k].y >> 16))};
+            float *dst = gs + (s & 1) * C::BUF + j * C::SNIP + 4 + (cl * (H + 1) + 2 * yo + 1) * C::RS + 8 * xq;
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                float v[8];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t a = (a4[k] >> (8 * i)) & 0xFFu;
+                    v[2 * i] = a == 2 * r ? g[i] : 0.0f;
+                    v[2 * i + 1] = a == 2 * r + 1 ? g[i] : 0.0f;
+                }
+                float4 *d = reinterpret_cast<float4 *>(dst + r * C::RS);
+                d[0] = make_float4(v[0], v[1], v[2], v[3]);
+                d[1] = make_float4(v[4], v[5], v[6], v[7]);
+            }
+        }
+    };
+    const int pt = tid % C::PT, ct = (tid / C::PT) % 2, sj = tid / (2 * C::PT);
+    const int ty = pt / (H / 4), tx = pt % (H / 4);
+    uint64_t acc[4][2][4];
+#pragma unroll
+    for (int cp = 0; cp < 4; ++cp)
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[cp][r][q] = 0ull;
+    fetch(0);
+    __syncthreads();
+    expand(0);
+    __syncthreads();
+    constexpr int NS = CO / C::COC;
+#pragma unroll 1
+    for (int s = 0; s < NS; ++s) {
+        if (s + 1 < NS) fetch(s + 1);
+        // padded row Y = 0..H+1 of a channel starts at 4 + (cl(H+1) + Y) RS; patch column 4tx - 1
+        const float *xb = gs + (s & 1) * C::BUF + sj * C::SNIP + 4 + 2 * ty * C::RS + 4 * tx;
+        const float *wb = ws + s * C::COC * 9 * CIB + ct * 8;
+#pragma unroll 1
+        for (int cl = 0; cl < C::COC; ++cl) {
+            uint64_t p[4][6];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float *row = xb + cl * C::CH + r * C::RS;
+                const float l = row[-1], h = row[4];
+                const float4 m = *reinterpret_cast<const float4 *>(row);
+                const float v[6] = {l, m.x, m.y, m.z, m.w, h};
+#pragma unroll
+                for (int k = 0; k < 6; ++k) p[r][k] = pk2(v[k], v[k]);
+            }
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const float4 wa = *reinterpret_cast<const float4 *>(wb + (cl * 9 + t) * CIB);
+                const float4 wc = *reinterpret_cast<const float4 *>(wb + (cl * 9 + t) * CIB + 4);
+                const uint64_t wv[4] = {pk2(wa.x, wa.y), pk2(wa.z, wa.w), pk2(wc.x, wc.y), pk2(wc.z, wc.w)};
+#pragma unroll
+                for (int cp = 0; cp < 4; ++cp)
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            acc[cp][r][q] = ffma2(wv[cp], p[r + t / 3][q + t % 3], acc[cp][r][q]);
+            }
+        }
+        if (s + 1 < NS) expand(s + 1);  // the other buffer: its readers passed the previous barrier
         __syncthreads();
     }
-    if (threadIdx.x == 0) *loss = (float)(s[0] / N);
-}
-
-__global__ void fc2_bwd_kernel(const float *__restrict__ dz, const uint16_t *__restrict__ h1,
-                               const uint16_t *__restrict__ w2, int N, float *__restrict__ g_w2,
-                               float *__restrict__ g_b2, float *__restrict__ dh) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < kFcHid) {
-        float acc = 0.0f;
-        for (int n = 0; n < N; ++n) acc += dz[n] * bf2f(h1[n * kFcHid + idx]);
-        g_w2[idx] = acc;
-    } else if (idx == kFcHid) {
-        float acc = 0.0f;
-        for (int n = 0; n < N; ++n) acc += dz[n];
-        *g_b2 = acc;
-    }
-    for (int k = idx; k < N * kFcHid; k += gridDim.x * blockDim.x) {
-        const int i = k % kFcHid, n = k / kFcHid;
-        dh[k] = bf2f(h1[k]) > 0.0f ? dz[n] * bf2f(w2[i]) : 0.0f;
-    }
-}
-
-__global__ void fc1_bwd_w_kernel(const float *__restrict__ dh, const uint16_t *__restrict__ feat, int N,
-                                 float *__restrict__ g_w1, float *__restrict__ g_b1) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < kFcHid * kFcIn) {
-        const int i = idx % kFcIn, o = idx / kFcIn;
-        float acc = 0.0f;
-        for (int n = 0; n < N; ++n) acc += dh[n * kFcHid + o] * bf2f(feat[(long long)n * kFcIn + i]);
-        g_w1[idx] = acc;
-    } else if (idx < kFcHid * kFcIn + kFcHid) {
-        const int o = idx - kFcHid * kFcIn;
-        float acc = 0.0f;
-        for (int n = 0; n < N; ++n) acc += dh[n * kFcHid + o];
-        g_b1[o] = acc;
-    }
-}
-
-__global__ void fc1_bwd_x_kernel(const float *__restrict__ dh, const uint16_t *__restrict__ w1, int N,
-                                 float *__restrict__ dfeat) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * kFcIn) return;
-    const int i = idx % kFcIn, n = idx / kFcIn;
-    float acc = 0.0f;
-    for (int o = 0; o < kFcHid; ++o) acc += dh[n * kFcHid + o] * bf2f(w1[(long long)o * kFcIn + i]);
-    dfeat[idx] = acc;
-}
-
-// gradient reaching pre-pool position (y, x) of channel co: only the pooled
-// maximum receives it, and only when it passed the ReLU
-template <int CO, int H>
-__device__ __forceinline__ float routed(const float *dpool, const uint16_t *pooled, const uint8_t *arg, int n, int co,
-                                        int y, int x) {
-    constexpr int HO = H / 2;
-    const long long o = (((long long)n * CO + co) * HO + (y >> 1)) * HO + (x >> 1);
-    if (arg[o] != ((y & 1) << 1 | (x & 1))) return 0.0f;
-    if (!(bf2f(pooled[o]) > 0.0f)) return 0.0f;
-    return dpool[o];
-}
-
-// stage 1: partial[chunk][wi] over the samples of the chunk (wi < CO*CI*9 weights, then CO biases)
-template <int CI, int CO, int H>
-__global__ void conv_bwd_w_kernel(const float *__restrict__ dpool, const uint16_t *__restrict__ pooled,
-                                  const uint8_t *__restrict__ arg, const uint16_t *__restrict__ in, int N,
-                                  float *__restrict__ partial) {
-    constexpr int HO = H / 2;
-    constexpr int NW = CO * CI * 9 + CO;
-    const int wi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int chunk = blockIdx.y;
-    if (wi >= NW) return;
-    const int n0 = chunk * kChunk, n1 = min(N, n0 + kChunk);
-    float acc = 0.0f;
-    if (wi < CO * CI * 9) {
-        const int kx = wi % 3, ky = (wi / 3) % 3, ci = (wi / 9) % CI, co = wi / (9 * CI);
-        for (int n = n0; n < n1; ++n) {
-            const uint16_t *src = in + ((long long)n * CI + ci) * H * H;
-            for (int yo = 0; yo < HO; ++yo)
-                for (int xo = 0; xo < HO; ++xo) {
-                    const long long o = (((long long)n * CO + co) * HO + yo) * HO + xo;
-                    if (!(bf2f(pooled[o]) > 0.0f)) continue;
-                    const int q = arg[o];
-                    const int yy = 2 * yo + (q >> 1) + ky - 1, xx = 2 * xo + (q & 1) + kx - 1;
-                    if (yy < 0 || yy >= H || xx < 0 || xx >= H) continue;
-                    acc += dpool[o] * bf2f(src[yy * H + xx]);
-                }
+    const int n = n0 + sj;
+    if (n >= N) return;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            float v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = (c & 1) ? hi_f(acc[c / 2][r][q]) : lo_f(acc[c / 2][r][q]);
+            *reinterpret_cast<float4 *>(din + (((long long)n * CI + ci0 + ct * 8 + c) * H + 2 * ty + r) * H + 4 * tx) =
+                make_float4(v[0], v[1], v[2], v[3]);
         }
-    } else {
-        const int co = wi - CO * CI * 9;
-        for (int n = n0; n < n1; ++n)
-            for (int k = 0; k < HO * HO; ++k) {
-                const long long o = ((long long)n * CO + co) * HO * HO + k;
-                if (bf2f(pooled[o]) > 0.0f) acc += dpool[o];
-            }
-    }
-    partial[(long long)chunk * NW + wi] = acc;
 }
 
-// stage 2: sum the chunks in order into the weight and bias gradients
-__global__ void conv_bwd_w_sum_kernel(const float *__restrict__ partial, int nchunks, int nw_weights, int nbias,
-                                      float *__restrict__ g_w, float *__restrict__ g_b) {
-    const int wi = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nw = nw_weights + nbias;
-    if (wi >= nw) return;
-    float acc = 0.0f;
-    for (int c = 0; c < nchunks; ++c) acc += partial[(long long)c * nw + wi];
-    if (wi < nw_weights) g_w[wi] = acc;
-    else g_b[wi - nw_weights] = acc;
+// Weight gradient of a 3x3 convolution: only one position per 2x2 window
+// carries a gradient, so a thread (one output channel, 4 input channels, all 9
+// taps: 36 sums) walks the windows of a sample, each a gradient, the position
+// that pooling kept and the 3x3 input patch around it: a quarter of the dense
+// multiply-adds.  A sample's input sits in shared memory channel-last with a
+// zero border (a lane's 4 channels are one 8-byte load, the lanes of one
+// output channel consecutive), its (gradient, patch offset) pairs beside it.
+// A block walks samples blockIdx.x, + gridDim.x, ...; its sums (SL window
+// slices joined in order) are one partial, and conv_bwd_w_sum_kernel adds the
+// partials in order, so the result is deterministic.  Issue-bound: about 64
+// instructions per 36 multiply-adds of a window.  (One thread per weight
+// reading the gradients from memory: 4470 us for the four layers at 256
+// snippets, 144 us with these and their sums.)
+template <int CI, int CO, int H, int COB, int SL>
+struct ConvBwdWCfg {
+    static constexpr int HO = H / 2, NWIN = HO * HO;
+    static constexpr int CQ = CI / 4;                // lanes of one output channel
+    static constexpr int THREADS = SL * COB * CQ;
+    static constexpr int GS = NWIN + 1;              // padded row of (gradient, offset) pairs
+    static constexpr int PIX = CI * 2;               // bytes of a pixel
+    static constexpr int IN_BYTES = (H + 2) * (H + 2) * PIX;
+    static constexpr int RED_BYTES = SL > 1 ? (SL - 1) * COB * CQ * 37 * 4 : 0;  // slices' sums, in the pairs' place
+    static constexpr int GP_BYTES = COB * GS * 8;
+    static constexpr size_t SMEM = (size_t)IN_BYTES + (GP_BYTES > RED_BYTES ? GP_BYTES : RED_BYTES);
+    static constexpr int NW = CO * CI * 9 + CO;
+    static_assert(CI % 4 == 0 && CO % COB == 0 && NWIN % SL == 0 && THREADS % 32 == 0, "tile shape");
+};
+
+template <int CI, int CO, int H, int COB, int SL>
+__global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
+    conv_bwd_w_kernel(const float *__restrict__ dpool, const uint16_t *__restrict__ pooled,
+                      const uint8_t *__restrict__ arg, const uint16_t *__restrict__ in, int N,
+                      float *__restrict__ partial) {
+    using C = ConvBwdWCfg<CI, CO, H, COB, SL>;
+    constexpr int HO = C::HO, T = C::THREADS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    unsigned char *xin = smem;
+    uint2 *gp = reinterpret_cast<uint2 *>(smem + C::IN_BYTES);
+    const int tid = threadIdx.x, co0 = blockIdx.y * COB;
+    const int cq = tid % C::CQ, co = (tid / C::CQ) % COB, sl = tid / (C::CQ * COB);
+    for (int i = tid; i < C::IN_BYTES / 8; i += T) reinterpret_cast<uint2 *>(xin)[i] = make_uint2(0, 0);
+    uint64_t acc[9][2];  // taps x two channel pairs
+#pragma unroll
+    for (int t = 0; t < 9; ++t) acc[t][0] = acc[t][1] = 0ull;
+    float bacc = 0.0f;
+#pragma unroll 1
+    for (int n = blockIdx.x; n < N; n += gridDim.x) {
+        __syncthreads();  // zeros written; the previous sample consumed
+        // input, channel-last: two neighbouring pixels of 4 channels at a time
+#pragma unroll 4
+        for (int e = tid; e < C::CQ * H * (H / 2); e += T) {
+            const int x2 = e % (H / 2), y = (e / (H / 2)) % H, q = e / (H / 2 * H);
+            uint32_t v[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                v[c] = __ldg(reinterpret_cast<const uint32_t *>(in + (((long long)n * CI + 4 * q + c) * H + y) * H +
+                                                                 2 * x2));
+            unsigned char *dst = xin + ((y + 1) * (H + 2) + 2 * x2 + 1) * C::PIX + 8 * q;
+            *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410));
+            *reinterpret_cast<uint2 *>(dst + C::PIX) =
+                make_uint2(__byte_perm(v[0], v[1], 0x7632), __byte_perm(v[2], v[3], 0x7632));
+        }
+#pragma unroll 4
+        for (int e = tid; e < COB * C::NWIN; e += T) {
+            const int k = e % C::NWIN, c = e / C::NWIN;
+            const long long o = ((long long)n * CO + co0 + c) * C::NWIN + k;
+            const int a = __ldg(arg + o);
+            // patch around (2 yo + a/2, 2 xo + a%2): its corner in padded coordinates is that position
+            const int off = ((2 * (k / HO) + (a >> 1)) * (H + 2) + 2 * (k % HO) + (a & 1)) * C::PIX;
+            gp[c * C::GS + k] = make_uint2(__float_as_uint(live_grad(__ldg(dpool + o), __ldg(pooled + o))), (uint32_t)off);
+        }
+        __syncthreads();
+        const uint2 *g = gp + co * C::GS + sl * (C::NWIN / SL);
+        const unsigned char *xb = xin + 8 * cq;
+#pragma unroll 2
+        for (int k = 0; k < C::NWIN / SL; ++k) {
+            const uint2 e = g[k];
+            const float gv = __uint_as_float(e.x);
+            const uint64_t g2 = pk2(gv, gv);
+            bacc += gv;
+            const unsigned char *px = xb + e.y;
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(px + ((t / 3) * (H + 2) + t % 3) * C::PIX);
+                acc[t][0] = ffma2(g2, pk2(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u)), acc[t][0]);
+                acc[t][1] = ffma2(g2, pk2(__uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u)), acc[t][1]);
+            }
+        }
+    }
+    float a[37];
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            a[(2 * p) * 9 + t] = lo_f(acc[t][p]);
+            a[(2 * p + 1) * 9 + t] = hi_f(acc[t][p]);
+        }
+    a[36] = bacc;
+    if constexpr (SL > 1) {
+        float *red = reinterpret_cast<float *>(smem + C::IN_BYTES);
+        constexpr int M = COB * C::CQ;  // threads of a slice
+        __syncthreads();
+        if (sl > 0)
+#pragma unroll
+            for (int i = 0; i < 37; ++i) red[((sl - 1) * 37 + i) * M + tid % M] = a[i];
+        __syncthreads();
+        if (sl > 0) return;
+        for (int s = 0; s < SL - 1; ++s)
+#pragma unroll
+            for (int i = 0; i < 37; ++i) a[i] += red[(s * 37 + i) * M + tid];
+    }
+    // sum i = 9 (channel of the 4) + tap of thread (co, cq): [36][CO][CQ], then the
+    // biases, so that neighbouring threads write neighbouring floats (in weight
+    // order a store touched 32 sectors and the 64x64 layer took 61 us at 256 snippets, 18 us
+    // this way)
+    float *dst = partial + (long long)blockIdx.x * C::NW;
+#pragma unroll
+    for (int i = 0; i < 36; ++i) dst[(i * CO + co0 + co) * C::CQ + cq] = a[i];
+    if (cq == 0) dst[CO * CI * 9 + co0 + co] = a[36];
 }
 
-// gradient w.r.t. the layer input (the previous layer's pooled output)
-template <int CI, int CO, int H>
-__global__ void conv_bwd_x_kernel(const float *__restrict__ dpool, const uint16_t *__restrict__ pooled,
-                                  const uint8_t *__restrict__ arg, const uint16_t *__restrict__ w, int N,
-                                  float *__restrict__ din) {
-    const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (long long)N * CI * H * H) return;
-    const int xx = (int)(idx % H), yy = (int)((idx / H) % H);
-    const int ci = (int)((idx / (H * H)) % CI);
-    const int n = (int)(idx / ((long long)H * H * CI));
-    float acc = 0.0f;
-    for (int co = 0; co < CO; ++co) {
-        const uint16_t *wk = w + ((long long)co * CI + ci) * 9;
+// The first layer (one input channel): warp w owns output channel w, its lanes
+// the windows of a row, 9 sums each; the sample's image sits in shared memory
+// as float with a zero border.
+__global__ void __launch_bounds__(512) conv0_bwd_w_kernel(const float *__restrict__ dpool,
+                                                          const uint16_t *__restrict__ pooled,
+                                                          const uint8_t *__restrict__ arg,
+                                                          const uint16_t *__restrict__ in, int N,
+                                                          float *__restrict__ partial) {
+    constexpr int H = 64, HO = 32, CO = 16, RS = H + 2;
+    __shared__ float img[RS * RS];
+    const int tid = threadIdx.x, co = tid >> 5, lane = tid & 31;
+    for (int i = tid; i < RS * RS; i += 512) img[i] = 0.0f;
+    float acc[10] = {};  // 9 taps and the bias
+#pragma unroll 1
+    for (int n = blockIdx.x; n < N; n += gridDim.x) {
+        __syncthreads();
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
+        for (int k = 0; k < H * H / 2 / 512; ++k) {
+            const int e = tid + 512 * k, y = e / (H / 2), x2 = e % (H / 2);
+            const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(in + ((long long)n * H + y) * H) + x2);
+            float *dst = img + (y + 1) * RS + 2 * x2 + 1;
+            dst[0] = __uint_as_float(v << 16);
+            dst[1] = __uint_as_float(v & 0xffff0000u);
+        }
+        __syncthreads();
+        const long long o = ((long long)n * CO + co) * HO * HO + lane;
+#pragma unroll 4
+        for (int yo = 0; yo < HO; ++yo) {
+            const int a = __ldg(arg + o + yo * HO);
+            const float g = live_grad(__ldg(dpool + o + yo * HO), __ldg(pooled + o + yo * HO));
+            const float *px = img + (2 * yo + (a >> 1)) * RS + 2 * lane + (a & 1);
 #pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-                const int y = yy - ky + 1, x = xx - kx + 1;
-                if (y < 0 || y >= H || x < 0 || x >= H) continue;
-                const float g = routed<CO, H>(dpool, pooled, arg, n, co, y, x);
-                if (g != 0.0f) acc += g * bf2f(wk[ky * 3 + kx]);
-            }
+            for (int t = 0; t < 9; ++t) acc[t] = fmaf(g, px[(t / 3) * RS + t % 3], acc[t]);
+            acc[9] += g;
+        }
     }
-    din[idx] = acc;
+    float *dst = partial + (long long)blockIdx.x * (CO * 9 + CO);
+#pragma unroll
+    for (int t = 0; t < 10; ++t) {
+        float v = acc[t];
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+        if (lane == 0) dst[t < 9 ? co * 9 + t : CO * 9 + co] = v;
+    }
+}
+
+// Sum the blocks' partials into the weight and bias gradients: 32 weights per
+// block, 8 interleaved slices of the partials joined in order.  cocq > 0: the
+// weights come as [36][co][cq] (conv_bwd_w_kernel), cocq = CO * CI / 4;
+// 0: in weight order.
+__global__ void __launch_bounds__(256) conv_bwd_w_sum_kernel(const float *__restrict__ partial, int nparts,
+                                                             int nw_weights, int nbias, int cocq,
+                                                             float *__restrict__ g_w, float *__restrict__ g_b) {
+    __shared__ float s[8][32];
+    const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
+    const int wi = blockIdx.x * 32 + lane, nw = nw_weights + nbias;
+    float acc = 0.0f;
+    if (wi < nw)
+#pragma unroll 8
+        for (int c = sl; c < nparts; c += 8) acc += __ldg(partial + (long long)c * nw + wi);
+    s[sl][lane] = acc;
+    __syncthreads();
+    if (sl > 0 || wi >= nw) return;
+#pragma unroll
+    for (int k = 1; k < 8; ++k) acc += s[k][lane];
+    if (wi >= nw_weights) g_b[wi - nw_weights] = acc;
+    else g_w[cocq > 0 ? wi % cocq * 36 + wi / cocq : wi] = acc;
 }
 
 // ---- optimiser -------------------------------------------------------------------
@@ -1012,7 +1355,7 @@ dd_status dd_nn_create(dd_nn **out, int max_batch) {
     size_t part = 0;
     for (int l = 0; l < kConvLayers; ++l) {
         const size_t nw = (size_t)kCout[l] * kCin[l] * 9 + kCout[l];
-        part = std::max(part, nw * ((nb + kChunk - 1) / kChunk));
+        part = std::max(part, nw * std::min<size_t>(nb, kMaxPartials));
     }
     if (e == cudaSuccess) e = cudaMalloc(&p->partial, part * 4);
     if (e == cudaSuccess) e = cudaMalloc(&p->tc_err, 4);
@@ -1101,32 +1444,37 @@ dd_status dd_nn_backward(dd_nn *nn, const uint16_t *d_x, const float *d_labels, 
     if (st != DD_OK) return st;
     const Layout &L = p->L;
     float *g = p->grad;
-    bce_kernel<<<1, 1024, 0, s>>>(p->z, d_labels, n, p->dz, p->loss);
-    fc2_bwd_kernel<<<(n * kFcHid + 255) / 256, 256, 0, s>>>(p->dz, p->h1, p->bf + L.f2w, n, g + L.f2w, g + L.f2b,
-                                                            p->dh);
-    fc1_bwd_w_kernel<<<(kFcHid * kFcIn + kFcHid + 255) / 256, 256, 0, s>>>(p->dh, p->pooled[3], n, g + L.f1w,
-                                                                          g + L.f1b);
-    fc1_bwd_x_kernel<<<(n * kFcIn + 255) / 256, 256, 0, s>>>(p->dh, p->bf + L.f1w, n, p->dpool[3]);
-    const int nchunks = (n + kChunk - 1) / kChunk;
-#define DD_CONV_BWD(l, CI, CO, H, INPTR)                                                                      \
+    bce_kernel<<<1, n <= 256 ? 256 : 1024, 0, s>>>(p->z, d_labels, n, p->dz, p->loss);
+    fc2_bwd_kernel<<<1 + std::min((n + 7) / 8, 2 * p->nsm), 1024, 0, s>>>(p->dz, p->h1, p->bf + L.f2w, n, g + L.f2w,
+                                                                          g + L.f2b, g + L.f1b, p->dh);
+    fc1_bwd_w_kernel<<<dim3(kFcIn / 64, kFcHid / 16), 256, 0, s>>>(p->dh, p->pooled[3], n, g + L.f1w);
+    fc1_bwd_x_kernel<<<dim3((unsigned)((n + 15) / 16), kFcIn / 64), 256, 0, s>>>(p->dh, p->bf + L.f1w, n, p->dpool[3]);
+    const int parts = std::min(n, kMaxPartials);
+#define DD_CONV_BWD(l, CI, CO, H, COB, SL)                                                                    \
     {                                                                                                         \
-        constexpr int NW = CO * CI * 9 + CO;                                                                  \
-        dim3 gw((NW + 127) / 128, nchunks);                                                                   \
-        conv_bwd_w_kernel<CI, CO, H><<<gw, 128, 0, s>>>(p->dpool[l], p->pooled[l], p->arg[l], INPTR, n,       \
-                                                         p->partial);                                         \
-        conv_bwd_w_sum_kernel<<<(NW + 255) / 256, 256, 0, s>>>(p->partial, nchunks, CO * CI * 9, CO,          \
-                                                               g + L.cw[l], g + L.cb[l]);                     \
-        if (l > 0) {                                                                                          \
-            const long long tot = (long long)n * CI * H * H;                                                  \
-            conv_bwd_x_kernel<CI, CO, H><<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(                      \
-                p->dpool[l], p->pooled[l], p->arg[l], p->bf + L.cw[l], n, (l) > 0 ? p->dpool[(l) - 1] : nullptr); \
-        }                                                                                                     \
+        using CW = ConvBwdWCfg<CI, CO, H, COB, SL>;                                                           \
+        using CX = ConvBwdXCfg<CI, CO, H>;                                                                    \
+        auto kw = conv_bwd_w_kernel<CI, CO, H, COB, SL>;                                                      \
+        auto kx = conv_bwd_x_kernel<CI, CO, H>;                                                               \
+        cudaError_t e = cudaFuncSetAttribute(kw, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CW::SMEM); \
+        if (e == cudaSuccess)                                                                                 \
+            e = cudaFuncSetAttribute(kx, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CX::SMEM);         \
+        if (e != cudaSuccess) return cuda_fail(e, "classifier backward");                                     \
+        const int pw = std::min(n, kMaxPartials / (CO / COB));                                                \
+        kw<<<dim3(pw, CO / COB), CW::THREADS, CW::SMEM, s>>>(p->dpool[l], p->pooled[l], p->arg[l],            \
+                                                                p->pooled[(l) - 1], n, p->partial);           \
+        conv_bwd_w_sum_kernel<<<(CW::NW + 31) / 32, 256, 0, s>>>(p->partial, pw, CO * CI * 9, CO, CO * CW::CQ,  \
+                                                                 g + L.cw[l], g + L.cb[l]);                     \
+        kx<<<dim3((unsigned)((n + CX::SPB - 1) / CX::SPB), CI / CX::CIB), CX::THREADS, CX::SMEM, s>>>(        \
+            p->dpool[l], p->pooled[l], p->arg[l], p->bf + L.cw[l], n, p->dpool[(l) - 1]);                     \
     }
-    DD_CONV_BWD(3, 64, 64, 8, p->pooled[2])
-    DD_CONV_BWD(2, 32, 64, 16, p->pooled[1])
-    DD_CONV_BWD(1, 16, 32, 32, p->pooled[0])
-    DD_CONV_BWD(0, 1, 16, 64, d_x)
+    DD_CONV_BWD(3, 64, 64, 8, 32, 1)
+    DD_CONV_BWD(2, 32, 64, 16, 64, 1)
+    DD_CONV_BWD(1, 16, 32, 32, 32, 4)
 #undef DD_CONV_BWD
+    conv0_bwd_w_kernel<<<parts, 512, 0, s>>>(p->dpool[0], p->pooled[0], p->arg[0], d_x, n, p->partial);
+    conv_bwd_w_sum_kernel<<<(16 * 9 + 16 + 31) / 32, 256, 0, s>>>(p->partial, parts, 16 * 9, 16, 0, g + L.cw[0],
+                                                                  g + L.cb[0]);
     return cuda_fail(cudaGetLastError(), "classifier backward");
 }
 

@@ -229,3 +229,36 @@ def test_training_reduces_loss(P):
     xt, yt = toy_batch(np.random.default_rng(99), 128)
     z = c.forward(to_dev(xt)).cpu().numpy()
     assert np.mean((z > 0) == (yt > 0.5)) > 0.9
+
+
+@pytest.mark.parametrize("n", [1, 9, 17])
+def test_backward_ragged_batches(P, n):
+    """Batches that leave partial blocks in every backward kernel (1, 2 and 8
+    snippets per input-gradient block, 16 and 32 in the fully connected ones)."""
+    import torch
+
+    p = params_with_biases(P, n)
+    x = snippets(60 + n, n)
+    y = (np.arange(n) % 2).astype(np.float32)
+    c = P.Classifier(max_batch=n, params=p)
+    c.backward(to_dev(x), torch.from_numpy(y).cuda())
+    loss_or, g_or, _ = oracle.nn_backward(p, x, y, round_bf16=True)
+    assert float(np.abs(c.grads() - g_or).max()) <= 1e-4 * float(np.abs(g_or).max())
+    assert abs(c.loss() - loss_or) <= 1e-6 * max(1.0, abs(loss_or))
+
+
+def test_backward_of_a_batch_is_the_mean_of_its_halves(P):
+    """626 snippets: more than one sample per weight-gradient block, in uneven
+    numbers.  The gradient is a mean over the batch, so it equals the mean of
+    the halves' gradients up to the float rounding of sums of 313 terms."""
+    import torch
+
+    p = params_with_biases(P, 2)
+    x, y = to_dev(snippets(77, 626)), torch.from_numpy((np.arange(626) % 3 == 0).astype(np.float32)).cuda()
+    c = P.Classifier(max_batch=626, params=p)
+    got = []
+    for lo, hi in ((0, 626), (0, 313), (313, 626)):
+        c.backward(x[lo:hi].contiguous(), y[lo:hi].contiguous())
+        got.append(c.grads().astype(np.float64))
+    want = 0.5 * (got[1] + got[2])
+    assert float(np.abs(got[0] - want).max()) <= 1e-5 * float(np.abs(want).max())
