@@ -75,7 +75,7 @@ __device__ __forceinline__ uint16_t f2bf(float f) {
 // pooled outputs side by side): per input channel it reads a 4x6 input patch
 // and 9x8 weights from shared memory and issues 576 FMAs.  One 512-thread
 // block per SM keeps the weights of its COB output channels resident
-// ([ci][tap][co], float, copied from a per-call float image) and walks groups
+// ([ci][tap][co], float, copied from a float image) and walks groups
 // of SPB snippets; each group's inputs arrive in stages of CIC input channels
 // by 4-byte cp.async copies into a ring of NBUF buffers, so the copies of
 // the next NBUF - 1 stages overlap the FMAs of this one.
@@ -94,15 +94,13 @@ __device__ __forceinline__ uint16_t f2bf(float f) {
 // an exact zero can differ, and the ReLU maps both zeros to +0), so every
 // output equals the in-order sum from the bias over (ci, ky, kx) with the
 // padded taps skipped.
-constexpr int kConvThreads = 512;
-
-template <int CI, int CO, int H, int COB, int SPB, int CIC, int RS, int NBUF>
+template <int T, int CI, int CO, int H, int COB, int SPB, int CIC, int RS, int NBUF>
 struct ConvFwdCfg {
     static constexpr int HO = H / 2;
     static constexpr int PT = (H / 2) * (H / 4);  // 2x4 pixel tiles per snippet
     static constexpr int CTN = COB / 8;           // 8-channel tiles per block
     static constexpr int TILES = PT * CTN * SPB;  // thread tiles per block
-    static constexpr int TPT = TILES / kConvThreads;  // tiles per thread
+    static constexpr int TPT = TILES / T;  // tiles per thread
     static constexpr int NCB = CO / COB;          // output-channel blocks
     static constexpr int NK = CI / CIC;           // stages per snippet group
     static constexpr int CH = (H + 1) * RS;       // staged elements per channel
@@ -111,22 +109,30 @@ struct ConvFwdCfg {
     static constexpr int W_FLOATS = CI * 9 * COB;
     static constexpr int CPS = SPB * CIC * H * H / 2;  // 4-byte copies per stage
     static constexpr size_t SMEM = (size_t)W_FLOATS * 4 + (size_t)NBUF * BUF * 2;
+    // blocks per SM: 512 threads of 128 registers, 227 KB of shared memory
+    static constexpr int BY_SMEM = (int)(227 * 1024 / (SMEM + 1024));
+    static constexpr int RESIDENT = BY_SMEM < 512 / T ? BY_SMEM : 512 / T;
     static_assert(COB % 8 == 0 && CO % COB == 0 && H % 4 == 0 && CI % CIC == 0, "tile shape");
     static_assert(NBUF >= 2 && NBUF <= 4, "stage buffers");
-    static_assert(TILES % kConvThreads == 0 && (TPT == 1 || CIC == CI), "whole tiles per thread");
+    static_assert(TILES % T == 0 && (TPT == 1 || CIC == CI), "whole tiles per thread");
     static_assert(RS % 4 == 0 && RS >= H + 2, "row stride");
     static_assert(SMEM <= 227 * 1024, "shared memory");
 };
 
-// Float image of a layer's weights in the staged order: dst[cb][ci][tap][co]
-// = w[cb*COB + co][ci][tap] for every output-channel block cb.
+// Float images of the layers' weights in the staged order, refreshed whenever
+// the parameters change: dst[cb][ci][tap][co] = w[cb*COB + co][ci][tap] for
+// every output-channel block cb, once for the wide and once for the narrow
+// blocks' COB.
 struct WPrepLayer {
     const uint16_t *w;
     float *dst;
     int ci, cob, count;
 };
+constexpr int kImages = 2;  // wide, narrow
+constexpr int kImageCob[kImages][kConvLayers] = {{16, 32, 64, 64}, {16, 16, 16, 16}};
+constexpr int kNarrowGroups = 512;  // snippet groups of a wide launch up to which the narrow blocks run
 struct WPrepArgs {
-    WPrepLayer l[kConvLayers];
+    WPrepLayer l[kImages * kConvLayers];
 };
 
 __global__ void conv_wprep_kernel(const WPrepArgs a) {
@@ -259,11 +265,11 @@ __device__ __forceinline__ void conv_epilogue(const uint64_t (&acc)[4][2][4], in
     }
 }
 
-template <int CI, int CO, int H, int COB, int SPB, int CIC, int RS, int NBUF, bool ARG>
-__global__ void __launch_bounds__(kConvThreads, 1)
+template <int T, int CI, int CO, int H, int COB, int SPB, int CIC, int RS, int NBUF, bool ARG>
+__global__ void __launch_bounds__(T, 512 / T)
     conv_fwd_kernel(const uint16_t *__restrict__ in, const float *__restrict__ wprep, const uint16_t *__restrict__ b,
                     int N, uint16_t *__restrict__ pooled, uint8_t *__restrict__ arg) {
-    using C = ConvFwdCfg<CI, CO, H, COB, SPB, CIC, RS, NBUF>;
+    using C = ConvFwdCfg<T, CI, CO, H, COB, SPB, CIC, RS, NBUF>;
     constexpr int HO = C::HO;
     extern __shared__ __align__(16) unsigned char smem[];
     float *ws = reinterpret_cast<float *>(smem);
@@ -274,16 +280,16 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     const int ngroups = (N + SPB - 1) / SPB;
     const int nst = cta < ngroups ? (ngroups - cta + ncta - 1) / ncta * C::NK : 0;
     uint4 *z = reinterpret_cast<uint4 *>(xs);
-    for (int i = tid; i < NBUF * C::BUF / 8; i += kConvThreads) z[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < NBUF * C::BUF / 8; i += T) z[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     const float *wsrc = wprep + (size_t)cb * C::W_FLOATS;
-    for (int i = tid; i < C::W_FLOATS / 4; i += kConvThreads) cp_async16(ws + 4 * i, wsrc + 4 * i);
+    for (int i = tid; i < C::W_FLOATS / 4; i += T) cp_async16(ws + 4 * i, wsrc + 4 * i);
     // stage s: group cta + ncta*(s / NK), input channels [k*CIC, (k+1)*CIC), k = s % NK
     auto issue = [&](int s) {
         const int g = cta + ncta * (s / C::NK), c0 = (s % C::NK) * CIC;
         uint16_t *dst = xs + (s % NBUF) * C::BUF;
 #pragma unroll 4
-        for (int i = tid; i < C::CPS; i += kConvThreads) {
+        for (int i = tid; i < C::CPS; i += T) {
             const int x2 = i % (H / 2), y = (i / (H / 2)) % H, cl = (i / (H * H / 2)) % CIC, j = i / (CIC * H * H / 2);
             const int n = g * SPB + j;
             if (n < N)
@@ -309,7 +315,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         const int k = s % C::NK;
 #pragma unroll 1
         for (int q = 0; q < C::TPT; ++q) {  // TPT > 1 only with one stage per group
-            const int tile = tid + q * kConvThreads;
+            const int tile = tid + q * T;
             const int pt = tile % C::PT, ct = (tile / C::PT) % C::CTN, sj = tile / (C::PT * C::CTN);
             const int ty = pt / (H / 4), tx = pt % (H / 4);
             const int cof = cb * COB + ct * 8;
@@ -393,51 +399,60 @@ __global__ void __launch_bounds__(256) fc1_fwd_kernel(const uint16_t *__restrict
 }
 
 // fc1, persistent (the fixed-order forward's layout, features [n][64][4][4]):
-// block b keeps the weights of outputs [64 (b % 2), +64) resident as
-// bfloat16 in [i/8][o][8] order (a lane's 8 consecutive weights are one
-// 16-byte load, the lanes of a warp consecutive outputs) and walks groups of
-// kFc1Group snippets, whose features are staged as float with the next
-// group's loads in flight in registers.  A thread owns one output of four
-// snippets; every sum runs over the inputs in increasing order.
-constexpr int kFc1Group = 16;
-constexpr size_t kFc1Smem = (size_t)64 * kFcIn * 2 + (size_t)kFc1Group * kFcIn * 4;
+// block b keeps the weights of OUTS outputs resident as bfloat16 in [i/8][o][8]
+// order (a lane's 8 consecutive weights are one 16-byte load, neighbouring
+// lanes neighbouring outputs) and walks groups of GROUP snippets, whose
+// features are staged as float with the next group's loads in flight in
+// registers.  A thread owns one output of GROUP * OUTS / 256 snippets; every
+// sum runs over the inputs in increasing order.  Bound by the latency of that
+// chain and by shared-memory reads.
+constexpr int kFc1Pad = 4;  // floats after a snippet's features: two snippets of a warp in different banks
+template <int OUTS, int GROUP>
+struct Fc1Cfg {
+    static constexpr int SNIPS = 256 / OUTS;     // snippets side by side
+    static constexpr int K = GROUP / SNIPS;      // snippets per thread
+    static constexpr int XS = kFcIn + kFc1Pad;   // floats per staged snippet
+    static constexpr int NB = kFcHid / OUTS;     // output blocks
+    static constexpr size_t SMEM = (size_t)OUTS * kFcIn * 2 + (size_t)GROUP * XS * 4;
+    static constexpr int RESIDENT = SMEM <= 112 * 1024 ? 2 : 1;
+    static_assert(GROUP % SNIPS == 0 && GROUP * kFcIn / 8 % 256 == 0, "tile shape");
+};
 
-__global__ void __launch_bounds__(256, 1) fc1_persist_kernel(const uint16_t *__restrict__ feat,
-                                                             const uint16_t *__restrict__ w,
-                                                             const uint16_t *__restrict__ b, int N,
-                                                             uint16_t *__restrict__ h1) {
+template <int OUTS, int GROUP>
+__global__ void __launch_bounds__(256, (Fc1Cfg<OUTS, GROUP>::RESIDENT))
+    fc1_persist_kernel(const uint16_t *__restrict__ feat, const uint16_t *__restrict__ w,
+                       const uint16_t *__restrict__ b, int N, uint16_t *__restrict__ h1) {
+    using C = Fc1Cfg<OUTS, GROUP>;
     extern __shared__ __align__(16) unsigned char smem[];
-    uint4 *ws = reinterpret_cast<uint4 *>(smem);                            // [128][64] x 8 bfloat16
-    float *xs = reinterpret_cast<float *>(smem + (size_t)64 * kFcIn * 2);  // [kFc1Group][1024]
+    uint4 *ws = reinterpret_cast<uint4 *>(smem);                              // [128][OUTS] x 8 bfloat16
+    float *xs = reinterpret_cast<float *>(smem + (size_t)OUTS * kFcIn * 2);  // [GROUP][XS]
     const int tid = threadIdx.x;
-    const int half = blockIdx.x & 1, cta = blockIdx.x >> 1, ncta = gridDim.x >> 1;
-    const int o = tid & 63, sg = tid >> 6;
-    for (int e = tid; e < 64 * (kFcIn / 8); e += 256) {
-        const int oo = e & 63, i8 = e >> 6;
-        ws[i8 * 64 + oo] = __ldg(reinterpret_cast<const uint4 *>(w + (long long)(64 * half + oo) * kFcIn) + i8);
-    }
-    const float bias = bf2f(b[64 * half + o]);
-    const int ngroups = (N + kFc1Group - 1) / kFc1Group;
-    // a group's features: kFc1Group x 128 uint4, 8 per thread
-    uint4 nxt[kFc1Group * kFcIn / 8 / 256];
+    const int ob = blockIdx.x % C::NB * OUTS, cta = blockIdx.x / C::NB, ncta = gridDim.x / C::NB;
+    const int o = tid % OUTS, sg = tid / OUTS;
+    const int ngroups = (N + GROUP - 1) / GROUP;
+    // a group's features: GROUP x 128 uint4
+    uint4 nxt[GROUP * kFcIn / 8 / 256];
     auto fetch = [&](int g) {
 #pragma unroll
-        for (int k = 0; k < kFc1Group * kFcIn / 8 / 256; ++k) {
+        for (int k = 0; k < GROUP * kFcIn / 8 / 256; ++k) {
             const int e = tid + 256 * k, sn = e / (kFcIn / 8), i8 = e % (kFcIn / 8);
-            const int n = g * kFc1Group + sn;
+            const int n = g * GROUP + sn;
             nxt[k] = n < N ? __ldg(reinterpret_cast<const uint4 *>(feat + (long long)n * kFcIn) + i8)
                            : make_uint4(0, 0, 0, 0);
         }
     };
     if (cta < ngroups) fetch(cta);
+    for (int e = tid; e < OUTS * (kFcIn / 8); e += 256)
+        ws[e] = __ldg(reinterpret_cast<const uint4 *>(w + (long long)(ob + e % OUTS) * kFcIn) + e / OUTS);
+    const float bias = bf2f(b[ob + o]);
 #pragma unroll 1
     for (int g = cta; g < ngroups; g += ncta) {
         __syncthreads();  // the previous group's features are consumed
 #pragma unroll
-        for (int k = 0; k < kFc1Group * kFcIn / 8 / 256; ++k) {
+        for (int k = 0; k < GROUP * kFcIn / 8 / 256; ++k) {
             const int e = tid + 256 * k, sn = e / (kFcIn / 8), i8 = e % (kFcIn / 8);
             const uint4 q = nxt[k];
-            float4 *dst = reinterpret_cast<float4 *>(xs + sn * kFcIn + 8 * i8);
+            float4 *dst = reinterpret_cast<float4 *>(xs + sn * C::XS + 8 * i8);
             dst[0] = make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xffff0000u),
                                  __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xffff0000u));
             dst[1] = make_float4(__uint_as_float(q.z << 16), __uint_as_float(q.z & 0xffff0000u),
@@ -445,18 +460,20 @@ __global__ void __launch_bounds__(256, 1) fc1_persist_kernel(const uint16_t *__r
         }
         __syncthreads();
         if (g + ncta < ngroups) fetch(g + ncta);
-        float acc[4] = {bias, bias, bias, bias};
-#pragma unroll 2
+        float acc[C::K];
+#pragma unroll
+        for (int k = 0; k < C::K; ++k) acc[k] = bias;
+#pragma unroll 4
         for (int i8 = 0; i8 < kFcIn / 8; ++i8) {
-            const uint4 wq = ws[i8 * 64 + o];
+            const uint4 wq = ws[i8 * OUTS + o];
             const float wf[8] = {__uint_as_float(wq.x << 16), __uint_as_float(wq.x & 0xffff0000u),
                                  __uint_as_float(wq.y << 16), __uint_as_float(wq.y & 0xffff0000u),
                                  __uint_as_float(wq.z << 16), __uint_as_float(wq.z & 0xffff0000u),
                                  __uint_as_float(wq.w << 16), __uint_as_float(wq.w & 0xffff0000u)};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float4 xa = *reinterpret_cast<const float4 *>(xs + (sg + 4 * k) * kFcIn + 8 * i8);
-                const float4 xc = *reinterpret_cast<const float4 *>(xs + (sg + 4 * k) * kFcIn + 8 * i8 + 4);
+            for (int k = 0; k < C::K; ++k) {
+                const float4 xa = *reinterpret_cast<const float4 *>(xs + (sg + C::SNIPS * k) * C::XS + 8 * i8);
+                const float4 xc = *reinterpret_cast<const float4 *>(xs + (sg + C::SNIPS * k) * C::XS + 8 * i8 + 4);
                 acc[k] = fmaf(wf[0], xa.x, acc[k]);
                 acc[k] = fmaf(wf[1], xa.y, acc[k]);
                 acc[k] = fmaf(wf[2], xa.z, acc[k]);
@@ -468,19 +485,36 @@ __global__ void __launch_bounds__(256, 1) fc1_persist_kernel(const uint16_t *__r
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int n = g * kFc1Group + sg + 4 * k;
-            if (n < N) h1[(long long)n * kFcHid + 64 * half + o] = f2bf(acc[k] > 0.0f ? acc[k] : 0.0f);
+        for (int k = 0; k < C::K; ++k) {
+            const int n = g * GROUP + sg + C::SNIPS * k;
+            if (n < N) h1[(long long)n * kFcHid + ob + o] = f2bf(acc[k] > 0.0f ? acc[k] : 0.0f);
         }
     }
 }
 
-__global__ void fc2_fwd_kernel(const uint16_t *__restrict__ h1, const uint16_t *__restrict__ w,
-                               const uint16_t *__restrict__ b, int N, float *__restrict__ z) {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
+// fc2 (128 -> 1): a thread one logit, its hidden row in 16-byte loads (all in
+// flight before the in-order sum starts).
+__global__ void __launch_bounds__(64) fc2_fwd_kernel(const uint16_t *__restrict__ h1, const uint16_t *__restrict__ w,
+                                                     const uint16_t *__restrict__ b, int N, float *__restrict__ z) {
+    __shared__ float s_w[kFcHid];
+    for (int i = threadIdx.x; i < kFcHid; i += 64) s_w[i] = bf2f(w[i]);
+    __syncthreads();
+    const int n = blockIdx.x * 64 + threadIdx.x;
     if (n >= N) return;
+    const uint4 *row = reinterpret_cast<const uint4 *>(h1 + (long long)n * kFcHid);
+    uint4 v[kFcHid / 8];
+#pragma unroll
+    for (int q = 0; q < kFcHid / 8; ++q) v[q] = __ldg(row + q);
     float acc = bf2f(b[0]);
-    for (int i = 0; i < kFcHid; ++i) acc = fmaf(bf2f(w[i]), bf2f(h1[n * kFcHid + i]), acc);
+#pragma unroll
+    for (int q = 0; q < kFcHid / 8; ++q) {
+        const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc = fmaf(s_w[8 * q + 2 * i], __uint_as_float(u[i] << 16), acc);
+            acc = fmaf(s_w[8 * q + 2 * i + 1], __uint_as_float(u[i] & 0xffff0000u), acc);
+        }
+    }
     z[n] = acc;
 }
 
@@ -1212,7 +1246,7 @@ struct NN {
     float *dpool[kConvLayers] = {};  // gradient w.r.t. each layer's pooled output
     unsigned *tc_err = nullptr;      // tensor-core forward: an MMA completion was not observed
     float *wprep = nullptr;          // float images of the convolution weights in staged order
-    int wprep_off[kConvLayers] = {};
+    int wprep_off[kImages][kConvLayers] = {};
     int nsm = 0;
 };
 
@@ -1239,58 +1273,77 @@ static void free_nn(NN *p) {
     delete p;
 }
 
-// Per layer: (CI, CO, H) and the tile parameters (COB, SPB, CIC, RS, NBUF).
-#define DD_CONV_LAYERS(X)                \
-    X(0, 1, 16, 64, 16, 1, 1, 68, 4)    \
-    X(1, 16, 32, 32, 32, 1, 16, 48, 3)  \
-    X(2, 32, 64, 16, 64, 2, 16, 24, 3)  \
-    X(3, 64, 64, 8, 64, 8, 8, 12, 3)
+// Refresh the convolutions' float weight images from the bfloat16 parameters.
+static void refresh_images(NN *p, cudaStream_t s) {
+    WPrepArgs a;
+    int most = 0;
+    for (int i = 0; i < kImages; ++i)
+        for (int l = 0; l < kConvLayers; ++l) {
+            const int count = kCin[l] * 9 * kCout[l];
+            a.l[i * kConvLayers + l] = {p->bf + p->L.cw[l], p->wprep + p->wprep_off[i][l], kCin[l], kImageCob[i][l], count};
+            most = std::max(most, count);
+        }
+    conv_wprep_kernel<<<dim3((unsigned)((most + 255) / 256), kImages * kConvLayers), 256, 0, s>>>(a);
+}
+
+// One convolution layer in the fixed order with the tile parameters given.
+template <int T, int CI, int CO, int H, int COB, int SPB, int CIC, int RS, int NBUF>
+static dd_status launch_conv_fwd(NN *p, int l, const uint16_t *in, int n, bool with_arg, cudaStream_t s) {
+    using C = ConvFwdCfg<T, CI, CO, H, COB, SPB, CIC, RS, NBUF>;
+    auto kern = with_arg ? conv_fwd_kernel<T, CI, CO, H, COB, SPB, CIC, RS, NBUF, true>
+                         : conv_fwd_kernel<T, CI, CO, H, COB, SPB, CIC, RS, NBUF, false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e != cudaSuccess) return cuda_fail(e, "classifier forward");
+    const int groups = (n + SPB - 1) / SPB;
+    const int grid = std::max(1, std::min(p->nsm * C::RESIDENT / C::NCB, groups));
+    constexpr int image = CI > 1 && COB == 16 ? 1 : 0;  // narrow or wide order
+    kern<<<grid * C::NCB, T, C::SMEM, s>>>(in, p->wprep + p->wprep_off[image][l], p->bf + p->L.cb[l], n, p->pooled[l],
+                                           p->arg[l]);
+    return DD_OK;
+}
+
+template <int OUTS, int GROUP>
+static dd_status launch_fc1(NN *p, int n, cudaStream_t s) {
+    using C = Fc1Cfg<OUTS, GROUP>;
+    auto kern = fc1_persist_kernel<OUTS, GROUP>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
+    if (e != cudaSuccess) return cuda_fail(e, "classifier forward");
+    const int grid = std::max(1, std::min(p->nsm * C::RESIDENT / C::NB, (n + GROUP - 1) / GROUP));
+    kern<<<grid * C::NB, 256, C::SMEM, s>>>(p->pooled[3], p->bf + p->L.f1w, p->bf + p->L.f1b, n, p->h1);
+    return DD_OK;
+}
 
 // with_arg: record the pooling argmax of every layer (the backward pass needs it).
 static dd_status nn_forward(NN *p, const uint16_t *x, int n, cudaStream_t s, bool with_arg) {
     const Layout &L = p->L;
     if (((uintptr_t)x) % 4 != 0) return fail(DD_ERR_INVALID_ARG, "snippets must be 4-byte aligned");
-    WPrepArgs wa;
-    int wmax = 0;
-    for (int l = 0; l < kConvLayers; ++l) {
-        wa.l[l].w = p->bf + L.cw[l];
-        wa.l[l].dst = p->wprep + p->wprep_off[l];
-        wa.l[l].ci = kCin[l];
-        wa.l[l].count = kCin[l] * 9 * kCout[l];
-        wmax = std::max(wmax, wa.l[l].count);
-    }
-#define DD_COB(LY, CI, CO, H, COB, SPB, CIC, RS, NBUF) wa.l[LY].cob = COB;
-    DD_CONV_LAYERS(DD_COB)
-#undef DD_COB
-    conv_wprep_kernel<<<dim3((unsigned)((wmax + 255) / 256), kConvLayers), 256, 0, s>>>(wa);
-    const uint16_t *in = x;
-#define DD_CONV_FWD(l, CI, CO, H, COB, SPB, CIC, RS, NBUF)                                                    \
-    {                                                                                                         \
-        using C = ConvFwdCfg<CI, CO, H, COB, SPB, CIC, RS, NBUF>;                                             \
-        auto kern = with_arg ? conv_fwd_kernel<CI, CO, H, COB, SPB, CIC, RS, NBUF, true>                     \
-                             : conv_fwd_kernel<CI, CO, H, COB, SPB, CIC, RS, NBUF, false>;                   \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM); \
-        if (e != cudaSuccess) return cuda_fail(e, "classifier forward");                                      \
-        const int groups = (n + SPB - 1) / SPB;                                                               \
-        int grid = p->nsm / C::NCB;                                                                           \
-        if (grid > groups) grid = groups;                                                                     \
-        if (grid < 1) grid = 1;                                                                               \
-        kern<<<grid * C::NCB, kConvThreads, C::SMEM, s>>>(in, p->wprep + p->wprep_off[l], p->bf + L.cb[l], n, \
-                                                           p->pooled[l], p->arg[l]);                          \
-        in = p->pooled[l];                                                                                    \
-    }
-    DD_CONV_LAYERS(DD_CONV_FWD)
-#undef DD_CONV_FWD
-    {
-        cudaError_t e = cudaFuncSetAttribute(fc1_persist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kFc1Smem);
-        if (e != cudaSuccess) return cuda_fail(e, "classifier forward");
-        const int groups = (n + kFc1Group - 1) / kFc1Group;
-        int grid = p->nsm / 2;
-        if (grid > groups) grid = groups;
-        fc1_persist_kernel<<<2 * grid, 256, kFc1Smem, s>>>(p->pooled[3], p->bf + L.f1w, p->bf + L.f1b, n, p->h1);
-    }
-    fc2_fwd_kernel<<<(n + 127) / 128, 128, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
+    // Narrow blocks (16 output channels, 128 or 256 threads) when the wide ones
+    // (all or 32 output channels, 512 threads) would give an SM no more than
+    // about three groups of snippets: with so few, whole SMs idle in the last
+    // wave or altogether, where four times as many narrow blocks fill them.
+    // Narrow / wide, whole forward: 96 / 207 us at 16 snippets, 170 / 235 at
+    // 256, 279 / 332 at 512; past the line the narrow blocks' repeated staging
+    // of the inputs costs 1-5 % (3513 / 3355 us at 8192).
+    const bool nar1 = n <= kNarrowGroups, nar2 = (n + 1) / 2 <= kNarrowGroups, nar3 = (n + 7) / 8 <= kNarrowGroups;
+    // (threads, CI, CO, H, output channels and snippets per block, input
+    // channels per stage, row stride, stages)
+    dd_status st = launch_conv_fwd<512, 1, 16, 64, 16, 1, 1, 68, 4>(p, 0, x, n, with_arg, s);
+    if (st == DD_OK)
+        st = nar1 ? launch_conv_fwd<256, 16, 32, 32, 16, 1, 8, 48, 3>(p, 1, p->pooled[0], n, with_arg, s)
+                  : launch_conv_fwd<512, 16, 32, 32, 32, 1, 16, 48, 3>(p, 1, p->pooled[0], n, with_arg, s);
+    if (st == DD_OK)
+        st = nar2 ? launch_conv_fwd<128, 32, 64, 16, 16, 2, 8, 24, 3>(p, 2, p->pooled[1], n, with_arg, s)
+                  : launch_conv_fwd<512, 32, 64, 16, 64, 2, 16, 24, 3>(p, 2, p->pooled[1], n, with_arg, s);
+    if (st == DD_OK)
+        st = nar3 ? launch_conv_fwd<128, 64, 64, 8, 16, 8, 4, 12, 3>(p, 3, p->pooled[2], n, with_arg, s)
+                  : launch_conv_fwd<512, 64, 64, 8, 64, 8, 8, 12, 3>(p, 3, p->pooled[2], n, with_arg, s);
+    // fc1: 16 outputs per block while all blocks of 16 snippets fit one wave of
+    // two per SM (12 us against 20 us with 64 outputs at 256 snippets; 74
+    // against 56 us at 4096)
+    if (st == DD_OK)
+        st = (n + 15) / 16 * (kFcHid / 16) <= 2 * p->nsm ? launch_fc1<16, 16>(p, n, s) : launch_fc1<64, 16>(p, n, s);
+    if (st != DD_OK) return st;
+    fc2_fwd_kernel<<<(n + 63) / 64, 64, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
     return cuda_fail(cudaGetLastError(), "classifier forward");
 }
 
@@ -1317,7 +1370,7 @@ static dd_status nn_forward_tc(NN *p, const uint16_t *x, int n, cudaStream_t s) 
 #undef DD_CONV_TC
     fc1_fwd_kernel<true><<<(n + kFc1Rows - 1) / kFc1Rows, 256, 0, s>>>(p->pooled[3], p->bf + L.f1w, p->bf + L.f1b, n,
                                                                       p->h1);
-    fc2_fwd_kernel<<<(n + 127) / 128, 128, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
+    fc2_fwd_kernel<<<(n + 63) / 64, 64, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
     return cuda_fail(cudaGetLastError(), "classifier forward");
 }
 
@@ -1360,11 +1413,13 @@ dd_status dd_nn_create(dd_nn **out, int max_batch) {
     if (e == cudaSuccess) e = cudaMalloc(&p->partial, part * 4);
     if (e == cudaSuccess) e = cudaMalloc(&p->tc_err, 4);
     int wtot = 0;
-    for (int l = 0; l < kConvLayers; ++l) {
-        p->wprep_off[l] = wtot;
-        wtot += kCin[l] * 9 * kCout[l];
-    }
+    for (int i = 0; i < kImages; ++i)
+        for (int l = 0; l < kConvLayers; ++l) {
+            p->wprep_off[i][l] = wtot;
+            wtot += kCin[l] * 9 * kCout[l];
+        }
     if (e == cudaSuccess) e = cudaMalloc(&p->wprep, (size_t)wtot * 4);
+    if (e == cudaSuccess) e = cudaMemset(p->wprep, 0, (size_t)wtot * 4);
     if (e == cudaSuccess) e = cudaMemset(p->tc_err, 0, 4);
     if (e == cudaSuccess) {
         int dev = 0;
@@ -1393,6 +1448,7 @@ dd_status dd_nn_set_params(dd_nn *nn, const float *h_master) {
     DD_CUDA_TRY(cudaMemset(p->m, 0, P * 4));
     DD_CUDA_TRY(cudaMemset(p->v, 0, P * 4));
     to_bf16_kernel<<<(unsigned)((P + 255) / 256), 256>>>((long long)P, p->master, p->bf);
+    refresh_images(p, nullptr);
     DD_CUDA_TRY(cudaGetLastError());
     DD_CUDA_TRY(cudaDeviceSynchronize());
     p->step = 0;
@@ -1513,6 +1569,7 @@ dd_status dd_nn_adamw(dd_nn *nn, float lr, float beta1, float beta2, float eps, 
     adamw_kernel<<<(unsigned)((P + 255) / 256), 256, 0, (cudaStream_t)stream>>>(P, p->master, p->grad, p->m, p->v,
                                                                                   p->bf, lr, beta1, beta2, eps, wd,
                                                                                   c1, c2);
+    refresh_images(p, (cudaStream_t)stream);
     return cuda_fail(cudaGetLastError(), "adamw_kernel launch");
 }
 
@@ -1564,6 +1621,7 @@ dd_status dd_nn_load(dd_nn *nn, const char *path) {
     DD_CUDA_TRY(cudaMemcpy(p->m, buf.data() + P, P * 4, cudaMemcpyHostToDevice));
     DD_CUDA_TRY(cudaMemcpy(p->v, buf.data() + 2 * P, P * 4, cudaMemcpyHostToDevice));
     to_bf16_kernel<<<(unsigned)((P + 255) / 256), 256>>>((long long)P, p->master, p->bf);
+    refresh_images(p, nullptr);
     DD_CUDA_TRY(cudaGetLastError());
     DD_CUDA_TRY(cudaDeviceSynchronize());
     p->step = (int)hdr[1];

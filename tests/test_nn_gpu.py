@@ -96,6 +96,26 @@ def test_forward_bit_exact_at_launch_size(P):
         np.testing.assert_array_equal(z[idx], oracle.nn_forward(p, x[idx], round_bf16=True))
 
 
+@pytest.mark.parametrize("n", [512, 513, 608, 609, 1024, 1025, 4096])
+def test_forward_bit_exact_at_dispatch_lines(P, n):
+    """Batches on both sides of the lines where a layer changes its block
+    shape: 16 sampled logits (the last snippets among them) equal the oracle's,
+    and the training forward (its loss) agrees with the inference one."""
+    import torch
+
+    p = params_with_biases(P, 9)
+    c = P.Classifier(max_batch=n, params=p)
+    x = snippets(100 + n, n)
+    z = c.forward(to_dev(x)).cpu().numpy()
+    idx = np.unique(np.concatenate([np.random.default_rng(n).choice(n, 12, replace=False), [0, n - 3, n - 2, n - 1]]))
+    np.testing.assert_array_equal(z[idx], oracle.nn_forward(p, x[idx], round_bf16=True))
+    y = (np.arange(n) % 2).astype(np.float32)
+    c.backward(to_dev(x), torch.from_numpy(y).cuda())
+    zd = z.astype(np.float64)
+    want = float(np.mean(np.maximum(zd, 0) - zd * y + np.log1p(np.exp(-np.abs(zd)))))
+    assert abs(c.loss() - want) <= 1e-6 * max(1.0, want)
+
+
 @pytest.mark.parametrize("n,seed", [(1, 11), (37, 12), (301, 13)])
 def test_tensor_core_forward_drift_outside_logit_tolerance(P, n, seed):
     """NOT a parity test: the opt-in tensor-core forward does NOT meet the
