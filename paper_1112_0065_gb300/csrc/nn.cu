@@ -122,14 +122,15 @@ struct ConvFwdCfg {
 // Float images of the layers' weights in the staged order, refreshed whenever
 // the parameters change: dst[cb][ci][tap][co] = w[cb*COB + co][ci][tap] for
 // every output-channel block cb, once for the wide and once for the narrow
-// blocks' COB.
+// blocks' COB.  A third image (cob 0) is the tensor-core kernels' bfloat16
+// operand: K-major over k = tap * ci + channel, 9 taps padded to 16 when ci = 1.
 struct WPrepLayer {
     const uint16_t *w;
     float *dst;
     int ci, cob, count;
 };
-constexpr int kImages = 2;  // wide, narrow
-constexpr int kImageCob[kImages][kConvLayers] = {{16, 32, 64, 64}, {16, 16, 16, 16}};
+constexpr int kImages = 3;  // wide, narrow, tensor cores
+constexpr int kImageCob[kImages][kConvLayers] = {{16, 32, 64, 64}, {16, 16, 16, 16}, {0, 0, 0, 0}};
 constexpr int kNarrowGroups = 512;  // snippet groups of a wide launch up to which the narrow blocks run
 struct WPrepArgs {
     WPrepLayer l[kImages * kConvLayers];
@@ -137,6 +138,15 @@ struct WPrepArgs {
 
 __global__ void conv_wprep_kernel(const WPrepArgs a) {
     const WPrepLayer L = a.l[blockIdx.y];
+    if (L.cob == 0) {
+        const int K = L.ci == 1 ? 16 : 9 * L.ci;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L.count; i += gridDim.x * blockDim.x) {
+            const int co = i / K, k = i % K, tap = k / L.ci, ci = k % L.ci;
+            reinterpret_cast<uint16_t *>(L.dst)[tc::kmajor_offset(co, k, K) / 2] =
+                tap < 9 ? L.w[(co * L.ci + ci) * 9 + tap] : (uint16_t)0;
+        }
+        return;
+    }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L.count; i += gridDim.x * blockDim.x) {
         const int co = i % L.cob, k = (i / L.cob) % 9, ci = (i / (L.cob * 9)) % L.ci, cb = i / (L.cob * 9 * L.ci);
         L.dst[i] = bf2f(L.w[((cb * L.cob + co) * L.ci + ci) * 9 + k]);
@@ -152,6 +162,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
@@ -341,63 +352,6 @@ __global__ void __launch_bounds__(T, 512 / T)
     cp_async_wait<0>();
 }
 
-// fc1 (1024 -> 128, ReLU) of the tensor-core forward (channel-last
-// features): a block computes 8 snippets x 128 outputs, a thread one output
-// of 4 snippets; the snippets' features sit in shared memory (float) and each
-// thread streams its weight row with 16-byte loads.  Every sum runs over the
-// inputs in increasing order.
-constexpr int kFc1Rows = 8;
-
-// NHWC: the features are stored channel-last ([4][4][64]); feature f of the
-// network's (channel, y, x) flattening then sits at (f % 16) * 64 + f / 16.
-template <bool NHWC>
-__global__ void __launch_bounds__(256) fc1_fwd_kernel(const uint16_t *__restrict__ feat,
-                                                      const uint16_t *__restrict__ w,
-                                                      const uint16_t *__restrict__ b, int N,
-                                                      uint16_t *__restrict__ h1) {
-    __shared__ __align__(16) float xs[kFc1Rows][kFcIn];
-    const int o = threadIdx.x % kFcHid, sg = threadIdx.x / kFcHid;
-    const int n0 = blockIdx.x * kFc1Rows;
-#pragma unroll 4
-    for (int e = threadIdx.x; e < kFc1Rows * kFcIn; e += 256) {
-        const int r = e / kFcIn, i = e % kFcIn;
-        const int src = NHWC ? (i % 16) * 64 + i / 16 : i;
-        xs[r][i] = (n0 + r < N) ? bf2f(__ldg(feat + (long long)(n0 + r) * kFcIn + src)) : 0.0f;
-    }
-    __syncthreads();
-    float acc[4];
-    const float bias = bf2f(b[o]);
-#pragma unroll
-    for (int s = 0; s < 4; ++s) acc[s] = bias;
-    const uint4 *wr = reinterpret_cast<const uint4 *>(w + (long long)o * kFcIn);  // 16-byte aligned rows
-#pragma unroll 4
-    for (int i8 = 0; i8 < kFcIn / 8; ++i8) {
-        const uint4 wq = __ldg(wr + i8);
-        const float wf[8] = {__uint_as_float(wq.x << 16), __uint_as_float(wq.x & 0xffff0000u),
-                             __uint_as_float(wq.y << 16), __uint_as_float(wq.y & 0xffff0000u),
-                             __uint_as_float(wq.z << 16), __uint_as_float(wq.z & 0xffff0000u),
-                             __uint_as_float(wq.w << 16), __uint_as_float(wq.w & 0xffff0000u)};
-#pragma unroll
-        for (int s = 0; s < 4; ++s) {
-            const float4 xa = *reinterpret_cast<const float4 *>(&xs[sg * 4 + s][i8 * 8]);
-            const float4 xc = *reinterpret_cast<const float4 *>(&xs[sg * 4 + s][i8 * 8 + 4]);
-            acc[s] = fmaf(wf[0], xa.x, acc[s]);
-            acc[s] = fmaf(wf[1], xa.y, acc[s]);
-            acc[s] = fmaf(wf[2], xa.z, acc[s]);
-            acc[s] = fmaf(wf[3], xa.w, acc[s]);
-            acc[s] = fmaf(wf[4], xc.x, acc[s]);
-            acc[s] = fmaf(wf[5], xc.y, acc[s]);
-            acc[s] = fmaf(wf[6], xc.z, acc[s]);
-            acc[s] = fmaf(wf[7], xc.w, acc[s]);
-        }
-    }
-#pragma unroll
-    for (int s = 0; s < 4; ++s) {
-        const int n = n0 + sg * 4 + s;
-        if (n < N) h1[(long long)n * kFcHid + o] = f2bf(acc[s] > 0.0f ? acc[s] : 0.0f);
-    }
-}
-
 // fc1, persistent (the fixed-order forward's layout, features [n][64][4][4]):
 // block b keeps the weights of OUTS outputs resident as bfloat16 in [i/8][o][8]
 // order (a lane's 8 consecutive weights are one 16-byte load, neighbouring
@@ -521,62 +475,248 @@ __global__ void __launch_bounds__(64) fc2_fwd_kernel(const uint16_t *__restrict_
 // ---- inference forward on the tensor cores -----------------------------------
 //
 // Implicit-GEMM convolution + ReLU + 2x2 max pooling with tcgen05.  A tile is
-// M = 128 convolution outputs = 32 pooled outputs x their 2x2 windows (row m =
-// 4 * pooled + position in the window), N = CO output channels, and K = the 9
-// taps x CI input channels ordered (tap, channel), so that with activations
-// stored channel-last (NHWC) 8 consecutive K values are one 16-byte load.
-// The CTA keeps the weights (N x K, bfloat16) in shared memory, builds the
-// im2col rows of its tiles K-chunk by K-chunk into two alternating buffers,
-// one thread issues the MMAs of each chunk into a tensor-memory accumulator
-// (two, alternating between tiles), and the epilogue of a tile -- bias,
-// ReLU, bfloat16 rounding, max over the window -- runs while the tensor cores
-// work on the next one.  Sums are fp32 in the tensor cores' own order, so the
-// logits agree with the fixed-order forward to float round-off (the training
-// path keeps the fixed-order kernels above).
+// M = 128 pooled outputs; its four window positions q are four accumulators of
+// N = CO columns in tensor memory, so pooling is a maximum over registers.  K
+// = the 9 taps x CI input channels in (tap, channel) order, 16 per MMA.
+//
+// No im2col: a snippet's input sits in shared memory as 16-byte cells (8
+// channels of one pixel), split by the parities of y and x.  For window
+// position q and tap (dy, dx) the input pixels of neighbouring pooled outputs
+// are neighbouring cells of one parity plane, so 8 of them are a core matrix
+// of the K-major operand where they lie, and a tap is only another start
+// address.  Zero cells after each row and before each plane are the padding.
+// Narrow images interleave snippets (rows of SUBS of them, cells of XS) so
+// that the 16 core matrices of a tile are equally spaced (PITCH).
+//
+// One unit (UNIT snippets) per step: warp 8 issues its MMAs, the other warps
+// fetch the next unit's cells (16-byte cp.async from channel-last memory) and
+// turn the previous unit's accumulators into outputs meanwhile.  Bound by the
+// MMAs' reads of the 4 KB operand tiles (32 cycles each): the im2col form this
+// replaces gathered 9 copies of the input and took 932 / 535 / 293 / 200 us
+// for the four layers at 8192 snippets, XX us now.  Sums are fp32 in the
+// tensor cores' own order, so the logits agree with the fixed-order forward to
+// float round-off (the training path keeps the fixed-order kernels above).
 // Polls of an MMA-completion mbarrier before a thread gives up (a poll that
 // finds the phase incomplete suspends the thread for ~4 us on GB300: ~60 ms,
 // against microseconds per tile); after a give-up a thread waits no more.
 constexpr uint32_t kTcWaitPolls = 1u << 14;
+constexpr int kTcThreads = 288;  // 8 warps of loads and outputs, one issuing MMAs
 
-template <int CI, int CO, int H, int TPC>
+template <int CI, int CO, int H>
 struct ConvTcCfg {
-    static constexpr int HO = H / 2;
-    static constexpr int K = CI == 1 ? 16 : 9 * CI;   // conv1: 9 taps padded to one MMA step
-    static constexpr int KC = CI == 1 ? 16 : TPC * CI;  // K per chunk
-    static constexpr int NCHUNK = K / KC;
-    static constexpr int A_BYTES = 128 * KC * 2;
+    static constexpr int HO = H / 2, K = 9 * CI, G = CI / 8;
+    static constexpr int XS = HO >= 8 ? 1 : 8 / HO;         // snippets interleaved within a row's cells
+    static constexpr int PITCH = (HO + 1) * XS;             // cells of a row with its zero cell
+    static constexpr int UNIT = HO >= 16 ? 1 : 16 / HO * XS;  // snippets per unit
+    static constexpr int SUBS = UNIT / XS;                  // rows interleaved
+    static constexpr int YS = PITCH * SUBS;                 // cells from pooled row to pooled row
+    static constexpr int LEAD = YS + XS;                    // zero cells before a plane
+    static constexpr int PS = LEAD + HO * YS;               // cells of a parity plane
+    static constexpr int GS = 4 * PS + 1;                   // cells of a channel group (odd: 8 groups, 8 banks)
+    static constexpr int CELLS = G * GS + LEAD;
+    static constexpr int TILES = HO * HO * UNIT / 128;
+    static constexpr int NBUF = CI == 64 ? 1 : 2;           // input buffers that fit beside the weights
+    static constexpr int DCOLS = TILES * 4 * CO;            // accumulator columns of a unit
     static constexpr int B_BYTES = CO * K * 2;
-    static constexpr size_t SMEM = (size_t)2 * A_BYTES + B_BYTES;
-    static constexpr uint32_t TCOLS = 2 * CO <= 32 ? 32 : (2 * CO <= 64 ? 64 : (2 * CO <= 128 ? 128 : 256));
-    static constexpr int MINB = SMEM <= 110 * 1024 ? 2 : 1;
-    static_assert(K % KC == 0 && KC % 16 == 0 && (CI == 1 || CI % 8 == 0), "chunking");
-    static_assert(CO % 16 == 0 && CO <= 128, "N of the MMA");
+    static constexpr bool FEATURES = HO == 4;               // last layer: [n][co][4][4] for fc1
+    static constexpr int OUT_PITCH = CO * HO * HO * 2 + 16; // bytes of a staged snippet of features
+    static constexpr int OUT_BYTES = FEATURES ? UNIT * OUT_PITCH : 0;
+    static constexpr size_t SMEM = (size_t)NBUF * CELLS * 16 + B_BYTES + OUT_BYTES;
+    static constexpr int UNIT_CELLS = UNIT * H * H * G;     // 16-byte copies per unit
+    static_assert(SMEM <= 227 * 1024 && 2 * DCOLS == 512, "shared and tensor memory");
+    static_assert(TILES * 128 == HO * HO * UNIT && UNIT_CELLS % 256 == 0, "whole tiles");
 };
 
-template <int CI, int CO, int H, int TPC>
-__global__ void __launch_bounds__(256, (ConvTcCfg<CI, CO, H, TPC>::MINB))
-    conv_tc_kernel(const uint16_t *__restrict__ in, const uint16_t *__restrict__ w, const uint16_t *__restrict__ b,
+template <int CI, int CO, int H>
+__global__ void __launch_bounds__(kTcThreads, 1)
+    conv_tc_kernel(const uint16_t *__restrict__ in, const uint16_t *__restrict__ wk, const uint16_t *__restrict__ b,
                    int N, uint16_t *__restrict__ out, unsigned *__restrict__ err) {
-    using C = ConvTcCfg<CI, CO, H, TPC>;
-    constexpr int HO = C::HO, HO2 = HO * HO, K = C::K, KC = C::KC;
+    using C = ConvTcCfg<CI, CO, H>;
+    constexpr int HO = C::HO;
     extern __shared__ __align__(1024) uint8_t tsm[];
     __shared__ uint32_t s_tmem;
     __shared__ __align__(8) uint64_t s_mbar[2];
     __shared__ float s_bias[CO];
     uint8_t *As = tsm;
-    uint8_t *Bs = tsm + 2 * C::A_BYTES;
+    uint8_t *Bs = tsm + (size_t)C::NBUF * C::CELLS * 16;
+    uint8_t *Os = Bs + C::B_BYTES;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nunits = (N + C::UNIT - 1) / C::UNIT;
+    const int nu = (int)blockIdx.x < nunits ? (nunits - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-    // weights as B = [co][k], k = tap * CI + ci (conv1: k = tap, taps 9..15 zero)
-    for (int e = tid; e < CO * K; e += 256) {
-        const int co = e / K, k = e % K;
-        const int tap = CI == 1 ? k : k / CI, ci = CI == 1 ? 0 : k % CI;
-        const uint16_t v = tap < 9 ? __ldg(w + ((long long)co * CI + ci) * 9 + tap) : (uint16_t)0;
-        *reinterpret_cast<uint16_t *>(Bs + tc::kmajor_offset(co, k, K)) = v;
-    }
+    // zero cells once (copies only ever write data cells), weights in MMA order
+    for (int i = tid; i < C::NBUF * C::CELLS; i += kTcThreads) reinterpret_cast<uint4 *>(As)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < C::B_BYTES / 16; i += kTcThreads)
+        cp_async16(Bs + 16 * i, reinterpret_cast<const uint4 *>(wk) + i);
     if (tid < CO) s_bias[tid] = bf2f(b[tid]);
+    if (warp == 0) tc::tmem_alloc(&s_tmem, 2 * C::DCOLS);
+    if (tid == 0) {
+        tc::mbar_init(&s_mbar[0], 1);
+        tc::mbar_init(&s_mbar[1], 1);
+    }
+    __syncthreads();
+    auto load = [&](int u) {  // unit u of this CTA -> its buffer
+        const int s0 = ((int)blockIdx.x + u * (int)gridDim.x) * C::UNIT;
+        uint8_t *dst = As + (size_t)(u % C::NBUF) * C::CELLS * 16;
+        const uint4 *src = reinterpret_cast<const uint4 *>(in) + (long long)s0 * H * H * C::G;
+#pragma unroll 4
+        for (int k = 0; k < C::UNIT_CELLS / 256; ++k) {
+            const int e = tid + 256 * k;
+            const int g = e % C::G, x = (e / C::G) % H, y = (e / (C::G * H)) % H, s = e / (C::G * H * H);
+            const int cell = g * C::GS + ((y & 1) * 2 + (x & 1)) * C::PS + C::LEAD + (y >> 1) * C::YS +
+                             s / C::XS * C::PITCH + (x >> 1) * C::XS + s % C::XS;
+            if (s0 + s < N) cp_async16(dst + 16 * cell, src + e);
+        }
+    };
+    if (warp < 8 && nu > 0) load(0);
+    cp_async_wait_all();
     tc::fence_async_smem();
-    if (warp == 0) tc::tmem_alloc(&s_tmem, C::TCOLS);
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = s_tmem;
+    bool ok = true;
+    auto wait = [&](int u) {
+        if (ok) ok = tc::mbar_wait(&s_mbar[u & 1], (uint32_t)(u >> 1) & 1u, kTcWaitPolls);
+    };
+    auto issue = [&](int u) {
+        const uint64_t a0 = tc::smem_desc(tc::smem_addr(As) + (uint32_t)(u % C::NBUF) * (C::CELLS * 16), C::GS * 16,
+                                          C::PITCH * 16);
+        const uint64_t b0 = tc::smem_desc(tc::smem_addr(Bs), 128, C::K / 8 * 128);
+#pragma unroll
+        for (int t = 0; t < C::TILES; ++t)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t d = tmem + (uint32_t)((u & 1) * C::DCOLS + (t * 4 + q) * CO);
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap) {
+                    const int uy = (q >> 1) + tap / 3 - 1, ux = (q & 1) + tap % 3 - 1;  // -1 .. 2
+                    const int yp = uy & 1, xp = ux & 1;
+                    const int cell = (yp * 2 + xp) * C::PS + C::LEAD + (uy - yp) / 2 * C::YS + (ux - xp) / 2 * C::XS +
+                                     t * 8 * C::XS;
+#pragma unroll
+                    for (int st = 0; st < CI / 16; ++st)
+                        tc::mma_bf16(d, a0 + (uint64_t)(cell + 2 * st * C::GS), b0 + (uint64_t)(16 * (tap * (CI / 16) + st)),
+                                     tc::idesc_bf16(128, CO), tap > 0 || st > 0);
+                }
+            }
+        tc::mma_commit(&s_mbar[u & 1]);
+    };
+    // maximum over the window (bias, ReLU and rounding never decrease, so they
+    // follow it), bias, ReLU and rounding of unit u's accumulators: warp w
+    // takes rows 32 (w % 4) .. +31 and, with w / 4, one tile or half the channels
+    auto epilogue = [&](int u) {
+        tc::fence_after_sync();
+        const int quad = warp & 3, half = warp >> 2;
+        const int m = 32 * quad + lane, grp = m >> 3, e = m & 7;
+        const int py = grp / C::SUBS, px = (C::TILES == 2 ? half * 8 : 0) + e / C::XS;
+        const int sn = grp % C::SUBS * C::XS + e % C::XS;
+        const int n = ((int)blockIdx.x + u * (int)gridDim.x) * C::UNIT + sn;
+        const int cb = C::TILES == 2 ? 0 : half * (CO / 2);
+        const uint32_t t0 = tmem + (uint32_t)((u & 1) * C::DCOLS + (C::TILES == 2 ? half * 4 * CO : 0) + cb) +
+                            ((uint32_t)(32 * quad) << 16);
+        static_assert((C::TILES == 2 ? CO : CO / 2) == 32, "32 channels per thread");
+#pragma unroll
+        for (int c0 = 0; c0 < 32; c0 += 16) {
+            float v[4][16];
+            tc::tmem_ld4x16(t0 + c0, CO, v);
+            uint32_t pk[8];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const float a = fmaxf(fmaxf(v[0][i], v[1][i]), fmaxf(v[2][i], v[3][i])) + s_bias[cb + c0 + i];
+                const uint32_t r = f2bf(a > 0.0f ? a : 0.0f);
+                pk[i / 2] = i % 2 ? pk[i / 2] | r << 16 : r;
+            }
+            if constexpr (C::FEATURES) {
+                uint16_t *o = reinterpret_cast<uint16_t *>(Os + sn * C::OUT_PITCH) + (cb + c0) * HO * HO + py * HO + px;
+#pragma unroll
+                for (int i = 0; i < 16; ++i) o[i * HO * HO] = (uint16_t)(pk[i / 2] >> (i % 2 * 16));
+            } else if (n < N) {
+                uint4 *o = reinterpret_cast<uint4 *>(out + (((long long)n * HO + py) * HO + px) * CO + cb + c0);
+                o[0] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                o[1] = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+            }
+        }
+        if constexpr (C::FEATURES) {
+            constexpr int Q = CO * HO * HO / 8;  // 16-byte pieces of a snippet
+            const int s0 = ((int)blockIdx.x + u * (int)gridDim.x) * C::UNIT;
+            asm volatile("bar.sync 1, 256;\n" ::: "memory");
+            for (int i = tid; i < C::UNIT * Q; i += 256)
+                if (s0 + i / Q < N)
+                    reinterpret_cast<uint4 *>(out)[(long long)s0 * Q + i] =
+                        *reinterpret_cast<const uint4 *>(Os + i / Q * C::OUT_PITCH + i % Q * 16);
+        }
+    };
+#pragma unroll 1
+    for (int u = 0; u < nu; ++u) {
+        if (warp == 8) {
+            if (lane == 0) issue(u);
+            __syncwarp();
+        } else if constexpr (C::NBUF == 2) {
+            if (u > 0) wait(u - 1);  // frees the other input buffer
+            if (u + 1 < nu) load(u + 1);
+            if (u > 0) epilogue(u - 1);
+        } else {
+            if (u > 0) epilogue(u - 1);
+            wait(u);
+            if (u + 1 < nu) load(u + 1);
+        }
+        cp_async_wait_all();
+        tc::fence_async_smem();
+        tc::fence_before_sync();
+        __syncthreads();
+        tc::fence_after_sync();
+    }
+    if (nu > 0) {
+        if (C::NBUF == 2 || warp == 8) wait(nu - 1);
+        if (warp < 8) epilogue(nu - 1);
+    }
+    tc::fence_before_sync();
+    if (__syncthreads_or(!ok)) {
+        // some completion was not observed: give the last two commits one
+        // more short bounded wait before the tensor memory is freed
+        for (int k = 1; k <= 2 && nu - k >= 0; ++k)
+            tc::mbar_wait(&s_mbar[(nu - k) & 1], (uint32_t)((nu - k) >> 1) & 1u, kTcWaitPolls / 64 + 1);
+        tc::fence_before_sync();
+        __syncthreads();
+    }
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(tmem, 2 * C::DCOLS);
+    if (!ok && lane == 0) atomicOr(err, 1u);
+}
+
+// The first layer (one input channel, 64x64): K = 9 taps padded to 16, built
+// per row.  A unit is 4 pooled rows of a snippet = 128 pooled outputs; thread
+// (p, qy) builds the rows of output p at window positions (qy, 0) and (qy, 1)
+// from 3 x 4 input pixels by byte permutes (three neighbouring words per image
+// row, fetched one unit ahead) and stores them as one 16-byte group of 8 taps
+// and the ninth tap; the other seven of the second group stay zero.  Bound by
+// issue and shared-memory stores; three CTAs per SM hide each other's
+// barriers.
+struct Conv0Tc {
+    static constexpr int A_BYTES = 4 * 128 * 32;  // four window positions
+    static constexpr int B_BYTES = 16 * 16 * 2;
+    static constexpr int DCOLS = 4 * 16;
+};
+
+__global__ void __launch_bounds__(256, 3) conv0_tc_kernel(const uint16_t *__restrict__ in,
+                                                          const uint16_t *__restrict__ wk,
+                                                          const uint16_t *__restrict__ b, int N,
+                                                          uint16_t *__restrict__ out, unsigned *__restrict__ err) {
+    using C = Conv0Tc;
+    __shared__ __align__(128) uint8_t As[2][C::A_BYTES];
+    __shared__ __align__(128) uint8_t Bs[C::B_BYTES];
+    __shared__ uint32_t s_tmem;
+    __shared__ __align__(8) uint64_t s_mbar[2];
+    __shared__ float s_bias[16];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int nunits = N * 8;
+    const int nu = (int)blockIdx.x < nunits ? (nunits - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    for (int i = tid; i < 2 * C::A_BYTES / 16; i += 256) reinterpret_cast<uint4 *>(As)[i] = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < C::B_BYTES / 16; i += 256)
+        reinterpret_cast<uint4 *>(Bs)[i] = __ldg(reinterpret_cast<const uint4 *>(wk) + i);
+    if (tid < 16) s_bias[tid] = bf2f(b[tid]);
+    if (warp == 0) tc::tmem_alloc(&s_tmem, 2 * C::DCOLS);
     if (tid == 0) {
         tc::mbar_init(&s_mbar[0], 1);
         tc::mbar_init(&s_mbar[1], 1);
@@ -585,128 +725,84 @@ __global__ void __launch_bounds__(256, (ConvTcCfg<CI, CO, H, TPC>::MINB))
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = s_tmem;
-    const uint32_t a_addr = tc::smem_addr(As), b_addr = tc::smem_addr(Bs);
-    const int ntiles = (N * HO2 + 31) / 32;
-    const int my_tiles = (int)blockIdx.x < ntiles ? (ntiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int nst = my_tiles * C::NCHUNK;
     bool ok = true;
-
-    // this thread's im2col row (fixed: 256 threads step over units of 128 rows)
-    const int m = tid & 127;
-    auto row_pos = [&](int tile, int &n, int &y, int &x) {
-        const int P = tile * 32 + (m >> 2);
-        n = P / HO2;
-        const int pp = P % HO2;
-        y = 2 * (pp / HO) + ((m >> 1) & 1);
-        x = 2 * (pp % HO) + (m & 1);
-    };
-    auto fill = [&](uint8_t *A, int tile, int c) {
-        int n, y, x;
-        row_pos(tile, n, y, x);
-        const bool live = n < N;
-        if constexpr (CI == 1) {
-            // one 16-byte group per thread: taps 8j .. 8j+7 of row m
-            const int j = tid >> 7;
-            uint32_t pk[4] = {0u, 0u, 0u, 0u};
+    const int p = tid & 127, qy = tid >> 7, px = p & 31;
+    uint32_t w[3][3];  // image rows y-1 .. y+1, pixel pairs px-1 .. px+1
+    auto fetch = [&](int u) {
+        const int unit = (int)blockIdx.x + u * (int)gridDim.x;
+        const uint32_t *img = reinterpret_cast<const uint32_t *>(in) + (long long)(unit >> 3) * (64 * 32);
+        const int y = 2 * (4 * (unit & 7) + (p >> 5)) + qy;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int t = 8 * j + i;
-                const int yy = y + t / 3 - 1, xx = x + t % 3 - 1;
-                uint16_t v = 0;
-                if (live && t < 9 && yy >= 0 && yy < H && xx >= 0 && xx < H)
-                    v = __ldg(in + ((long long)n * H + yy) * H + xx);
-                pk[i >> 1] |= (uint32_t)v << (16 * (i & 1));
-            }
-            *reinterpret_cast<uint4 *>(A + tc::kmajor_offset(m, 8 * j, KC)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-        } else {
-            constexpr int G = CI / 8;                // 16-byte groups per pixel
-            constexpr int UNITS = TPC * G;           // per row in this chunk
-#pragma unroll 4
-            for (int r = tid >> 7; r < UNITS; r += 2) {
-                const int g = r % G, tl = r / G;
-                const int tap = c * TPC + tl;
-                const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (live && yy >= 0 && yy < H && xx >= 0 && xx < H)
-                    v = __ldg(reinterpret_cast<const uint4 *>(in + (((long long)n * H + yy) * H + xx) * CI) + g);
-                *reinterpret_cast<uint4 *>(A + tc::kmajor_offset(m, tl * CI + 8 * g, KC)) = v;
+        for (int r = 0; r < 3; ++r) {
+            const int yy = y + r - 1;
+            const bool row = yy >= 0 && yy < 64;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int xx = px + c - 1;
+                w[r][c] = row && xx >= 0 && xx < 32 ? __ldg(img + yy * 32 + xx) : 0u;
             }
         }
     };
-    // bias, ReLU, bfloat16 rounding and 2x2 max of local tile lt (global tile `tile`)
-    auto epilogue = [&](int lt, int tile, int stage) {
-        if (ok) ok = tc::mbar_wait(&s_mbar[stage & 1], (uint32_t)(stage >> 1) & 1u, kTcWaitPolls);
+    auto build = [&](int u) {
+        uint8_t *A = As[u & 1];
+        // taps of column x-1, x, x+1: hi of pair 0, lo and hi of pair 1 (x even); both of pair 1, lo of pair 2 (x odd)
+        uint8_t *d0 = A + (2 * qy) * 4096 + tc::kmajor_offset(p, 0, 16), *d1 = d0 + 4096;
+        *reinterpret_cast<uint4 *>(d0) =
+            make_uint4(__byte_perm(w[0][0], w[0][1], 0x5432), __byte_perm(w[0][1], w[1][0], 0x7632), w[1][1],
+                       __byte_perm(w[2][0], w[2][1], 0x5432));
+        *reinterpret_cast<uint32_t *>(d0 + 128) = w[2][1] >> 16;
+        *reinterpret_cast<uint4 *>(d1) = make_uint4(w[0][1], __byte_perm(w[0][2], w[1][1], 0x5410),
+                                                    __byte_perm(w[1][1], w[1][2], 0x5432), w[2][1]);
+        *reinterpret_cast<uint32_t *>(d1 + 128) = w[2][2] & 0xFFFFu;
+    };
+    auto epilogue = [&](int u) {
+        if (ok) ok = tc::mbar_wait(&s_mbar[u & 1], (uint32_t)(u >> 1) & 1u, kTcWaitPolls);
         tc::fence_after_sync();
-        constexpr int HALVES = CO >= 32 ? 2 : 1;  // column halves over the two warpgroups
-        constexpr int CW = CO / HALVES;
-        const int quad = warp & 3, half = warp >> 2;
-        if (half < HALVES) {
-            const int mm = 32 * quad + lane;
-            const int P = tile * 32 + (mm >> 2);
-            const int n = P / HO2, pp = P % HO2, q = mm & 3;
+        const int quad = warp & 3, cb = (warp >> 2) * 8;
+        const int unit = (int)blockIdx.x + u * (int)gridDim.x;
+        float v[4][8];
+        tc::tmem_ld4x8(tmem + (uint32_t)((u & 1) * C::DCOLS + cb) + ((uint32_t)(32 * quad) << 16), 16, v);
+        uint32_t pk[4];
 #pragma unroll
-            for (int c0 = 0; c0 < CW; c0 += 16) {
-                const int cb = half * CW + c0;
-                float v[16];
-                tc::tmem_ld16(tmem + (uint32_t)((lt & 1) * CO + cb) + ((uint32_t)(32 * quad) << 16), v);
-                float mx[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float a = v[i] + s_bias[cb + i];
-                    float r = bf2f(f2bf(a > 0.0f ? a : 0.0f));
-                    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 1));
-                    r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, 2));
-                    mx[i] = r;
-                }
-                // lane q of the window writes channels cb + 4q .. cb + 4q + 3
-                uint32_t w01 = 0, w23 = 0;
-#pragma unroll
-                for (int qq = 0; qq < 4; ++qq)
-                    if (q == qq) {
-                        w01 = (uint32_t)f2bf(mx[4 * qq]) | ((uint32_t)f2bf(mx[4 * qq + 1]) << 16);
-                        w23 = (uint32_t)f2bf(mx[4 * qq + 2]) | ((uint32_t)f2bf(mx[4 * qq + 3]) << 16);
-                    }
-                if (n < N)
-                    *reinterpret_cast<uint2 *>(out + ((long long)n * HO2 + pp) * CO + cb + 4 * q) = make_uint2(w01, w23);
-            }
+        for (int i = 0; i < 8; ++i) {
+            const float a = fmaxf(fmaxf(v[0][i], v[1][i]), fmaxf(v[2][i], v[3][i])) + s_bias[cb + i];
+            const uint32_t r = f2bf(a > 0.0f ? a : 0.0f);
+            pk[i / 2] = i % 2 ? pk[i / 2] | r << 16 : r;
         }
+        *reinterpret_cast<uint4 *>(out + ((long long)unit * 128 + 32 * quad + lane) * 16 + cb) =
+            make_uint4(pk[0], pk[1], pk[2], pk[3]);
     };
-
-    for (int s = 0; s < nst; ++s) {
-        const int lt = s / C::NCHUNK, c = s % C::NCHUNK;
-        const int tile = (int)blockIdx.x + lt * (int)gridDim.x;
-        const int buf = s & 1;
-        if (s >= 2 && ok) ok = tc::mbar_wait(&s_mbar[buf], (uint32_t)((s - 2) >> 1) & 1u, kTcWaitPolls);
-        fill(As + buf * C::A_BYTES, tile, c);
+    if (nu > 0) fetch(0);
+#pragma unroll 1
+    for (int u = 0; u < nu; ++u) {
+        build(u);  // its buffer's last MMAs were waited for by the epilogue of unit u - 2
+        if (u + 1 < nu) fetch(u + 1);
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
         tc::fence_after_sync();
         if (tid == 0) {
-            const uint32_t acc = tmem + (uint32_t)((lt & 1) * CO);
-#pragma unroll 1
-            for (int st = 0; st < KC / 16; ++st)
-                tc::mma_bf16(acc, tc::smem_desc(a_addr + buf * C::A_BYTES + 256 * st, 128, KC / 8 * 128),
-                             tc::smem_desc(b_addr + 256 * (c * (KC / 16) + st), 128, K / 8 * 128),
-                             tc::idesc_bf16(128, CO), c > 0 || st > 0);
-            tc::mma_commit(&s_mbar[buf]);
+            const uint64_t a0 = tc::smem_desc(tc::smem_addr(As[u & 1]), 128, 256);
+            const uint64_t b0 = tc::smem_desc(tc::smem_addr(Bs), 128, 256);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                tc::mma_bf16(tmem + (uint32_t)((u & 1) * C::DCOLS + 16 * q), a0 + (uint64_t)(256 * q), b0,
+                             tc::idesc_bf16(128, 16), false);
+            tc::mma_commit(&s_mbar[u & 1]);
         }
-        if (c == 0 && lt > 0) epilogue(lt - 1, tile - (int)gridDim.x, s - 1);
+        __syncwarp();
+        if (u > 0) epilogue(u - 1);
     }
-    if (nst > 0) epilogue(my_tiles - 1, (int)blockIdx.x + (my_tiles - 1) * (int)gridDim.x, nst - 1);
+    if (nu > 0) epilogue(nu - 1);
     tc::fence_before_sync();
     if (__syncthreads_or(!ok)) {
-        // some completion was not observed: give the last two commits one
-        // more short bounded wait before the tensor memory is freed
-        for (int k = 1; k <= 2 && nst - k >= 0; ++k) {
-            const int sg = nst - k;
-            tc::mbar_wait(&s_mbar[sg & 1], (uint32_t)(sg >> 1) & 1u, kTcWaitPolls / 64 + 1);
-        }
+        for (int k = 1; k <= 2 && nu - k >= 0; ++k)
+            tc::mbar_wait(&s_mbar[(nu - k) & 1], (uint32_t)((nu - k) >> 1) & 1u, kTcWaitPolls / 64 + 1);
         tc::fence_before_sync();
         __syncthreads();
     }
     tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tmem, C::TCOLS);
+    if (warp == 0) tc::tmem_dealloc(tmem, 2 * C::DCOLS);
     if (!ok && lane == 0) atomicOr(err, 1u);
 }
 
@@ -1279,7 +1375,7 @@ static void refresh_images(NN *p, cudaStream_t s) {
     int most = 0;
     for (int i = 0; i < kImages; ++i)
         for (int l = 0; l < kConvLayers; ++l) {
-            const int count = kCin[l] * 9 * kCout[l];
+            const int count = (kImageCob[i][l] == 0 && kCin[l] == 1 ? 16 : 9 * kCin[l]) * kCout[l];
             a.l[i * kConvLayers + l] = {p->bf + p->L.cw[l], p->wprep + p->wprep_off[i][l], kCin[l], kImageCob[i][l], count};
             most = std::max(most, count);
         }
@@ -1313,9 +1409,20 @@ static dd_status launch_fc1(NN *p, int n, cudaStream_t s) {
     return DD_OK;
 }
 
+// The fully connected layers, from the features in pooled[3] to the logits in z.
+static dd_status nn_fc(NN *p, int n, cudaStream_t s) {
+    // fc1: 16 outputs per block while all blocks of 16 snippets fit one wave of
+    // two per SM (12 us against 20 us with 64 outputs at 256 snippets; 74
+    // against 56 us at 4096)
+    const dd_status st =
+        (n + 15) / 16 * (kFcHid / 16) <= 2 * p->nsm ? launch_fc1<16, 16>(p, n, s) : launch_fc1<64, 16>(p, n, s);
+    if (st != DD_OK) return st;
+    fc2_fwd_kernel<<<(n + 63) / 64, 64, 0, s>>>(p->h1, p->bf + p->L.f2w, p->bf + p->L.f2b, n, p->z);
+    return DD_OK;
+}
+
 // with_arg: record the pooling argmax of every layer (the backward pass needs it).
 static dd_status nn_forward(NN *p, const uint16_t *x, int n, cudaStream_t s, bool with_arg) {
-    const Layout &L = p->L;
     if (((uintptr_t)x) % 4 != 0) return fail(DD_ERR_INVALID_ARG, "snippets must be 4-byte aligned");
     // Narrow blocks (16 output channels, 128 or 256 threads) when the wide ones
     // (all or 32 output channels, 512 threads) would give an SM no more than
@@ -1337,40 +1444,34 @@ static dd_status nn_forward(NN *p, const uint16_t *x, int n, cudaStream_t s, boo
     if (st == DD_OK)
         st = nar3 ? launch_conv_fwd<128, 64, 64, 8, 16, 8, 4, 12, 3>(p, 3, p->pooled[2], n, with_arg, s)
                   : launch_conv_fwd<512, 64, 64, 8, 64, 8, 8, 12, 3>(p, 3, p->pooled[2], n, with_arg, s);
-    // fc1: 16 outputs per block while all blocks of 16 snippets fit one wave of
-    // two per SM (12 us against 20 us with 64 outputs at 256 snippets; 74
-    // against 56 us at 4096)
-    if (st == DD_OK)
-        st = (n + 15) / 16 * (kFcHid / 16) <= 2 * p->nsm ? launch_fc1<16, 16>(p, n, s) : launch_fc1<64, 16>(p, n, s);
+    if (st == DD_OK) st = nn_fc(p, n, s);
     if (st != DD_OK) return st;
-    fc2_fwd_kernel<<<(n + 63) / 64, 64, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
     return cuda_fail(cudaGetLastError(), "classifier forward");
 }
 
 // Inference forward: tensor-core convolutions with channel-last activations
-// (stored in the pooled buffers), then the fully connected layers.
+// (stored in the pooled buffers; the last layer writes fc1's order), then the
+// fully connected layers.
 static dd_status nn_forward_tc(NN *p, const uint16_t *x, int n, cudaStream_t s) {
     const Layout &L = p->L;
-    const uint16_t *in = x;
-#define DD_CONV_TC(l, CI, CO, H, TPC)                                                                         \
+    auto wk = [&](int l) { return reinterpret_cast<const uint16_t *>(p->wprep + p->wprep_off[2][l]); };
+    conv0_tc_kernel<<<std::min(3 * p->nsm, 8 * n), 256, 0, s>>>(x, wk(0), p->bf + L.cb[0], n, p->pooled[0], p->tc_err);
+#define DD_CONV_TC(l, CI, CO, H)                                                                              \
     {                                                                                                         \
-        using C = ConvTcCfg<CI, CO, H, TPC>;                                                                  \
-        auto kern = conv_tc_kernel<CI, CO, H, TPC>;                                                           \
+        using C = ConvTcCfg<CI, CO, H>;                                                                       \
+        auto kern = conv_tc_kernel<CI, CO, H>;                                                                \
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM); \
         if (e != cudaSuccess) return cuda_fail(e, "classifier forward");                                      \
-        const int ntiles = (n * C::HO * C::HO + 31) / 32;                                                     \
-        const int grid = ntiles < p->nsm * C::MINB ? ntiles : p->nsm * C::MINB;                               \
-        kern<<<grid, 256, C::SMEM, s>>>(in, p->bf + L.cw[l], p->bf + L.cb[l], n, p->pooled[l], p->tc_err);    \
-        in = p->pooled[l];                                                                                    \
+        const int grid = std::min(p->nsm, (n + C::UNIT - 1) / C::UNIT);                                       \
+        kern<<<grid, kTcThreads, C::SMEM, s>>>(p->pooled[(l) - 1], wk(l), p->bf + L.cb[l], n, p->pooled[l],   \
+                                               p->tc_err);                                                    \
     }
-    DD_CONV_TC(0, 1, 16, 64, 1)
-    DD_CONV_TC(1, 16, 32, 32, 9)
-    DD_CONV_TC(2, 32, 64, 16, 3)
-    DD_CONV_TC(3, 64, 64, 8, 1)
+    DD_CONV_TC(1, 16, 32, 32)
+    DD_CONV_TC(2, 32, 64, 16)
+    DD_CONV_TC(3, 64, 64, 8)
 #undef DD_CONV_TC
-    fc1_fwd_kernel<true><<<(n + kFc1Rows - 1) / kFc1Rows, 256, 0, s>>>(p->pooled[3], p->bf + L.f1w, p->bf + L.f1b, n,
-                                                                      p->h1);
-    fc2_fwd_kernel<<<(n + 63) / 64, 64, 0, s>>>(p->h1, p->bf + L.f2w, p->bf + L.f2b, n, p->z);
+    dd_status st = nn_fc(p, n, s);
+    if (st != DD_OK) return st;
     return cuda_fail(cudaGetLastError(), "classifier forward");
 }
 
@@ -1416,7 +1517,7 @@ dd_status dd_nn_create(dd_nn **out, int max_batch) {
     for (int i = 0; i < kImages; ++i)
         for (int l = 0; l < kConvLayers; ++l) {
             p->wprep_off[i][l] = wtot;
-            wtot += kCin[l] * 9 * kCout[l];
+            wtot += std::max(kCin[l] * 9, 16) * kCout[l];
         }
     if (e == cudaSuccess) e = cudaMalloc(&p->wprep, (size_t)wtot * 4);
     if (e == cudaSuccess) e = cudaMemset(p->wprep, 0, (size_t)wtot * 4);
