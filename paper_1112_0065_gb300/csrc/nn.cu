@@ -26,7 +26,7 @@
 #include <vector>
 
 #include "dd_internal.h"
-#include "tc.cuh"
+#include "tmem.cuh"
 
 namespace dd {
 namespace {
@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(64) fc2_fwd_kernel(const uint16_t *__restrict_
 // turn the previous unit's accumulators into outputs meanwhile.  Bound by the
 // MMAs' reads of the 4 KB operand tiles (32 cycles each): the im2col form this
 // replaces gathered 9 copies of the input and took 932 / 535 / 293 / 200 us
-// for the four layers at 8192 snippets, XX us now.  Sums are fp32 in the
+// for the four layers at 8192 snippets, 131, 121, 76 and 63 us now.  Sums are fp32 in the
 // tensor cores' own order, so the logits agree with the fixed-order forward to
 // float round-off (the training path keeps the fixed-order kernels above).
 // Polls of an MMA-completion mbarrier before a thread gives up (a poll that
