@@ -38,6 +38,8 @@ METRIC = "dedispersion Gsamp/s (nchan*ndm*nsamp)"
 KERNEL_SRCS = [os.path.join(ROOT, "paper_1112_0065_gb300", "csrc", f)
                for f in ("dedisp_kernels.cu", "tiled_tile.cuh", "tiled_launch.cuh", "tiled_g64.cu", "tc.cuh")]
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "dd_tiled_kernel_htru_1024x1500.md")
+GROUP_SRCS = [os.path.join(ROOT, "paper_1112_0065_gb300", "csrc", f) for f in ("gsum.cu", "gsum.cuh", "tma.cuh", "tc.cuh")]
+GROUP_PROFILE = os.path.join(ROOT, "profiles", "dd_gsum_kernel_htru_1024x1500.md")
 WIDTHS = tuple(1 << k for k in range(11))
 CLF_BATCH = 32768  # snippets per classifier launch (a gulp's candidates in one launch chain)
 NCU_NN_BATCH = 8192  # snippets of the classifier's profiling case
@@ -46,11 +48,12 @@ NCU_NN_BATCH = 8192  # snippets of the classifier's profiling case
 CLF_MAC_PER_SNIPPET = (64 * 64 * 16 * 1 + 32 * 32 * 32 * 16 + 16 * 16 * 64 * 32 + 8 * 8 * 64 * 64) * 9 + 1024 * 128 + 128
 
 
-def kernel_source_hash() -> str:
-    """sha256 (first 16 hex digits) of the tiled kernel's sources, in order,
-    without their whole-line // comments (a comment edit changes no kernel)."""
+def kernel_source_hash(srcs=None) -> str:
+    """sha256 (first 16 hex digits) of a kernel's sources (default: the tiled
+    kernel's), in order, without their whole-line // comments (a comment edit
+    changes no kernel)."""
     h = hashlib.sha256()
-    for path in KERNEL_SRCS:
+    for path in KERNEL_SRCS if srcs is None else srcs:
         with open(path, "rb") as f:
             for line in f:
                 if not line.lstrip().startswith(b"//"):
@@ -89,6 +92,20 @@ def profiled_traffic(shape):
                 v = line.split(":", 1)[1].split()
                 per_shape[tuple(int(x) for x in v[:3])] = float(v[3])
     return per_shape.get(tuple(shape)) if h == src_hash else None
+
+
+def profiled_group_traffic():
+    """As profiled_traffic, for the channel-group kernel on this bench's gulp."""
+    if not os.path.exists(GROUP_PROFILE):
+        return None
+    found = {}
+    with open(GROUP_PROFILE) as f:
+        for line in f:
+            key, _, v = line.partition(":")
+            if key in ("kernel_source_sha256_16", "kernel_dram"):
+                found[key] = v.strip()
+    ok = found.get("kernel_source_sha256_16") == kernel_source_hash(GROUP_SRCS)
+    return float(found["kernel_dram"]) if ok else None
 
 
 class ClockSampler:
@@ -648,7 +665,8 @@ def run_gpu(args):
         avg_kern_s = float(np.mean(kern_ms)) / 1e3
         achieved = samples_per_step / avg_kern_s / 1e12
         peak = alu_peak_tadds(float(peaks.get("sm_max_mhz", 2070.0)))
-        traffic = profiled_traffic((shape[1], shape[2], shape[3]))
+        groups = plan.uses_channel_groups(nsamp)
+        traffic = profiled_group_traffic() if groups else profiled_traffic((shape[1], shape[2], shape[3]))
         bytes_algo = NCHAN * ld_in + len(dms) * NOUT * 4
         probe = {k: round(v, 2) for k, v in probes.int_rates().items()}
         fp = probes.fp_rates()
@@ -693,7 +711,7 @@ def run_gpu(args):
                          "frac": round(achieved / peak, 4), "traffic": traffic,
                          "peak_source": ("of measured: 152 SMs x 128 INT32 add lanes x sm_max_mhz "
                                          "(MEASURED_PEAKS.json)") if peak_src == "measured" else "of fallback",
-                         "kernel": "dd_tiled_kernel", "kernel_ms": round(avg_kern_s * 1e3, 4),
+                         "kernel": "dd_gsum_kernel" if groups else "dd_tiled_kernel", "kernel_ms": round(avg_kern_s * 1e3, 4),
                          "int_issue_probe_tops": probe,
                          "hbm_frac": round(bytes_algo / avg_kern_s / 1e9 / float(peaks.get("hbm_gbs", 6800.0)), 4),
                          "realtime_factor": round(NOUT * TSAMP / avg_kern_s, 2)},
@@ -773,17 +791,20 @@ def run_ncu_nn_case(args):
 
 
 def run_ncu_case(args):
-    """Small case for an ncu capture of the tiled kernel: the single-beam band
-    and DM list with 2^18 output samples (72 MB in, 1.5 GB out), one warm-up
-    launch and two more, default tile shape."""
+    """Small case for an ncu capture of the tiled kernel (of the automatic
+    choice with --ncu-dpb 0): the single-beam band and DM list with 2^18 output
+    samples (72 MB in, 1.5 GB out), one warm-up launch and two more."""
     import torch
 
     import paper_1112_0065_gb300 as P
 
     f = synth.band_freqs(NCHAN)
     dms = synth.dm_list_piecewise(1000.0)
-    plan = P.Plan(f, TSAMP, dms, kernel=P.KERNEL_TILED, dms_per_block=args.ncu_dpb, words_per_thread=args.ncu_w,
-                  chan_chunk=args.ncu_g)
+    if args.ncu_dpb:
+        plan = P.Plan(f, TSAMP, dms, kernel=P.KERNEL_TILED, dms_per_block=args.ncu_dpb, words_per_thread=args.ncu_w,
+                      chan_chunk=args.ncu_g)
+    else:
+        plan = P.Plan(f, TSAMP, dms)
     nsamp = (1 << 18) + plan.maxdelay
     d_in = synth.device_noise_packed(NCHAN, nsamp, seed=synth.BASE_SEED)
     out = plan.alloc_output(nsamp)
@@ -836,7 +857,7 @@ def launch_table(path: str) -> int:
     """Per-step table of an ncu launch list (``--metrics gpu__time_duration.sum
     --csv`` of this bench): every kernel's launches and device time per step,
     steps counted by the median-baseline launches (one per gulp); of the
-    dedispersion kernels only the shape launched most often (the autotuner's
+    dedispersion kernels only the one launched most often (the autotuner's
     choice, once per gulp) is kept; PyTorch and library kernels of the input
     generator are left out."""
     import collections
@@ -863,11 +884,11 @@ def launch_table(path: str) -> int:
             a[0] += 1
             a[1] += v
     steps = sum(n for k, (n, _) in agg.items() if k.startswith("dd_median_kernel"))
-    tiled = [k for k in agg if k.startswith("dd_tiled_kernel")]
+    tiled = [k for k in agg if k.startswith(("dd_tiled_kernel", "dd_gsum_kernel"))]
     chosen = max(tiled, key=lambda k: agg[k][0]) if tiled else None
     rows = {}
     for k, (n, t) in agg.items():
-        if k.startswith("dd_tiled_kernel"):
+        if k in tiled:
             if k == chosen:
                 rows[k] = (t / n, 1.0)
         elif not (k.startswith("probe_kernel") or "elementwise" in k or "distribution" in k):

@@ -81,7 +81,8 @@ typedef struct dd_plan dd_plan;
 
 /* Kernel selection for a plan. */
 enum {
-    DD_KERNEL_AUTO = 0,   /* the tiled sm_103a kernel, shape from the autotuner */
+    DD_KERNEL_AUTO = 0,   /* channel-group or tiled sm_103a kernel by band, trials and gulp; tile shape from the
+                             autotuner */
     DD_KERNEL_SIMPLE = 1, /* one thread per (DM, 4 samples), global loads; for checking */
     DD_KERNEL_TILED = 2   /* the tiled kernel with the shape given in dd_options */
 };
@@ -129,6 +130,10 @@ dd_status dd_plan_kernel_shape(const dd_plan *plan, int *kernel, int *dms_per_bl
  * time in *best_ms (0 when the shape came from the cache).
  */
 dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stream, float *best_ms);
+
+/* 1 in *channel_groups if a gulp of nsamp_in samples goes to the channel-group
+ * kernel, 0 if to the tiled or the simple one. */
+dd_status dd_plan_route(const dd_plan *plan, size_t nsamp_in, int *channel_groups);
 
 /*
  * Direct dedispersion of one gulp (paper Section 2.2):
@@ -231,7 +236,8 @@ dd_status dd_batch_set(dd_batch *batch, int nbeams, const dd_beam *beams, void *
  * when the batch was created with use_graph). */
 dd_status dd_batch_launch(dd_batch *batch, void *stream);
 
-/* Batch facts: beams, output tiles, persistent grid size, tile shape. */
+/* Batch facts of the tiled kernel's form: beams, output tiles, persistent grid
+ * size, tile shape. */
 dd_status dd_batch_info(const dd_batch *batch, int *nbeams, long long *ntiles, int *grid, int *dms_per_block,
                         int *words_per_thread);
 

@@ -33,6 +33,7 @@ SIGNATURES = {
     "dd_plan_delay_table": (_I, [_P, _P]),
     "dd_plan_kernel_shape": (_I, [_P, _PI, _PI, _PI, _PI]),
     "dd_plan_autotune": (_I, [_P, _SZ, _P, _PF]),
+    "dd_plan_route": (_I, [_P, _SZ, _PI]),
     "dd_execute": (_I, [_P, _P, _SZ, _SZ, _P, _SZ, _P]),
     "dd_execute_host": (_I, [_P, _P, _SZ, _SZ, _P, _SZ, _P]),
     "dd_destroy": (None, [_P]),

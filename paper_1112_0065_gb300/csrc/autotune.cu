@@ -1,7 +1,8 @@
-// Autotuner for the tiled dedispersion kernel: times every supported tile
-// shape (DM trials per CTA x 16-sample words per lane) on the plan's own
-// delay table and a scratch gulp, keeps the fastest, and caches the choice
-// in a small text file keyed by (device name, nchan, ndm, maxdelay, gulp
+// Autotuner of the dedispersion kernels: times every supported tile shape (DM
+// trials per CTA x 16-sample words per lane) of the tiled kernel, and the
+// channel-group kernel where the plan would take it, on the plan's own delay
+// table and a scratch gulp, keeps the fastest, and caches the choice in a small
+// text file keyed by (device name, nchan, ndm, maxdelay, gulp
 // length bucket).
 #include <stdio.h>
 #include <string.h>
@@ -29,7 +30,7 @@ static std::string cache_key(const Plan *p, size_t nsamp_in) {
     return key;
 }
 
-bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out) {
+static bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out, bool *gsum_off) {
     if (p->tune_cache.empty()) return false;
     std::lock_guard<std::mutex> g(g_cache_mutex);
     FILE *f = fopen(p->tune_cache.c_str(), "r");
@@ -43,9 +44,11 @@ bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out) {
         *bar = 0;
         if (key == line) {
             TiledShape s;
-            if (sscanf(bar + 1, "%d %d %d", &s.dms_per_warp, &s.words_per_lane, &s.chan_chunk) == 3 &&
+            int tiled_won = 0;  // absent in files written before the channel-group kernel
+            if (sscanf(bar + 1, "%d %d %d %d", &s.dms_per_warp, &s.words_per_lane, &s.chan_chunk, &tiled_won) >= 3 &&
                 tiled_shape_supported(s)) {
                 *out = s;
+                *gsum_off = tiled_won != 0;
                 found = true;
             }
         }
@@ -54,12 +57,13 @@ bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out) {
     return found;
 }
 
-static void cache_store(const Plan *p, size_t nsamp_in, const TiledShape &s) {
+static void cache_store(const Plan *p, size_t nsamp_in, const TiledShape &s, bool gsum_off) {
     if (p->tune_cache.empty()) return;
     std::lock_guard<std::mutex> g(g_cache_mutex);
     FILE *f = fopen(p->tune_cache.c_str(), "a");
     if (!f) return;
-    fprintf(f, "%s|%d %d %d\n", cache_key(p, nsamp_in).c_str(), s.dms_per_warp, s.words_per_lane, s.chan_chunk);
+    fprintf(f, "%s|%d %d %d %d\n", cache_key(p, nsamp_in).c_str(), s.dms_per_warp, s.words_per_lane, s.chan_chunk,
+            gsum_off ? 1 : 0);
     fclose(f);
 }
 
@@ -73,8 +77,10 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     if (nsamp_in <= (size_t)p->maxdelay) return fail(DD_ERR_TOO_SHORT, "gulp shorter than the maximum delay");
     if (p->kernel == DD_KERNEL_SIMPLE) return fail(DD_ERR_INVALID_ARG, "plan uses the simple kernel");
     TiledShape cached;
-    if (cache_lookup(p, nsamp_in, &cached) && ensure_shape_table(p, cached) == DD_OK) {
+    bool gsum_off = false;
+    if (cache_lookup(p, nsamp_in, &cached, &gsum_off) && ensure_shape_table(p, cached) == DD_OK) {
         p->shape = cached;
+        p->gs.off = gsum_off;
         if (best_ms) *best_ms = 0.0f;
         return DD_OK;
     }
@@ -94,27 +100,41 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
     if (e != cudaSuccess) st = cuda_fail(e, "autotune setup");
+    auto timed = [&](auto launch, float &ms) {
+        const int reps = 3;
+        dd_status r = launch();  // warm-up
+        if (r != DD_OK) return r;
+        if ((e = cudaEventRecord(e0, s)) != cudaSuccess) return cuda_fail(e, "event");
+        for (int i = 0; i < reps && r == DD_OK; ++i) r = launch();
+        if (r != DD_OK) return r;
+        if ((e = cudaEventRecord(e1, s)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess)
+            return cuda_fail(e, "event");
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= reps;
+        return DD_OK;
+    };
     for (const TiledShape &cand : tiled_shape_candidates()) {
         if (st != DD_OK) break;
         if (ensure_shape_table(p, cand) != DD_OK) continue;  // shape does not fit this band
-        st = launch_tiled(p, cand, in, ld_in, nsamp_in, out, ld_out, s);  // warm-up
-        if (st != DD_OK) break;
-        const int reps = 3;
-        if ((e = cudaEventRecord(e0, s)) != cudaSuccess) { st = cuda_fail(e, "event"); break; }
-        for (int r = 0; r < reps && st == DD_OK; ++r) st = launch_tiled(p, cand, in, ld_in, nsamp_in, out, ld_out, s);
-        if (st != DD_OK) break;
-        if ((e = cudaEventRecord(e1, s)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess) {
-            st = cuda_fail(e, "event");
-            break;
-        }
         float ms = 0.f;
-        cudaEventElapsedTime(&ms, e0, e1);
-        ms /= reps;
-        if (ms < best) {
+        st = timed([&] { return launch_tiled(p, cand, in, ld_in, nsamp_in, out, ld_out, s); }, ms);
+        if (st == DD_OK && ms < best) {
             best = ms;
             best_shape = cand;
         }
     }
+    // the channel-group kernel, where the plan would take it for this gulp
+    const Plan *self = p;
+    const long long outputs = (long long)nout;
+    const bool was_off = p->gs.off;
+    p->gs.off = false;
+    if (st == DD_OK && use_gsum(&self, &outputs, 1)) {
+        float ms = 0.f;
+        st = timed([&] { return launch_gsum(p, in, ld_in, nsamp_in, out, ld_out, s); }, ms);
+        p->gs.off = st == DD_OK && ms > best;
+        if (st == DD_OK && ms < best) best = ms;
+    }
+    if (st != DD_OK) p->gs.off = was_off;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (in) cudaFree(in);
@@ -132,7 +152,7 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
             ++it;
         }
     }
-    cache_store(p, nsamp_in, best_shape);
+    cache_store(p, nsamp_in, best_shape, p->gs.off);
     if (best_ms) *best_ms = best;
     return DD_OK;
 }

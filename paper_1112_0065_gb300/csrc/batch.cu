@@ -1,6 +1,10 @@
 // Multi-beam batches: every output tile of every beam's gulp in one launch of
 // a persistent kernel (one CTA per resident slot, tiles taken from a global
-// atomic work counter), optionally captured once in a CUDA graph.
+// atomic work counter), optionally captured once in a CUDA graph.  A batch
+// whose beams, when it is created, suit the channel-group kernel launches that
+// one's persistent form and then the tiled one's; the beams are in the work
+// list of one of the two and the other finds its list empty, so that new beams
+// of another kind are served by the same launches, captured ones too.
 #include <string.h>
 
 #include <algorithm>
@@ -8,6 +12,7 @@
 #include <vector>
 
 #include "dd_internal.h"
+#include "gsum.cuh"        // gsum::BatchDesc, Args
 #include "tiled_tile.cuh"  // BatchDesc, TiledArgs, kThreads
 
 namespace dd {
@@ -21,12 +26,44 @@ struct Batch {
     std::vector<Plan *> plans;  // plans whose tables the descriptors point at
     size_t smem = 0;
     int grid = 0;
-    BatchDesc host;
+    BatchDesc host;                   // every beam, but no tiles when the channel-group kernel has them
+    long long ntiles = 0;             // tiles of the tiled kernel's shape, whichever has them
     BatchDesc *desc = nullptr;
-    unsigned long long *counter = nullptr;
+    bool may_gsum = true;             // false: the tiled kernel alone
+    GsumBatchFn gs_kernel = nullptr;
+    bool gs_big = false;
+    size_t gs_smem = 0;
+    int gs_grid = 0;
+    gsum::BatchDesc gs_host;
+    gsum::BatchDesc *gs_desc = nullptr;
+    unsigned long long *counter = nullptr;  // one per list
     bool use_graph = false;
     cudaGraphExec_t exec = nullptr;
 };
+
+// The channel-group list, empty when the beams go to the tiled kernel.
+static dd_status fill_gsum(Batch *b, int nbeams, const dd_beam *beams) {
+    gsum::BatchDesc &h = b->gs_host;
+    memset(&h, 0, sizeof(h));
+    const Plan *plans[DD_BATCH_MAX_BEAMS];
+    long long nout[DD_BATCH_MAX_BEAMS];
+    for (int i = 0; i < nbeams; ++i) {
+        plans[i] = reinterpret_cast<const Plan *>(beams[i].plan);
+        nout[i] = (long long)beams[i].nsamp_in - plans[i]->maxdelay;
+    }
+    if (!use_gsum(plans, nout, nbeams)) return DD_OK;
+    if (b->gs_kernel && gsum_big(plans[0]) != b->gs_big) return DD_OK;
+    h.nbeams = nbeams;
+    for (int i = 0; i < nbeams; ++i) {
+        dd_status st = gsum_args(plans[i], beams[i].nsamp_in, beams[i].d_out, beams[i].ld_out, &h.beam[i]);
+        if (st == DD_OK) st = gsum_map(plans[i], beams[i].d_in, beams[i].ld_in_bytes, beams[i].nsamp_in, &h.map[i]);
+        if (st != DD_OK) return st;
+        h.tile_start[i] = h.ntiles;
+        h.ntiles += (nout[i] + gsum::kTile - 1) / gsum::kTile * plans[i]->gs.n_dmb;
+    }
+    h.tile_start[nbeams] = h.ntiles;
+    return DD_OK;
+}
 
 static dd_status fill_desc(Batch *b, int nbeams, const dd_beam *beams) {
     if (nbeams < 1 || nbeams > DD_BATCH_MAX_BEAMS || !beams)
@@ -72,6 +109,12 @@ static dd_status fill_desc(Batch *b, int nbeams, const dd_beam *beams) {
     h.tile_start[nbeams] = tiles;
     h.ntiles = tiles;
     if (smem > b->smem) return fail(DD_ERR_INVALID_ARG, "beams need more shared memory than the batch was sized for");
+    if (b->may_gsum) {
+        const dd_status gs = fill_gsum(b, nbeams, beams);
+        if (gs != DD_OK) return gs;
+        if (b->gs_host.ntiles) h.ntiles = 0;
+    }
+    b->ntiles = tiles;
     // the plans' tables must outlive this batch's descriptors (the autotuner
     // keeps every table of a plan with live batches)
     for (Plan *p : b->plans) --p->live_batches;
@@ -91,8 +134,17 @@ static void free_batch(Batch *b) {
     for (Plan *p : b->plans) --p->live_batches;
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->desc) cudaFree(b->desc);
+    if (b->gs_desc) cudaFree(b->gs_desc);
     if (b->counter) cudaFree(b->counter);
     delete b;
+}
+
+static cudaError_t launch(const Batch *b, cudaStream_t stream) {
+    cudaError_t e = cudaMemsetAsync(b->counter, 0, 2 * sizeof(unsigned long long), stream);
+    if (e != cudaSuccess) return e;
+    if (b->may_gsum) b->gs_kernel<<<b->gs_grid, gsum::kThreads, b->gs_smem, stream>>>(b->gs_desc, b->counter + 1);
+    b->kernel<<<b->grid, kThreads, b->smem, stream>>>(b->desc, b->counter);
+    return cudaGetLastError();
 }
 
 }  // namespace dd
@@ -138,7 +190,17 @@ dd_status dd_batch_create(dd_batch **out, int nbeams, const dd_beam *beams, int 
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, b->kernel, kThreads, b->smem);
     if (e == cudaSuccess && per_sm < 1) e = cudaErrorInvalidConfiguration;
     if (e == cudaSuccess) e = cudaMalloc(&b->desc, sizeof(BatchDesc));
-    if (e == cudaSuccess) e = cudaMalloc(&b->counter, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc(&b->counter, 2 * sizeof(unsigned long long));
+    b->may_gsum = b->gs_host.ntiles > 0;
+    if (e == cudaSuccess && b->may_gsum) {
+        b->gs_big = gsum_big(p0);
+        b->gs_kernel = gsum_batch_kernel(b->gs_big);
+        b->gs_smem = gsum_smem();
+        b->gs_grid = sms;
+        e = cudaFuncSetAttribute(b->gs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->gs_smem);
+        if (e == cudaSuccess) e = cudaMalloc(&b->gs_desc, sizeof(gsum::BatchDesc));
+        if (e == cudaSuccess) e = cudaMemcpy(b->gs_desc, &b->gs_host, sizeof(gsum::BatchDesc), cudaMemcpyHostToDevice);
+    }
     if (e == cudaSuccess) e = cudaMemcpy(b->desc, &b->host, sizeof(BatchDesc), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         st = cuda_fail(e, "batch setup");
@@ -152,8 +214,7 @@ dd_status dd_batch_create(dd_batch **out, int nbeams, const dd_beam *beams, int 
         e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaMemsetAsync(b->counter, 0, sizeof(unsigned long long), cs);
-            b->kernel<<<b->grid, kThreads, b->smem, cs>>>(b->desc, b->counter);
+            launch(b, cs);
             e = cudaStreamEndCapture(cs, &g);
         }
         if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, g, 0);
@@ -174,9 +235,11 @@ dd_status dd_batch_set(dd_batch *batch, int nbeams, const dd_beam *beams, void *
     if (!b) return fail(DD_ERR_INVALID_ARG, "NULL batch");
     dd_status st = fill_desc(b, nbeams, beams);
     if (st != DD_OK) return st;
-    return cuda_fail(cudaMemcpyAsync(b->desc, &b->host, sizeof(BatchDesc), cudaMemcpyHostToDevice,
-                                     (cudaStream_t)stream),
-                     "uploading batch descriptors");
+    cudaError_t e = cudaMemcpyAsync(b->desc, &b->host, sizeof(BatchDesc), cudaMemcpyHostToDevice, (cudaStream_t)stream);
+    if (e == cudaSuccess && b->may_gsum)
+        e = cudaMemcpyAsync(b->gs_desc, &b->gs_host, sizeof(gsum::BatchDesc), cudaMemcpyHostToDevice,
+                            (cudaStream_t)stream);
+    return cuda_fail(e, "uploading batch descriptors");
 }
 
 dd_status dd_batch_launch(dd_batch *batch, void *stream) {
@@ -184,9 +247,7 @@ dd_status dd_batch_launch(dd_batch *batch, void *stream) {
     if (!b) return fail(DD_ERR_INVALID_ARG, "NULL batch");
     cudaStream_t s = (cudaStream_t)stream;
     if (b->use_graph) return cuda_fail(cudaGraphLaunch(b->exec, s), "cudaGraphLaunch");
-    DD_CUDA_TRY(cudaMemsetAsync(b->counter, 0, sizeof(unsigned long long), s));
-    b->kernel<<<b->grid, kThreads, b->smem, s>>>(b->desc, b->counter);
-    return cuda_fail(cudaGetLastError(), "dd_batch_kernel launch");
+    return cuda_fail(launch(b, s), "dd_batch_kernel launch");
 }
 
 dd_status dd_batch_info(const dd_batch *batch, int *nbeams, long long *ntiles, int *grid, int *dms_per_block,
@@ -194,7 +255,7 @@ dd_status dd_batch_info(const dd_batch *batch, int *nbeams, long long *ntiles, i
     const Batch *b = reinterpret_cast<const Batch *>(batch);
     if (!b) return fail(DD_ERR_INVALID_ARG, "NULL batch");
     if (nbeams) *nbeams = b->host.nbeams;
-    if (ntiles) *ntiles = b->host.ntiles;
+    if (ntiles) *ntiles = b->ntiles;
     if (grid) *grid = b->grid;
     if (dms_per_block) *dms_per_block = kWarps * b->shape.dms_per_warp;
     if (words_per_thread) *words_per_thread = b->shape.words_per_lane;

@@ -2,6 +2,7 @@
 // Nothing here is part of the C ABI (include/dd.h is).
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -44,6 +45,17 @@ struct ShapeTable {
     int group = 64;            // channels per shared-memory stage
 };
 
+// Device tables of the channel-group kernel (gsum.cuh); ok: the plan's delays
+// suit it (few distinct combinations, everything fits in shared memory).
+struct GsumTable {
+    bool ok = false;
+    bool off = false;        // the autotuner measured the tiled kernel faster
+    uint32_t *tab = nullptr;
+    int32_t *ws = nullptr;
+    int n_dmb = 0, nchunks = 0, slot = 0, sms = 0;
+    double tile_cycles = 0;  // estimated SM cycles of one tile
+};
+
 struct Plan {
     int nchan = 0;
     int ndm = 0;
@@ -57,6 +69,7 @@ struct Plan {
     int kernel = DD_KERNEL_AUTO;
     TiledShape shape;
     std::map<int, ShapeTable> tables;   // keyed by shape_key()
+    GsumTable gs;                       // channel-group tables (automatic plans only)
     int live_batches = 0;               // batches whose descriptors point at these tables
     std::string tune_cache;
     // host-API staging (dd_execute_host), grown on demand
@@ -95,6 +108,26 @@ DD_DECLARE_GROUP(64)
 DD_DECLARE_GROUP(128)
 #undef DD_DECLARE_GROUP
 BatchKernelFn batch_kernel(const TiledShape &s, bool big);
+
+// Channel-group kernel (gsum.cu).  build_gsum leaves p->gs.ok false when the
+// plan does not suit it; use_gsum decides for n gulps of nout[i] outputs with
+// plans p[i] that go in one launch.
+namespace gsum {
+struct Args;
+struct BatchDesc;
+}
+using GsumBatchFn = void (*)(const gsum::BatchDesc *, unsigned long long *);
+void build_gsum(Plan *p);
+void free_gsum(Plan *p);
+bool use_gsum(const Plan *const *p, const long long *nout, int n);
+inline bool gsum_big(const Plan *p) { return 3 * p->nchan >= 1 << 12; }  // 14 bit-planes instead of 12
+dd_status launch_gsum(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, size_t nsamp_in, uint32_t *d_out,
+                      size_t ld_out, cudaStream_t stream);
+dd_status gsum_args(const Plan *p, size_t nsamp_in, uint32_t *d_out, size_t ld_out, gsum::Args *out);
+dd_status gsum_map(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, size_t nsamp_in, CUtensorMap *map);
+GsumBatchFn gsum_batch_kernel(bool big);
+size_t gsum_smem();
+
 bool tiled_shape_supported(const TiledShape &s);
 dd_status ensure_shape_table(Plan *p, const TiledShape &s);
 void free_shape_tables(Plan *p);

@@ -93,9 +93,16 @@ int max_block_spread(const Plan *p, int dpb) {
     return best;
 }
 
+static bool takes_gsum(const Plan *p, size_t nsamp_in) {
+    const long long nout = (long long)nsamp_in - p->maxdelay;
+    return use_gsum(&p, &nout, 1);
+}
+
 static dd_status run(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, size_t nsamp_in, uint32_t *d_out,
                      size_t ld_out, cudaStream_t stream) {
     if (p->kernel == DD_KERNEL_SIMPLE) return launch_simple(p, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
+    if (takes_gsum(p, nsamp_in))
+        return launch_gsum(p, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
     return launch_tiled(p, p->shape, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
 }
 
@@ -195,6 +202,8 @@ dd_status dd_plan_create(dd_plan **out, int nchan, const double *freqs_mhz, doub
             p->kernel = DD_KERNEL_SIMPLE;  // delay spread beyond the tiled kernel's shared memory
         }
     }
+    // the channel-group kernel for automatic plans (a given shape asks for the tiled kernel)
+    if (p->kernel == DD_KERNEL_AUTO && !(o.dms_per_block || o.words_per_thread || o.chan_chunk)) build_gsum(p);
     *out = reinterpret_cast<dd_plan *>(p);
     return DD_OK;
 }
@@ -223,6 +232,14 @@ dd_status dd_plan_kernel_shape(const dd_plan *plan, int *kernel, int *dms_per_bl
     if (dms_per_block) *dms_per_block = p->shape.dms_per_warp * 8;
     if (words_per_thread) *words_per_thread = p->shape.words_per_lane;
     if (chan_chunk) *chan_chunk = p->shape.chan_chunk;
+    return DD_OK;
+}
+
+dd_status dd_plan_route(const dd_plan *plan, size_t nsamp_in, int *channel_groups) {
+    const Plan *p = reinterpret_cast<const Plan *>(plan);
+    if (!p || !channel_groups) return fail(DD_ERR_INVALID_ARG, "NULL plan or output");
+    if (nsamp_in <= (size_t)p->maxdelay) return fail(DD_ERR_TOO_SHORT, "gulp shorter than the maximum delay");
+    *channel_groups = takes_gsum(p, nsamp_in) ? 1 : 0;
     return DD_OK;
 }
 
@@ -270,6 +287,7 @@ void dd_destroy(dd_plan *plan) {
     if (!p) return;
     if (p->delays_dev) cudaFree(p->delays_dev);
     free_shape_tables(p);
+    free_gsum(p);
     if (p->stage_in) cudaFree(p->stage_in);
     if (p->stage_out) cudaFree(p->stage_out);
     delete p;

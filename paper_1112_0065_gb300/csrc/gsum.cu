@@ -1,0 +1,389 @@
+// Host side of the channel-group dedispersion (gsum.cuh): the vectors of a
+// plan, its tables, the rule that chooses between it and the tiled kernel, and
+// the launches.
+#include <stdlib.h>
+#include <math.h>
+#include <stdio.h>
+#include <string.h>
+
+#include <algorithm>
+#include <vector>
+
+#include "dd_internal.h"
+#include "gsum.cuh"
+
+namespace dd {
+
+using namespace gsum;
+
+namespace {
+
+template <int NP>
+__global__ void __launch_bounds__(kThreads, 1)
+    dd_gsum_kernel(const __grid_constant__ Args args, const __grid_constant__ CUtensorMap map) {
+    extern __shared__ __align__(128) unsigned char gsum_smem[];
+    Args a = args;
+    a.map = &map;
+    init_bars(gsum_smem);
+    Phases phase;
+    gsum_tile<NP>(a, (int)(blockIdx.x % (unsigned)a.n_dmb), (long long)(blockIdx.x / (unsigned)a.n_dmb), gsum_smem,
+                  phase);
+}
+
+// Persistent multi-beam form, as tiled::dd_batch_kernel.
+template <int NP>
+__global__ void __launch_bounds__(kThreads, 1)
+    dd_gsum_batch_kernel(const gsum::BatchDesc *__restrict__ desc, unsigned long long *__restrict__ counter) {
+    extern __shared__ __align__(128) unsigned char gsum_smem[];
+    long long &s_tile = *reinterpret_cast<long long *>(gsum_smem + kTileWord);
+    const long long ntiles = desc->ntiles;
+    init_bars(gsum_smem);
+    // the maps lie in global memory, which the host writes between launches
+    if ((int)threadIdx.x < desc->nbeams) tc::fence_tensormap(&desc->map[threadIdx.x]);
+    Phases phase;
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = (long long)atomicAdd(counter, 1ULL);
+        __syncthreads();
+        const long long g = s_tile;
+        __syncthreads();
+        if (g >= ntiles) break;
+        int b = 0;
+        while (b + 1 < desc->nbeams && g >= desc->tile_start[b + 1]) ++b;
+        Args a = desc->beam[b];
+        a.map = &desc->map[b];
+        const long long local = g - desc->tile_start[b];
+        if (!gsum_tile<NP>(a, (int)(local % a.n_dmb), local / a.n_dmb, gsum_smem, phase)) break;
+        __syncthreads();
+    }
+}
+
+// The vectors of one group over one block of trials.
+struct Group {
+    int nchan = 0;         // channels of the band in it
+    int nvec = 0;
+    int words = 0;         // words of a vector that some trial reads
+    int start[kG] = {};    // first sample of each channel relative to the tile
+    uint32_t vec[kD];      // extra delays of channels 1..4, 8 bits each (channel 1 highest), ascending
+    uint8_t of[kD];        // vector of each trial
+    int off[kD];           // the trial's offset in samples
+};
+
+// false: some channel's delay, relative to the group's first, spreads over
+// more than one word.
+bool make_group(const Plan *p, int d0, int c0, Group &g) {
+    g.nchan = std::min(kG, p->nchan - c0);
+    const int nd = std::min(kD, p->ndm - d0);
+    const int32_t *first = p->delays_host.data() + (size_t)d0 * p->nchan + c0;
+    int lo[kG], rel[kD][kG] = {};
+    for (int i = 0; i < kG; ++i) lo[i] = i < g.nchan ? 0x7fffffff : 0;
+    for (int j = 0; j < nd; ++j) {
+        const int32_t *r = first + (size_t)j * p->nchan;
+        g.off[j] = r[0] - first[0];
+        for (int i = 0; i < g.nchan; ++i) {
+            rel[j][i] = r[i] - r[0];
+            lo[i] = std::min(lo[i], rel[j][i]);
+        }
+    }
+    for (int i = 0; i < kG; ++i) g.start[i] = first[0] + lo[i];
+    uint32_t key[kD];
+    g.nvec = 0;
+    for (int j = 0; j < nd; ++j) {
+        key[j] = 0;
+        for (int i = 1; i < kG; ++i) {
+            const int e = rel[j][i] - lo[i];
+            if (e > 15) return false;
+            key[j] = key[j] << 8 | (uint32_t)e;
+        }
+        if (j && key[j] == key[j - 1]) continue;
+        uint32_t *end = g.vec + g.nvec, *at = std::lower_bound(g.vec, end, key[j]);
+        if (at != end && *at == key[j]) continue;
+        memmove(at + 1, at, (size_t)(end - at) * sizeof(uint32_t));
+        *at = key[j];
+        ++g.nvec;
+    }
+    for (int j = 0; j < nd; ++j)
+        g.of[j] = j && key[j] == key[j - 1] ? g.of[j - 1]
+                                            : (uint8_t)(std::lower_bound(g.vec, g.vec + g.nvec, key[j]) - g.vec);
+    for (int j = nd; j < kD; ++j) {  // past the last trial: as the last
+        g.off[j] = g.off[nd - 1];
+        g.of[j] = g.of[nd - 1];
+    }
+    g.words = (g.off[kD - 1] >> 4) + kHalfWords + 1;  // delays never fall with the trial
+    return true;
+}
+
+using Encode = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                            const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                            CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// The driver's tensor-map encoder, nullptr when it has none.
+Encode gsum_encoder() {
+    static const Encode encode = [] {
+        void *fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) !=
+                cudaSuccess ||
+            found != cudaDriverEntryPointSuccess)
+            fn = nullptr;
+        return reinterpret_cast<Encode>(fn);
+    }();
+    return encode;
+}
+
+}  // namespace
+
+// Dynamic shared memory of a CTA, for every plan: all there is.
+size_t gsum_smem() { return 227 * 1024; }
+
+// Sizes and host tables of a plan; t.ok stays false when the plan does not suit.
+static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab, std::vector<int32_t> &ws) {
+    if (p->nchan < kChunkChans || 3 * p->nchan >= 1 << 14) return;
+    t.n_dmb = (p->ndm + kD - 1) / kD;
+    const int ngroups = (p->nchan + kG - 1) / kG;
+    t.nchunks = ((ngroups + kCG - 1) / kCG + 1) / 2 * 2;
+    std::vector<Group> groups((size_t)t.n_dmb * t.nchunks * kCG);
+    std::vector<int> from_word((size_t)t.n_dmb * t.nchunks * kParts);  // first staged word of each part
+    int most = 0;
+    for (int b = 0; b < t.n_dmb; ++b)
+        for (int s = 0; s < t.nchunks * kParts; ++s) {
+            const size_t k = (size_t)b * t.nchunks * kParts + s;
+            int lo = 0x7fffffff, end = 0;
+            for (int g = 0; g < kHalfCG && s * kHalfCG + g < ngroups; ++g) {
+                Group &x = groups[k * kHalfCG + g];
+                if (!make_group(p, b * kD, (s * kHalfCG + g) * kG, x)) return;
+                for (int i = 0; i < x.nchan; ++i) {
+                    lo = std::min(lo, x.start[i] >> 4);
+                    end = std::max(end, (x.start[i] >> 4) + x.words);
+                }
+            }
+            if (s * kHalfCG >= ngroups) continue;
+            from_word[k] = lo & ~3;
+            most = std::max(most, end - from_word[k]);
+        }
+    t.slot = (most + kHalfWords + 2 + 3) / 4 * 4;
+    if (t.slot > 256) return;  // a tensor map's box
+    tab.assign((size_t)t.n_dmb * t.nchunks * kRecWords, 0u);
+    ws.assign((size_t)t.n_dmb * 2 * kParts, 0);
+    // Places in the pool.  First choice for a DM block: each chunk after one of
+    // the chunks before it or at the bottom, clear of at least the two before it.
+    // Else even chunks at the bottom and odd ones at the top.  Half a vector is
+    // padded to 4 cells more than a multiple of 8 where there is room in the DM
+    // block: the even and odd words that a quarter-warp stores then fall into
+    // different banks.
+    const int pool = (int)gsum_smem() - vec_at(t.slot);
+    const int nparts = t.nchunks * kParts;
+    std::vector<int> need((size_t)t.n_dmb * nparts), half(need.size()), place(need.size());
+    std::vector<int> keep((size_t)t.n_dmb * t.nchunks);  // chunks before it that a chunk's place is clear of
+    for (int b = 0; b < t.n_dmb; ++b) {
+        bool fits = false;
+        for (int way = 0; way < 4 && !fits; ++way) {
+            const bool pad = !(way & 1), ends = way >= 2;
+            long long from[kBRing] = {}, to[kBRing] = {};  // by chunk % kBRing
+            fits = true;
+            for (int s = 0; s < t.nchunks && fits; ++s) {
+                long long bytes[kParts], all = 0;
+                for (int q = 0; q < kParts; ++q) {
+                    const size_t n = (size_t)b * nparts + s * kParts + q;
+                    int nv = 0;
+                    need[n] = 0;
+                    for (int g = 0; g < kHalfCG; ++g) {
+                        need[n] = std::max(need[n], groups[n * kHalfCG + g].words);
+                        nv += groups[n * kHalfCG + g].nvec;
+                    }
+                    half[n] = (need[n] + 1) / 2;
+                    while (pad && half[n] && half[n] % 8 != 4) ++half[n];
+                    bytes[q] = (long long)nv * half[n] * 32;
+                    all += bytes[q];
+                }
+                // how many of the chunks just before s (kBRing - 1 at most) a place is clear of
+                auto clear = [&](long long at) {
+                    int w = 0;
+                    if (at < 0 || at + all > pool) return 0;
+                    for (; w < kBRing - 1 && w < s; ++w)
+                        if (at < to[(s - 1 - w) % kBRing] && at + all > from[(s - 1 - w) % kBRing]) return w;
+                    return kBRing - 1;
+                };
+                long long at = ends && (s & 1) ? pool - all : 0;
+                int w = clear(at);
+                for (int q = 0; q < kBRing - 1 && q < s && !ends; ++q)
+                    if (clear(to[(s - 1 - q) % kBRing]) > w) {
+                        at = to[(s - 1 - q) % kBRing];
+                        w = clear(at);
+                    }
+                fits = w >= (ends ? 1 : 2);
+                keep[(size_t)b * t.nchunks + s] = w;
+                from[s % kBRing] = at;
+                to[s % kBRing] = at + all;
+                for (int q = 0; q < kParts; ++q) {
+                    place[(size_t)b * nparts + s * kParts + q] = (int)at;
+                    at += bytes[q];
+                }
+            }
+        }
+        if (!fits) return;
+    }
+    double alu = 0;  // ALU instructions of all DM blocks' tiles, per warp
+    int turn = 0;  // items go round the warps
+    for (int b = 0; b < t.n_dmb; ++b) {
+        for (int q = 0; q < 2 * kParts; ++q) ws[(size_t)b * 2 * kParts + q] = from_word[(size_t)b * nparts + q];
+        for (int s = 0; s < t.nchunks; ++s) {
+            const size_t k = (size_t)b * t.nchunks + s;
+            uint32_t *ra = tab.data() + k * kRecWords;
+            uint32_t *rb = ra + kAWords;
+            for (int part = 0; part < kParts; ++part) {
+                const Group *gr = &groups[k * kCG + part * kHalfCG];
+                const size_t n = k * kParts + part;
+                uint32_t *r = ra + part * kPartWords;
+                const int units = (kHalfCG * need[n] + 31) / 32;
+                r[0] = (uint32_t)half[n];
+                r[1] = (uint32_t)need[n];
+                r[3] = s + 2 < t.nchunks ? (uint32_t)from_word[(k + 2) * kParts + part] : 0u;
+                r[2] = (uint32_t)units | (uint32_t)(turn % kWarps) << 8 | (uint32_t)keep[k] << 16;
+                turn += units;
+                uint32_t at = (uint32_t)(vec_at(t.slot) + place[n]);
+                double vwork = 0;
+                for (int g = 0; g < kHalfCG; ++g) {
+                    const Group &x = gr[g];
+                    uint32_t *q = r + 4 + g * kARec;
+                    for (int i = 0; i < kG; ++i) {
+                        q[i] = i < x.nchan
+                                   ? (uint32_t)(raw_at(t.slot, s & 1) + part * raw_bytes(t.slot) +
+                                                4 * ((g * kG + i) * t.slot + (x.start[i] >> 4) - from_word[k * kParts + part])) << 5 |
+                                         (uint32_t)(2 * (x.start[i] & 15))
+                                   : (uint32_t)zero_at(t.slot) << 5;
+                    }
+                    q[5] = at;
+                    q[6] = (uint32_t)x.nvec;
+                    for (int v = 0; v < x.nvec; ++v) {
+                        const uint32_t e = x.vec[v];
+                        const bool fresh = v == 0 || (e >> 16) != (x.vec[v - 1] >> 16);
+                        q[8 + 2 * v] = 2 * (e >> 8 & 255) | 2 * (e & 255) << 8 | (fresh ? 0x80u : 0u);
+                        q[9 + 2 * v] = 2 * (e >> 24) | 2 * (e >> 16 & 255) << 8;
+                        vwork += fresh ? 28 : 20;
+                    }
+                    for (int j = 0; j < kD; ++j) {
+                        uint32_t *e = rb + ((part * kHalfCG + g) * kD + j) * 2;
+                        if (x.nchan == 0) {
+                            e[0] = (uint32_t)zero_at(t.slot);
+                            continue;
+                        }
+                        const int o = x.off[j] >> 4, h16 = 16 * half[n];
+                        e[0] = at + (uint32_t)(x.of[j] * 2 * h16 + ((o & 1) ? h16 : 0) + 16 * (o >> 1));
+                        e[1] = (uint32_t)((o & 1) ? 16 - h16 : h16) << 5 | (uint32_t)(2 * (x.off[j] & 15));
+                    }
+                    at += (uint32_t)(x.nvec * 32 * half[n]);
+                }
+                alu += kWarps * kDT * kHalfCG * 31.0 + units * (70 + vwork / kHalfCG);
+            }
+        }
+    }
+    if (pool < kWarps * kHalf * 4) return;  // the finished sums pass through the pool's place
+    // two of the ALU's warp instructions a cycle at the 80 % that the kernel reaches
+    t.tile_cycles = 0.615 * alu / t.n_dmb + 14400;
+    t.ok = true;
+}
+
+void build_gsum(Plan *p) {
+    GsumTable &t = p->gs;
+    std::vector<uint32_t> tab;
+    std::vector<int32_t> ws;
+    gsum_tables(p, t, tab, ws);
+    if (!t.ok || !gsum_encoder()) return free_gsum(p);
+    cudaError_t e = cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e == cudaSuccess) e = cudaMalloc(&t.tab, tab.size() * 4);
+    if (e == cudaSuccess) e = cudaMalloc(&t.ws, ws.size() * 4);
+    if (e == cudaSuccess) e = cudaMemcpy(t.tab, tab.data(), tab.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(t.ws, ws.data(), ws.size() * 4, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {  // no memory for them: the tiled kernel serves the plan
+        cudaGetLastError();
+        free_gsum(p);
+    }
+}
+
+void free_gsum(Plan *p) {
+    if (p->gs.tab) cudaFree(p->gs.tab);
+    if (p->gs.ws) cudaFree(p->gs.ws);
+    p->gs = GsumTable();
+}
+
+// The rule compares estimates of SM cycles: tiles in waves of one per SM here
+// (GsumTable::tile_cycles each), and in half waves on the tiled kernel (two of
+// its CTAs, 16 trials x 1536 outputs, share an SM), whose tiles take 9200 + 86
+// cycles a channel (98 with 15 bit-planes).  Both fit the measured times within
+// 4 % over 20 to 2048 channels, 24 to 1500 trials and 2000 to 131072 outputs,
+// and what they leave out, some 8 us of launch and first copies, is the same.
+// A gulp too short to fill the waves stays on the tiled kernel, whose tiles are
+// smaller.  Measured, tiled / here, in us: 1024 channels x 1500 trials x 6208
+// outputs 214 / 236, x 10000 267 / 243, x 131072 2778 / 2372; 1024 x 64 x 40000
+// 64 / 111, x 131072 165 / 111; 2048 x 700 x 131072 2783 / 2069; 1024 x 1000
+// linear trials to DM 1000 (many vectors) x 20000 320 / 390, x 131072 1861 /
+// 1799; 96 x 1500 x 131072 531 / 367; 20 x 400 x 6208 13.6 / 14.9, x 10000
+// 19.4 / 15.1.
+bool use_gsum(const Plan *const *p, const long long *nout, int n) {
+    double tiles = 0, work = 0, tiles16 = 0, work16 = 0;
+    for (int i = 0; i < n; ++i) {
+        const GsumTable &t = p[i]->gs;
+        if (!t.ok || t.off || gsum_big(p[i]) != gsum_big(p[0])) return false;
+        const double m = (double)((nout[i] + kTile - 1) / kTile) * t.n_dmb;
+        tiles += m;
+        work += m * t.tile_cycles;
+        const double m16 = (double)((nout[i] + 1535) / 1536) * ((p[i]->ndm + 15) / 16);
+        tiles16 += m16;
+        work16 += m16 * (9200.0 + p[i]->nchan * (p[i]->nchan < 2048 ? 86.0 : 98.0));
+    }
+    const double sms = p[0]->gs.sms;
+    return work / tiles * ceil(tiles / sms) < work16 / tiles16 * ceil(tiles16 / sms);
+}
+
+// Tensor map of a gulp's packed rows as words, box = the windows of a part's
+// channels; words past the gulp's end read as 0.
+dd_status gsum_map(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, size_t nsamp_in, CUtensorMap *map) {
+    const cuuint64_t dim[2] = {(cuuint64_t)((nsamp_in + 15) / 16), (cuuint64_t)p->nchan};
+    const cuuint64_t stride[1] = {(cuuint64_t)ld_in_bytes};
+    const cuuint32_t box[2] = {(cuuint32_t)p->gs.slot, (cuuint32_t)kPartChans}, one[2] = {1, 1};
+    const CUresult r = gsum_encoder()(map, CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, const_cast<uint8_t *>(d_in), dim, stride,
+                                      box, one, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? DD_OK : fail(DD_ERR_CUDA, "cuTensorMapEncodeTiled: error %d", (int)r);
+}
+
+dd_status gsum_args(const Plan *p, size_t nsamp_in, uint32_t *d_out, size_t ld_out, gsum::Args *out) {
+    const GsumTable &t = p->gs;
+    Args a;
+    a.map = nullptr;
+    a.tab = t.tab;
+    a.ws = t.ws;
+    a.nchan = p->nchan;
+    a.nchunks = t.nchunks;
+    a.ndm = p->ndm;
+    a.n_dmb = t.n_dmb;
+    a.slot = t.slot;
+    a.nout = (long long)nsamp_in - p->maxdelay;
+    a.out = d_out;
+    a.ld_out = (long long)ld_out;
+    a.poll_limit = tiled::kStagePollLimit;
+    const dd_status es = tile_error_word(&a.err);
+    if (es != DD_OK) return es;
+    *out = a;
+    return DD_OK;
+}
+
+GsumBatchFn gsum_batch_kernel(bool big) { return big ? dd_gsum_batch_kernel<14> : dd_gsum_batch_kernel<12>; }
+
+dd_status launch_gsum(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, size_t nsamp_in, uint32_t *d_out,
+                      size_t ld_out, cudaStream_t stream) {
+    Args a;
+    dd_status st = gsum_args(p, nsamp_in, d_out, ld_out, &a);
+    if (st != DD_OK) return st;
+    CUtensorMap map;
+    st = gsum_map(p, d_in, ld_in_bytes, nsamp_in, &map);
+    if (st != DD_OK) return st;
+    const long long nblocks = (a.nout + kTile - 1) / kTile * a.n_dmb;
+    if (nblocks > 0x7fffffffLL) return fail(DD_ERR_INVALID_ARG, "gulp too long for one launch");
+    auto kern = gsum_big(p) ? dd_gsum_kernel<14> : dd_gsum_kernel<12>;
+    DD_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsum_smem()));
+    kern<<<(unsigned)nblocks, kThreads, gsum_smem(), stream>>>(a, map);
+    return cuda_fail(cudaGetLastError(), "dd_gsum_kernel launch");
+}
+
+}  // namespace dd

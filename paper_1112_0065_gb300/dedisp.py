@@ -76,6 +76,12 @@ class Plan:
         _lib.check(self._L.dd_plan_kernel_shape(self._h, *[ctypes.byref(x) for x in v]), "dd_plan_kernel_shape")
         return tuple(x.value for x in v)
 
+    def uses_channel_groups(self, nsamp_in: int) -> bool:
+        """Whether a gulp of nsamp_in samples goes to the channel-group kernel."""
+        v = ctypes.c_int()
+        _lib.check(self._L.dd_plan_route(self._h, nsamp_in, ctypes.byref(v)), "dd_plan_route")
+        return bool(v.value)
+
     def autotune(self, nsamp_in: int, stream=None) -> float:
         ms = ctypes.c_float()
         _lib.check(self._L.dd_plan_autotune(self._h, nsamp_in, _stream_handle(stream), ctypes.byref(ms)),

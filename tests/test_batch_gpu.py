@@ -222,3 +222,41 @@ def test_multibeam_batch_equals_single_gulp(P):
         got = out[torch.as_tensor(di, device="cuda").long(), torch.as_tensor(ti, device="cuda").long()]
         np.testing.assert_array_equal(got.cpu().numpy().view(np.uint32), want)
     batch.close()
+
+
+@pytest.mark.parametrize("use_graph", [False, True])
+def test_batch_changes_kernels_with_its_beams(P, use_graph):
+    """A batch created on beams that the channel-group kernel takes serves, by
+    its own launch and by a captured one, such beams, then one that the tiled
+    kernel takes, then others and the first again."""
+    import torch
+
+    f = synth.band_freqs(40)
+    dms = synth.dm_list_linear(96, 5.0)
+    kinds, wants = [], []
+    for nouts in ((70001, 52000), (5000,), (90000, 40010)):  # 5000 outputs: too few for the channel-group kernel
+        beams, want = [], []
+        for i, nout in enumerate(nouts):
+            plan = P.Plan(f, 64e-6, dms)
+            nsamp = nout + plan.maxdelay
+            packed, _ = synth.make_gulp(nout, 40, nsamp)
+            out = plan.alloc_output(nsamp)
+            beams.append((plan, torch.from_numpy(packed).cuda(), nsamp, out))
+            want.append(oracle.dedisperse(oracle.delay_table(f, 64e-6, dms), packed, nsamp))
+        kinds.append(beams)
+        wants.append(want)
+    b = P.Batch(kinds[0], use_graph=use_graph)
+    assert kinds[0][0][0].uses_channel_groups(kinds[0][0][2]) and not kinds[1][0][0].uses_channel_groups(kinds[1][0][2])
+    b.launch()
+    _check(P, kinds[0], wants[0])
+    captured = torch.cuda.CUDAGraph() if not use_graph else None
+    if captured is not None:
+        with torch.cuda.graph(captured):
+            b.launch()
+    for beams, want in list(zip(kinds, wants))[1:] + [(kinds[0], wants[0])]:
+        for _, _, _, out in beams:
+            out.fill_(-1)
+        b.set(beams)
+        captured.replay() if captured is not None else b.launch()
+        _check(P, beams, want)
+    b.close()

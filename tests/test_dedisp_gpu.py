@@ -374,3 +374,47 @@ def test_tile_gives_up_without_fault(P):
     plan = P.Plan(f, 64e-6, dms)
     np.testing.assert_array_equal(_run(P, plan, packed, nsamp), oracle.dedisperse(delays, packed, nsamp))
     plan.close()
+
+
+# gulps long enough for the automatic choice to leave the tiled kernel:
+# (nchan, trials, last DM, outputs): partial groups and chunks of channels,
+# blocks of trials (32) and tiles (2048 outputs), the last channel counts of
+# 12 bit-planes and the first of 14, many and few vectors, long delays
+GROUP_CASES = [
+    (20, 400, 3.0, 10240), (21, 385, 3.0, 10239), (39, 64, 5.0, 153600), (40, 33, 5.0, 155648),
+    (63, 65, 8.0, 102397), (96, 1500, 60.0, 4609), (333, 90, 10.0, 78000), (1024, 0, 250.0, 9217),
+    (1365, 64, 8.0, 150001), (1366, 64, 8.0, 150001), (2048, 32, 30.0, 309000),
+]
+
+
+@pytest.mark.parametrize("case", GROUP_CASES)
+def test_channel_groups_equal_the_tiled_kernel(P, case):
+    """The automatic choice on gulps that the channel-group kernel takes: every
+    sum equals the tiled kernel's (and sampled ones the oracle's), the columns
+    past the outputs stay untouched, and neither the bits past the last sample
+    nor a time slice's neighbours count."""
+    import torch
+
+    nchan, ndm, dm_end, nout = case
+    f = synth.band_freqs(nchan)
+    dms = synth.dm_list_linear(ndm, dm_end) if ndm else synth.dm_list_piecewise(dm_end)
+    plan = P.Plan(f, 64e-6, dms)
+    tiled = P.Plan(f, 64e-6, dms, kernel=P.KERNEL_TILED)
+    nsamp = nout + plan.maxdelay
+    gen = torch.Generator(device="cuda").manual_seed(nchan * 7 + nout)
+    whole = torch.randint(0, 256, (nchan, P.row_bytes(nsamp) + 48), dtype=torch.uint8, device="cuda", generator=gen)
+    part = whole[:, 16:-16]  # rows that start and end inside a longer one
+    ld = ((nout + 3) // 4 + 2) * 4
+    outs = [torch.full((len(dms), ld), -1, dtype=torch.int32, device="cuda") for _ in range(2)]
+    assert plan.uses_channel_groups(nsamp) and not tiled.uses_channel_groups(nsamp)
+    plan.execute(part, nsamp, outs[0])
+    tiled.execute(part, nsamp, outs[1])
+    assert bool((outs[0] == outs[1]).all())
+    assert bool((outs[0][:, nout:] == -1).all())
+    delays = oracle.delay_table(f, 64e-6, dms)
+    trials = sorted({0, len(dms) // 2, len(dms) - 1})
+    first = min(nout, 3000)
+    n = first + plan.maxdelay
+    packed = np.ascontiguousarray(part[:, : P.row_bytes(n)].cpu().numpy())
+    want = oracle.dedisperse(delays[trials], packed, n)[:, :first]
+    np.testing.assert_array_equal(P.as_uint32(outs[0])[trials][:, :first], want)
