@@ -4,10 +4,10 @@
 // each event for the classifier.
 //
 // Kernels (all exact integer arithmetic up to the S/N division):
-//  * dd_median_kernel   every lane keeps a histogram of the sliding window
-//                    [t-half, t+half) of its own row segment in shared memory
-//                    and walks the lower median as the window moves; writes
-//                    y = x - median and adds sum(y^2) to the row total (int64).
+//  * dd_median_kernel   every warp follows the lower median of the sliding window
+//                    [t-half, t+half) of its own row segment, 32 outputs at a
+//                    time; writes y = x - median and adds sum(y^2) to the row
+//                    total (int64).
 //  * dd_xprefix_kernel, dd_mean_apply_kernel  the paper's running mean instead
 //                    (an option): row prefix sums, then x minus the window mean
 //                    rounded half up.
@@ -30,6 +30,7 @@
 
 #include <algorithm>
 #include <new>
+#include <type_traits>
 
 #include "dd_internal.h"
 
@@ -61,423 +62,358 @@ constexpr int kPows = 11;  // possible widths 2^0 .. 2^10
 // baseline: sliding lower median by histogram walk
 // ---------------------------------------------------------------------------
 
-// Each lane walks the lower median of one row segment of h = half_window
-// outputs; lane slot g = d * nseg + s owns outputs [s*h, min(n, (s+1)*h)) of
-// row d.  The window [t-h, t+h) of any of them lies in segments s-1..s+1, so
-// the three value streams a lane needs at step t (x[t-h] leaving, x[t], and
-// x[t+h] entering the window) are, at the same offset, the values of slots
-// g-1, g and g+1.  A warp therefore stages, 32 steps at a time, the values of
-// the 34 slots g0-1 .. g0+32 with one coalesced load per slot, and each lane
-// reads its three streams from that tile.
+// A warp takes the lower medians of one row segment, 32 consecutive outputs (one
+// per lane) at a time.  It keeps m, a value near the coming medians, how many
+// values of the window [t - h, t + h) of the step's first output lie below m and
+// how many not above it, and a histogram of the values around m.  Ballots over
+// the values that enter and leave with the step's 32 moves give both counts for
+// every lane's own window; only where some lane's median is not m does the warp
+// walk along the histogram, one pair of ballots per value.
 //
-// A lane's histogram has kMedBins 32-bit counts (words interleaved across
-// lanes so each lane stays in its own bank): bin 0 counts
-// values below `base`, bins 1..kMedBins-2 the values base..base+kMedBins-3,
-// and the last bin values above; the median walks over the inner bins and the
-// lane rebuilds its histogram around the median when it reaches an edge.
-// `below` counts the window's values < m and `hm` those equal to m.
-constexpr int kMedBins = 64;
-constexpr int kMedWords = kMedBins;  // one count per word
-constexpr int kMedInner = kMedBins - 2;  // values covered by the inner bins
-constexpr int kMedStage = 34;            // staged slots per warp
-constexpr int kTileStride = 33;          // padded tile row (conflict-free)
-constexpr uint16_t kNoValue = 0xFFFFu;   // values are clipped to 3*nchan <= 65532 first
+// Bound by instruction issue.  One lane per row segment, its histogram in its
+// own bank (what this replaces), took about as many instructions, but all of an
+// output's bookkeeping was one dependency chain, 8192 outputs and counts long,
+// with too few lanes to hide it.  Measured, window 8192: the search of a
+// dedispersed gulp of 1500 x 131072 with pulses and interference 2606 us before,
+// 1875 now (the medians 1496 of 2780 before); searches of noise rows, 700 x 100003:
+// 1800 before, 999 now, 16 x 100000: 1126 and 116; 1500 x 40000 with window
+// 1000: 1009 and 889.  A bound on the counts by one warp sum before the ballots
+// settled two steps in three at window 8192 and cost more than it saved.
+constexpr int kMwWarps = 4;    // warps per block, each on its own row segment
+constexpr int kMwBins = 256;   // values base .. base + 255 are counted
+constexpr int kMwUnroll = 2;   // of the step loop (4: 2457 us instead of 2399 for a search with window 2048)
+constexpr int kMwBlocks = 8;   // blocks per SM: 64 registers a thread
+constexpr unsigned kMwGroup = 4;  // steps of 32 outputs per group of copies; two groups are on their way
 
-struct MedSlot {
-    long long xoff;  // element offset of the slot's first value in x
-    int yoff;        // element offset of its first output in y
-    int len;         // values in the slot (0: no slot)
-};
-
-__device__ __forceinline__ int med_bin(int v, int base) { return min(max(v - base + 1, 0), kMedBins - 1); }
-// Bin of the sweep: like med_bin for the inner bins and bin 0; values below
-// base - 1 land in the last bin instead of the first.
-__device__ __forceinline__ int sweep_bin(int v, int base) {
-    return (int)min((unsigned)(v - base + 1), (unsigned)(kMedBins - 1));
+__device__ __forceinline__ void copy_async4(uint32_t *dst, const uint32_t *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
 }
-__device__ __forceinline__ int hget(const uint32_t *H, int b, int lane) { return (int)H[b * 32 + lane]; }
-// A shared-memory atomic add whose result is unused: the update leaves the
-// lane's dependency chain (the walk's later reads of its own column see it).
-__device__ __forceinline__ void hadd(uint32_t *H, int b, int lane, uint32_t one) {
-    atomicAdd(&H[b * 32 + lane], one);  // one = 1 or 0xFFFFFFFF (-1)
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Median of rank r from a complete histogram: -> bin index, count below it, its count.
-__device__ __forceinline__ int med_scan(const uint32_t *H, int lane, int r, int &below, int &hm) {
-    int cum = 0;
-    for (int b = 0; b < kMedBins; ++b) {
-        const int c = hget(H, b, lane);
-        if (cum + c > r) {
-            below = cum;
-            hm = c;
-            return b;
-        }
-        cum += c;
-    }
-    below = cum;
-    hm = 0;
-    return kMedBins - 1;  // not reached for a consistent histogram
+// H[bin] += by, if the bin is one.
+__device__ __forceinline__ void mw_bump(uint32_t h_addr, int bin, uint32_t by) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.lt.u32 p, %1, %3;\n@p red.shared.add.u32 [%0], %2;\n}" ::"r"(h_addr + 4u * (uint32_t)bin),
+        "r"(bin), "r"(by), "n"(kMwBins)
+        : "memory");
 }
 
-// Warp-cooperative rebuild of the histograms of the lanes in `need` (a
-// ballot): for each such lane L all 32 lanes read L's window row[lo, hi)
-// (clipped to top) with coalesced loads and add it into L's histogram column
-// with shared atomics around L's new base; L then takes the median of rank r
-// and, when it lands on an edge bin, moves the base and the warp counts again
-// (a bounded number of times; `bad` is set if that runs out).  Called by all
-// 32 lanes together.
-__device__ __forceinline__ void med_coop_rebuild(unsigned need, const uint32_t *__restrict__ x, long long ld_x, int d, long long lo,
-                                 long long hi, int top, int r, uint32_t *H, int lane, int &base, int &m, int &below,
-                                 int &hm, bool &bad) {
-    const int maxbase = max(0, top - (kMedInner - 1));
-    while (need) {
-        const int L = __ffs(need) - 1;
-        need &= need - 1;
-        const int dL = __shfl_sync(0xffffffffu, d, L);
-        const long long loL = __shfl_sync(0xffffffffu, lo, L), hiL = __shfl_sync(0xffffffffu, hi, L);
-        const int rL = __shfl_sync(0xffffffffu, r, L);
-        int baseL = __shfl_sync(0xffffffffu, base, L);
-        const uint32_t *rowL = x + (long long)dL * ld_x;
-        for (int guard = 0; guard < 4096; ++guard) {
-            H[lane * 32 + L] = 0u;  // lane L's column: words lane and lane + 32
-            H[(lane + 32) * 32 + L] = 0u;
-            __syncwarp();
-            // eight coalesced loads in flight per round, then their counts
-            for (long long i0 = loL; i0 < hiL; i0 += 8 * 32) {
-                uint32_t v[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const long long i = i0 + 32 * u + lane;
-                    v[u] = i < hiL ? __ldg(rowL + i) : 0u;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (i0 + 32 * u + lane < hiL) atomicAdd(&H[med_bin((int)min(v[u], (uint32_t)top), baseL) * 32 + L], 1u);
-            }
-            __syncwarp();
-            int retry = 0;
-            if (lane == L) {
-                const int b = med_scan(H, lane, rL, below, hm);
-                if (b == 0 && baseL > 0) {
-                    baseL = max(0, baseL - kMedInner / 2);
-                    retry = 1;
-                } else if (b == kMedBins - 1 && baseL < maxbase) {
-                    baseL = min(maxbase, baseL + kMedInner / 2);
-                    retry = 1;
-                } else {
-                    base = baseL;
-                    m = baseL + b - 1;
-                    bad |= !(b > 0 && b < kMedBins - 1);
-                }
-            }
-            retry = __shfl_sync(0xffffffffu, retry, L);
-            baseL = __shfl_sync(0xffffffffu, baseL, L);
-            if (!retry) break;
-            if (guard == 4095 && lane == L) bad = true;
-            __syncwarp();
-        }
-    }
-}
-
-// Loads of the values of slots g0-1 .. g0+32 at offsets [bt, bt+32): one
-// chunk is in flight in registers while the warp works on the previous one.
-struct MedPrefetch {
-    uint32_t v[kMedStage];
-    unsigned long long valid;  // bit j: slot j has a value at this offset
-    bool full;                 // every slot has all 32 values (valid unused)
-};
-
-// full: bt + 32 <= the shortest of the 34 slots (warp-uniform), so no value
-// needs a bounds test.
-__device__ __forceinline__ void med_issue(const uint32_t *__restrict__ x, const MedSlot *slot, int bt, int lane,
-                                          bool full, MedPrefetch &pf) {
-    pf.full = full;
-    if (full) {
-#pragma unroll
-        for (int j = 0; j < kMedStage; ++j) pf.v[j] = __ldg(x + slot[j].xoff + bt + lane);
-        return;
-    }
-    pf.valid = 0;
-#pragma unroll
-    for (int j = 0; j < kMedStage; ++j) {
-        const MedSlot sl = slot[j];
-        const bool ok = bt + lane < sl.len;
-        pf.v[j] = ok ? __ldg(x + sl.xoff + bt + lane) : 0u;
-        pf.valid |= (unsigned long long)ok << j;
-    }
-}
-
-// Clip the prefetched values to top and store them as tile[j][lane] (NoValue
-// where a slot has no value).  Returns true when a value above top was seen.
-__device__ __forceinline__ bool med_commit(const MedPrefetch &pf, uint32_t top, uint16_t *tile, int lane) {
-    bool over = false;
-    if (pf.full) {
-#pragma unroll
-        for (int j = 0; j < kMedStage; ++j) {
-            over |= pf.v[j] > top;
-            tile[j * kTileStride + lane] = (uint16_t)min(pf.v[j], top);
-        }
-        return over;
-    }
-#pragma unroll
-    for (int j = 0; j < kMedStage; ++j) {
-        const bool ok = (pf.valid >> j) & 1ull;
-        over |= ok && pf.v[j] > top;
-        tile[j * kTileStride + lane] = ok ? (uint16_t)min(pf.v[j], top) : kNoValue;
-    }
-    return over;
-}
-
-// Shared memory of one warp: the histograms, the value tile, then (WIDE) the
-// int32 output tile or (narrow: |y| <= top <= 32767) slot g0-1's counts --
-// narrow outputs go back into the value tile as int16.
-template <bool WIDE>
-constexpr size_t med_smem_bytes() {
-    return (size_t)kMedWords * 32 * 4 + ((size_t)kMedStage * kTileStride * 2 + 3) / 4 * 4 +
-           (WIDE ? (size_t)32 * kTileStride * 4 : (size_t)kMedWords * 4);
-}
-
-template <bool WIDE>
-__global__ void __launch_bounds__(32, WIDE ? 14 : 16) dd_median_kernel(const uint32_t *__restrict__ x, long long ld_x,
-                                                                      int ndm, long long n, int h, int nbins,
-                                                                      int32_t *__restrict__ y, long long ld_y,
-                                                                      unsigned long long *__restrict__ sumsq,
-                                                                      DevState *st) {
-    extern __shared__ __align__(16) uint32_t H[];  // kMedWords x 32 lanes, then the tiles
-    uint16_t *tile = reinterpret_cast<uint16_t *>(H + kMedWords * 32);                   // [34][33] values
-    // after the value tile: [32][33] int32 outputs (WIDE) or slot g0-1's counts
-    uint32_t *after = H + kMedWords * 32 + (kMedStage * kTileStride * 2 + 3) / 4;
-    int32_t *t_y = reinterpret_cast<int32_t *>(after);
-    __shared__ MedSlot slot[kMedStage];
-    const int lane = threadIdx.x;
-    const long long nseg = (n + h - 1) / h;
-    const long long nslots = (long long)ndm * nseg;
-    const long long g0 = (long long)blockIdx.x * 32;
-    for (int j = lane; j < kMedStage; j += 32) {
-        const long long gj = g0 - 1 + j;
-        MedSlot sl{0, 0, 0};
-        if (gj >= 0 && gj < nslots) {
-            const long long dj = gj / nseg, sj = gj % nseg;
-            sl.xoff = dj * ld_x + sj * h;
-            sl.yoff = (int)(dj * ld_y + sj * h);
-            sl.len = (int)min((long long)h, n - sj * h);
-        }
-        slot[j] = sl;
-    }
+// Histogram of row[lo, hi) (values clipped to top) in kMwBins bins of 2^shift
+// values from base; returns the count of values below base.
+__device__ __forceinline__ int mw_count(const uint32_t *__restrict__ row, unsigned lo, unsigned hi, uint32_t top,
+                                        int base, int shift, uint32_t *H, int lane) {
     __syncwarp();
-    // shortest staged slot (0 where a slot is missing) and shortest output slot
-    const int minlen_all = __reduce_min_sync(0xffffffffu, (unsigned)min(slot[lane].len, lane < 2 ? slot[lane + 32].len
-                                                                                                 : slot[lane].len));
-    const int minlen_out = __reduce_min_sync(0xffffffffu, (unsigned)slot[lane + 1].len);
-    const long long g = g0 + lane;
-    const bool active = g < nslots;
-    const int d = active ? (int)(g / nseg) : 0;
-    const long long s = active ? g % nseg : 0;
-    const long long s0 = s * h;
-    const int len = slot[lane + 1].len;       // outputs of this lane (0 when inactive)
-    const bool has_prev = s > 0;              // x[t-h] exists for every t of the segment
-    const bool has_next = s + 1 < nseg;       // x[t+h] lies in the next slot of the same row
-    const uint32_t *row = x + (long long)d * ld_x;
-    const int top = nbins - 1;
-    const int maxbase = max(0, top - (kMedInner - 1));
-    const int seglen_max = __reduce_max_sync(0xffffffffu, len);  // steps of the sweep
-    // steps of the build: the previous slot (h values) and this one
-    const int build_steps = max(seglen_max, __reduce_max_sync(0xffffffffu, has_prev ? h : 0));
-    const int nb = (build_steps + 31) / 32, ns = (seglen_max + 31) / 32;
-    bool bad = false;
-
-    // first window [s0-h, s0+h) = slot g-1 + slot g.  Every lane counts its
-    // own slot and then adds lane l-1's counts (lane 0 those of slot g0-1,
-    // counted by the whole warp into Hx), so the warp shares one histogram
-    // range: around the median of the lanes' estimates, each the median of
-    // 7 values spread over the lane's window.
-    const long long lo = max(0LL, s0 - h), hi = min(n, s0 + h);
-    int wsize = (int)(hi - lo);
-    int est = -1;
-    if (active) {
-        int a[7];
 #pragma unroll
-        for (int j = 0; j < 7; ++j) a[j] = (int)min(__ldg(row + lo + (hi - 1 - lo) * j / 6), (uint32_t)top);
+    for (int k = 0; k < kMwBins / 32; ++k) H[32 * k + lane] = 0u;
+    __syncwarp();
+    int below = 0;
+    unsigned i = lo + (unsigned)lane;
+    const uint32_t h_addr = (uint32_t)__cvta_generic_to_shared(H);
+    auto one = [&](uint32_t v) {
+        const int e = (int)min(v, top) - base;
+        below -= e >> 31;
+        mw_bump(h_addr, e >> shift, 1u);
+    };
+    for (; i + 7 * 32 < hi; i += 8 * 32) {
+        uint32_t v[8];
 #pragma unroll
-        for (int p = 0; p < 7; ++p)
+        for (int u = 0; u < 8; ++u) v[u] = __ldg(row + i + 32 * u);
 #pragma unroll
-            for (int j = p & 1; j + 1 < 7; j += 2) {
-                const int lo2 = min(a[j], a[j + 1]), hi2 = max(a[j], a[j + 1]);
-                a[j] = lo2;
-                a[j + 1] = hi2;
-            }
-        est = a[3];
+        for (int u = 0; u < 8; ++u) one(v[u]);
     }
-    int base = 0;
+    for (; i < hi; i += 32) one(__ldg(row + i));
+    __syncwarp();
+    return __reduce_add_sync(0xffffffffu, below);
+}
+
+// Bin of rank r from below values under the first bin: -> false when it lies
+// outside; c0 / c1: values under the bin, and under the next.
+__device__ __forceinline__ bool mw_find(const uint32_t *H, int lane, int below, int r, int &bin, int &c0, int &c1) {
+    constexpr int kPer = kMwBins / 32;
+    uint32_t v[kPer];
+    int sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        v[k] = H[kPer * lane + k];
+        sum += (int)v[k];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    int lo = below + incl - sum;
+    const unsigned who = __ballot_sync(0xffffffffu, lo <= r && r < lo + sum);
+    if (!who) return false;
+    int b = kPer * lane, hi = lo;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+        if (hi <= r) {  // the bin is k or a later one
+            lo = hi;
+            hi += (int)v[k];
+            b = kPer * lane + k;
+        }
+    const int src = __ffs(who) - 1;
+    bin = __shfl_sync(0xffffffffu, b, src);
+    c0 = __shfl_sync(0xffffffffu, lo, src);
+    c1 = __shfl_sync(0xffffffffu, hi, src);
+    return true;
+}
+
+__global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
+    const uint32_t *__restrict__ x, long long ld_x, int ndm, unsigned n, unsigned h, unsigned seg, unsigned nseg,
+    uint32_t top, int32_t *__restrict__ y, long long ld_y, unsigned long long *__restrict__ sumsq, DevState *st) {
+    __shared__ __align__(16) uint32_t s_hist[kMwWarps][kMwBins];
+    __shared__ uint32_t s_ring[kMwWarps][2][kMwGroup][3][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t *const H = s_hist[wid];
+    const uint32_t h_addr = (uint32_t)__cvta_generic_to_shared(H);
+    const long long g = (long long)blockIdx.x * kMwWarps + wid;
+    const int d = (int)(g / nseg);
+    if (d >= ndm) return;
+    unsigned t0 = (unsigned)(g % nseg) * seg;
+    const unsigned t_end = min(n, t0 + seg);
+    const uint32_t *const row = x + (long long)d * ld_x;
+    int32_t *const yrow = y + (long long)d * ld_y;
+
+    // the first window's median is expected near that of 64 of its values
+    int guess;
     {
-        int lt = 0, le = 0;
-        for (int k = 0; k < 32; ++k) {
-            const int o = __shfl_sync(0xffffffffu, est, k);
-            lt += (o >= 0) & (o < est);
-            le += (o >= 0) & (o <= est);
-        }
-        const int want = (__popc(__ballot_sync(0xffffffffu, est >= 0)) - 1) >> 1;
-        const unsigned pick = __ballot_sync(0xffffffffu, est >= 0 && lt <= want && want < le);
-        const int mest = pick ? __shfl_sync(0xffffffffu, est, __ffs(pick) - 1) : 0;
-        base = max(0, min(maxbase, mest - kMedInner / 2));
-    }
-    const bool prev0 = __shfl_sync(0xffffffffu, has_prev, 0);  // slot g0-1 is in lane 0's row
-    uint32_t *Hx = after;  // slot g0-1's counts (WIDE: in t_y, free until the sweep)
-    Hx[lane] = 0u;
-    Hx[lane + 32] = 0u;
-    for (int w = 0; w < kMedWords; ++w) H[w * 32 + lane] = 0u;
-    int r = (wsize - 1) >> 1;
-    int m = 0, below = 0, hm = 0;
-    unsigned long long ssq = 0;
-
-    MedPrefetch pf;
-    med_issue(x, slot, 0, lane, 32 <= minlen_all, pf);
-    for (int c = 0; c < nb + ns; ++c) {
-        const bool building = c < nb;
-        const int bt = (building ? c : c - nb) * 32;
-        bad |= med_commit(pf, (uint32_t)top, tile, lane);
-        __syncwarp();
-        if (c + 1 < nb + ns) {
-            const int bn = (c + 1 < nb ? c + 1 : c + 1 - nb) * 32;
-            med_issue(x, slot, bn, lane, bn + 32 <= minlen_all, pf);
-        }
-        if (building) {
-            // ---- histograms of the lanes' slots and of slot g0-1
-            if (active) {
-#pragma unroll 4
-                for (int i = 0; i < 32; ++i) {
-                    const int vc = tile[(lane + 1) * kTileStride + i];
-                    hadd(H, med_bin(vc, base), lane, (uint32_t)(vc != kNoValue));
-                }
-            }
-            if (prev0) {
-                const int v0 = tile[lane];
-                if (v0 != kNoValue) {
-                    const int b = med_bin(v0, base);
-                    atomicAdd(&Hx[b], 1u);
-                }
-            }
-            if (c == nb - 1) {
-                // window = own slot + previous slot
-                __syncwarp();
-#pragma unroll 1
-                for (int w0 = 0; w0 < kMedWords; w0 += 16) {
-                    uint32_t nbh[16];
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) nbh[k] = lane == 0 ? Hx[w0 + k] : H[(w0 + k) * 32 + lane - 1];
-                    __syncwarp();
-                    if (has_prev) {
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) H[(w0 + k) * 32 + lane] += nbh[k];
-                    }
-                    __syncwarp();
-                }
-                bool need = false;
-                if (active) {
-                    const int b = med_scan(H, lane, r, below, hm);
-                    m = base + b - 1;
-                    if (b == 0 || b == kMedBins - 1) {
-                        base = max(0, min(maxbase, (b == 0 ? base - kMedInner : base + kMedInner)));
-                        need = true;
-                    }
-                }
-                __syncwarp();
-                const unsigned nmask = __ballot_sync(0xffffffffu, need);
-                if (nmask) {
-                    if (lane == 0) atomicAdd(&st->nrebuild, (unsigned long long)__popc(nmask));
-                    med_coop_rebuild(nmask, x, ld_x, d, lo, hi, top, r, H, lane, base, m, below, hm, bad);
-                }
-            }
-            __syncwarp();
-            continue;
-        }
-        // ---- sweep: output y[t] = x[t] - m, then move the window to t+1 (also
-        // after a segment's last output: harmless, the state is dropped)
-        {
-            const int nst = active ? min(32, len - bt) : 0;
-            const int nst_w = __reduce_max_sync(0xffffffffu, nst);  // the warp steps together
-            int32_t yprev = 0;
-#pragma unroll 2
-            for (int i = 0; i < nst_w; ++i) {
-                bool need = false;
-                if (i < nst) {
-                const int vc = tile[(lane + 1) * kTileStride + i];
-                const int32_t yv = vc - m;
-                if (WIDE) {
-                    t_y[lane * kTileStride + i] = yv;
-                } else {
-                    // column i-1 of the tile was read by every lane before the
-                    // previous step's ballot: it takes that step's output
-                    if (i > 0) tile[(lane + 1) * kTileStride + i - 1] = (uint16_t)yprev;
-                    yprev = yv;
-                }
-                ssq += (uint32_t)yv * (uint32_t)yv;  // |y| <= 65532: the square fits 32 bits
-                const int vo = has_prev ? tile[lane * kTileStride + i] : kNoValue;
-                const int vi = has_next ? tile[(lane + 2) * kTileStride + i] : kNoValue;
-                // Branch-free.  The sweep reads only the inner bins, so values
-                // outside them (and kNoValue, which lies above every median)
-                // all go to the last bin, whose count it never reads.
-                hadd(H, sweep_bin(vo, base), lane, 0xFFFFFFFFu);
-                hadd(H, sweep_bin(vi, base), lane, 1u);
-                wsize += (vi != kNoValue) - (vo != kNoValue);
-                below += (vi < m) - (vo < m);
-                hm += (vi == m) - (vo == m);
-                r = (wsize - 1) >> 1;
-                if (below > r || below + hm <= r) {  // the median moves (rarely)
-                    bool rebuild = false;
-                    while (below > r) {
-                        if (m <= base) {
-                            rebuild = true;
-                            break;
-                        }
-                        --m;
-                        hm = hget(H, m - base + 1, lane);
-                        below -= hm;
-                    }
-                    while (!rebuild && below + hm <= r) {
-                        if (m >= base + kMedInner - 1) {
-                            rebuild = true;
-                            break;
-                        }
-                        below += hm;
-                        ++m;
-                        hm = hget(H, m - base + 1, lane);
-                    }
-                    if (rebuild) {
-                        base = max(0, min(maxbase, m - kMedInner / 2));
-                        need = true;
-                    }
-                }
-                }
-                const unsigned nmask = __ballot_sync(0xffffffffu, need);
-                if (nmask) {
-                    if (lane == 0) atomicAdd(&st->nrebuild, (unsigned long long)__popc(nmask));
-                    const long long t1 = s0 + bt + i + 1;
-                    med_coop_rebuild(nmask, x, ld_x, d, max(0LL, t1 - h), min(n, t1 + h), top, r, H, lane, base, m,
-                                     below, hm, bad);
-                }
-            }
-            if (!WIDE && nst > 0) tile[(lane + 1) * kTileStride + nst - 1] = (uint16_t)yprev;
-        }
-        __syncwarp();
-        // coalesced write-back of the 32 outputs of every lane
-        auto yval = [&](int j) -> int32_t {
-            return WIDE ? t_y[j * kTileStride + lane] : (int32_t)(int16_t)tile[(j + 1) * kTileStride + lane];
-        };
-        if (bt + 32 <= minlen_out) {
+        const unsigned lo = t0 - min(t0, h);
+        const unsigned long long span = min(n, t0 + h) - 1 - lo;
+        const uint32_t v0 = min(__ldg(row + lo + (unsigned)(span * (unsigned)lane / 63u)), top);
+        const uint32_t v1 = min(__ldg(row + lo + (unsigned)(span * (unsigned)(lane + 32) / 63u)), top);
+        int less = 0, same = 0;
 #pragma unroll 8
-            for (int j = 0; j < 32; ++j) y[slot[j + 1].yoff + bt + lane] = yval(j);
-        } else {
-#pragma unroll 4
-            for (int j = 0; j < 32; ++j) {
-                const MedSlot sl = slot[j + 1];
-                if (bt + lane < sl.len) y[sl.yoff + bt + lane] = yval(j);
-            }
+        for (int k = 0; k < 32; ++k) {
+            const uint32_t a = __shfl_sync(0xffffffffu, v0, k), b = __shfl_sync(0xffffffffu, v1, k);
+            less += (a < v0) + (b < v0);
+            same += (a == v0) + (b == v0);
         }
-        __syncwarp();
+        // the value of the first half whose rank comes nearest the middle
+        const int off = max(0, max(less - 31, 32 - (less + same)));
+        const int best = (int)__reduce_min_sync(0xffffffffu, (unsigned)off);
+        guess = (int)__shfl_sync(0xffffffffu, v0, __ffs(__ballot_sync(0xffffffffu, off == best)) - 1);
     }
-    if (active) atomicAdd(sumsq + d, ssq);
-    if (bad) atomicOr(&st->err, 1u);
+    unsigned long long ssq = 0;
+    uint32_t most = 0;
+    unsigned builds = 0;
+    int singles = 0;  // outputs to take one by one
+
+    // One go: the histogram from the window of t0, then steps of 32 outputs
+    // until the segment ends or a median lies beyond the bins; the next go has
+    // its bins around the present median.  Where that one fails at once, the 32
+    // medians lie too far apart for any bins and 32 goes take one output each.
+#pragma unroll 1
+    while (t0 < t_end) {
+        const unsigned start = t0, stop = singles ? t0 + 1 : t_end;
+        // the values of kMwGroup steps: x[t], x[t + h], x[t - h] of the lane's
+        // outputs (each lane reads only what it copied itself)
+        auto inside = [&](unsigned t) {  // every output has its whole window in the row, and is of this go
+            return t >= h && t + 32 * kMwGroup + h <= n && t + 32 * kMwGroup <= stop;
+        };
+        auto fetch = [&](unsigned tg, int half) {
+            uint32_t *to = &s_ring[wid][half][0][0][lane];
+            const unsigned t = tg + (unsigned)lane;
+            const uint32_t *p = row + t;
+            if (inside(tg)) {
+#pragma unroll
+                for (int j = 0; j < (int)kMwGroup; ++j) {
+                    copy_async4(to + 96 * j, p + 32 * j);
+                    copy_async4(to + 96 * j + 32, p + h + 32 * j);
+                    copy_async4(to + 96 * j + 64, p - h + 32 * j);
+                }
+            } else {
+#pragma unroll 1
+                for (unsigned j = 0; j < kMwGroup; ++j)
+                    if (t + 32 * j < stop) {
+                        copy_async4(to + 96 * j, p + 32 * j);
+                        if (t + 32 * j + h < n) copy_async4(to + 96 * j + 32, p + h + 32 * j);
+                        if (t + 32 * j >= h) copy_async4(to + 96 * j + 64, row + (t + 32 * j - h));
+                    }
+            }
+            copy_commit();
+        };
+        fetch(t0, 0);
+        fetch(t0 + 32 * kMwGroup, 1);
+
+        // state: base = value of the first bin, m = a value near the coming
+        // medians, b0 / b1 = values of the window below m / not above it
+        int base = max(0, guess - kMwBins / 2), m, b0, b1;
+        {
+            const unsigned lo = t0 - min(t0, h), hi = min(n, t0 + h);
+            const int rank = (int)(hi - lo - 1) >> 1;
+            // around the guess; where the median is not there, it is narrowed
+            // down from all values (65532 at most), 32 bins at a time
+            int shift = 0, at = 0, bin;
+            bool narrowing = false;
+#pragma unroll 1
+            for (;;) {
+                const int below = mw_count(row, lo, hi, top, base, shift, H, lane);
+                const bool found = mw_find(H, lane, below, rank, bin, b0, b1);
+                if (found && shift == 0) break;
+                if (!narrowing) {
+                    narrowing = true;
+                    shift = 11;
+                } else {
+                    at += bin << shift;
+                    shift = shift == 1 ? 0 : shift - 5;
+                }
+                base = shift ? at : max(0, at - kMwBins / 2);
+            }
+            m = base + bin;
+            ++builds;
+        }
+
+        // 32 outputs; FULL: of an inside group.  false: a median lies beyond the bins.
+        auto step = [&](auto is_full, unsigned ts, const uint32_t *from) {
+            constexpr bool FULL = decltype(is_full)::value;
+            const unsigned t = ts + (unsigned)lane;
+            const bool act = FULL || t < stop;
+            const uint32_t nc = from[0];
+            int vi = (int)min(from[32], top), vo = (int)min(from[64], top);
+            if (!FULL) {  // past the row: above every median
+                if (t + h >= n) vi = (int)top + 1;
+                if (t < h) vo = (int)top + 1;
+            }
+            // values that enter and leave with the 32 moves: below m, not above it
+            const unsigned lt = (1u << lane) - 1u;
+            const unsigned i0 = __ballot_sync(0xffffffffu, vi < m), o0 = __ballot_sync(0xffffffffu, vo < m);
+            const unsigned i1 = __ballot_sync(0xffffffffu, vi <= m), o1 = __ballot_sync(0xffffffffu, vo <= m);
+            // the median's rank (past the row of no use)
+            const int r = FULL ? (int)h - 1 : ((int)(min(n, t + h) - (t - min(t, h))) - 1) >> 1;
+            // m is the median of all 32?  (Of a window of 8192 noise values nine
+            // times in ten.)
+            const int c0 = b0 + __popc(i0 & lt) - __popc(o0 & lt), c1 = b1 + __popc(i1 & lt) - __popc(o1 & lt);
+            int med = m, to = m;
+            if (__any_sync(0xffffffffu, act && (c0 > r || c1 <= r))) {
+                // values of the window of output t that are below v: (those of
+                // the window of ts) + (entered since) - (left since)
+                auto since = [&](int v) {
+                    return __popc(__ballot_sync(0xffffffffu, vi < v) & lt) -
+                           __popc(__ballot_sync(0xffffffffu, vo < v) & lt);
+                };
+                __syncwarp();
+                int v = m + 1, b = b1, c = c1;
+#pragma unroll 1
+                while (__any_sync(0xffffffffu, act && c <= r)) {
+                    if (v - base >= kMwBins) return false;
+                    if (c <= r) med = v;
+                    b += (int)H[v - base];
+                    ++v;
+                    c = b + since(v);
+                }
+                v = m, b = b0, c = c0;
+#pragma unroll 1
+                while (__any_sync(0xffffffffu, act && c > r)) {
+                    --v;
+                    if (v < base) return false;
+                    if (c > r) med = v;
+                    b -= (int)H[v - base];
+                    c = b + since(v);
+                }
+                to = __shfl_sync(0xffffffffu, med, 31);
+                __syncwarp();
+            }
+            if (act) {
+                most = max(most, nc);
+                const int yv = (int)min(nc, top) - med;
+                yrow[t] = yv;
+                ssq += (unsigned long long)((long long)yv * yv);
+            }
+            // the window moves on by 32
+            mw_bump(h_addr, vi - base, 1u);
+            mw_bump(h_addr, vo - base, 0xffffffffu);
+            b0 += __popc(i0) - __popc(o0);
+            b1 += __popc(i1) - __popc(o1);
+            if (m != to) {
+                __syncwarp();
+                while (m < to) {
+                    b0 = b1;
+                    ++m;
+                    b1 += (int)H[m - base];
+                }
+                while (m > to) {
+                    b1 = b0;
+                    --m;
+                    b0 -= (int)H[m - base];
+                }
+                __syncwarp();
+            }
+            return true;
+        };
+        int half = 0;
+        bool far = false;
+#pragma unroll 1
+        while (t0 < stop) {
+            copy_wait<1>();
+            const uint32_t *from = &s_ring[wid][half][0][0][lane];
+            if (inside(t0)) {
+#pragma unroll kMwUnroll
+                for (unsigned j = 0; j < kMwGroup; ++j) {
+                    far = !step(std::true_type(), t0 + 32 * j, from + 96 * j);
+                    if (far) {
+                        t0 += 32 * j;
+                        break;
+                    }
+                }
+            } else {
+#pragma unroll 1
+                for (unsigned j = 0; j < kMwGroup && t0 + 32 * j < stop; ++j) {
+                    far = !step(std::false_type(), t0 + 32 * j, from + 96 * j);
+                    if (far) {
+                        t0 += 32 * j;
+                        break;
+                    }
+                }
+            }
+            if (far) break;
+            fetch(t0 + 64 * kMwGroup, half);
+            half ^= 1;
+            t0 += 32 * kMwGroup;
+        }
+        copy_wait<0>();
+        __syncwarp();
+        guess = m;
+        if (singles) {
+            --singles;
+            t0 = start + 1;
+        } else if (far && t0 == start) {
+            singles = 32;
+        }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) ssq += __shfl_down_sync(0xffffffffu, ssq, o);
+    if (lane == 0) {
+        atomicAdd(sumsq + d, ssq);
+        if (builds > 1) atomicAdd(&st->nrebuild, (unsigned long long)(builds - 1));
+    }
+    if (most > top) atomicOr(&st->err, 1u);
+}
+
+// Outputs per segment.  A segment counts its first window (2 h values, 0.15 of a
+// step per 32 values), so long ones are cheaper, but the warps have to fill the
+// device (32 per SM, half a segment's time lost at the end).  Measured for whole
+// searches of 1500 x 131072, h 4096, segments of 2048 / 4096 / 8192 (chosen):
+// 2718 / 2576 / 2504 us (40 warps per SM then); 16 x 100000, segments of 256 (chosen) / 4096: 142 / 167.
+unsigned median_segment(int ndm, long long n, long long h) {
+    unsigned best = 0;
+    double least = 0;
+    for (unsigned seg = 256; seg <= 32768; seg *= 2) {
+        const double warps = (double)ndm * (double)((n + seg - 1) / seg);
+        const double cost = (std::max(warps / (152.0 * kMwBlocks * kMwWarps), 1.0) + 0.5) * (0.3 * (double)h + seg);
+        if (!best || cost < least) {
+            best = seg;
+            least = cost;
+        }
+    }
+    return best;
 }
 
 // ---------------------------------------------------------------------------
@@ -1582,14 +1518,11 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
             d_x, (long long)ld_x, (long long)n, h, (uint32_t)(s->nbins - 1), s->pre, s->tile_off, s->tile_sum,
             s->ntiles, s->y, s->ld_y, s->sumsq);
     } else {
-        const long long nsegs = (long long)ndm * (((long long)n + h - 1) / h);
-        const unsigned grid = (unsigned)((nsegs + 31) / 32);
-        if (s->nbins - 1 > 32767)  // outputs need more than 16 bits
-            dd_median_kernel<true><<<grid, 32, med_smem_bytes<true>(), st>>>(
-                d_x, (long long)ld_x, ndm, (long long)n, (int)h, s->nbins, s->y, s->ld_y, s->sumsq, s->st);
-        else
-            dd_median_kernel<false><<<grid, 32, med_smem_bytes<false>(), st>>>(
-                d_x, (long long)ld_x, ndm, (long long)n, (int)h, s->nbins, s->y, s->ld_y, s->sumsq, s->st);
+        const unsigned seg = median_segment(ndm, (long long)n, h);
+        const unsigned nseg = (unsigned)(((long long)n + seg - 1) / seg);
+        dd_median_kernel<<<(unsigned)(((long long)ndm * nseg + kMwWarps - 1) / kMwWarps), 32 * kMwWarps, 0, st>>>(
+            d_x, (long long)ld_x, ndm, (unsigned)n, (unsigned)h, seg, nseg, (uint32_t)(s->nbins - 1), s->y, s->ld_y,
+            s->sumsq, s->st);
     }
     DD_CUDA_TRY(cudaGetLastError());
     // matched filter + sigma cut

@@ -142,6 +142,37 @@ def test_baseline_median_edge_shapes(P, n, half):
     s.close()
 
 
+@pytest.mark.parametrize("ndm,n,half", [(3, 255, 64), (3, 256, 64), (3, 257, 128), (5, 383, 127), (5, 385, 129),
+                                        (2, 1024, 256), (40, 2177, 513), (700, 4609, 1024), (1600, 4230, 96)])
+def test_baseline_median_segment_edges(P, ndm, n, half):
+    """Lengths around a warp's segments and groups of steps, windows around a
+    group's, rows at odd offsets, noise with stuck and jumping stretches: y
+    equals the oracle's; a value above the largest possible sum is clipped to
+    it and flagged."""
+    import torch
+
+    rng = np.random.default_rng(ndm * n + half)
+    x = (700 + 20 * rng.standard_normal((ndm, n))).round().astype(np.uint32)
+    x[:, n // 3:n // 2] += rng.integers(0, 400, (ndm, 1)).astype(np.uint32)
+    x[1] = np.where((np.arange(n) // 45) % 2 == 0, 3, 3000)
+    x[ndm - 1, n // 2:] = 768
+    wide = np.full((ndm, n + 5), 0xFFFFFFFF, dtype=np.uint32)
+    for flagged in (False, True):
+        if flagged:
+            x[0, n // 2] = 0xFFFFFFFF
+            x[ndm // 2, n - 1] = 3073
+        wide[:, 3:n + 3] = x
+        d_x = torch.from_numpy(wide.view(np.int32)).cuda()[:, 3:n + 3]
+        s = P.Search(ndm, n, nchan=1024, half_window=half, widths=(1,), thresh=50.0, max_cands=64)
+        s.run(d_x, ndm, n)
+        assert s.result()["flags"] & 1 == int(flagged)
+        y, ss, _, _ = s.buffers()
+        y_or = oracle.baseline(np.minimum(x, 3072), half)
+        np.testing.assert_array_equal(y.cpu().numpy(), y_or)
+        np.testing.assert_array_equal(ss.cpu().numpy(), [oracle.sumsq(r) for r in y_or])
+        s.close()
+
+
 def test_search_constant_rows_and_empty_result(P):
     import torch
 
