@@ -669,8 +669,13 @@ __global__ void dd_thresh_kernel(const unsigned long long *__restrict__ sumsq, l
 // threads' totals), and tests its cells four at a time: a lane owns four
 // consecutive cells, reads P at the cells and at the cells + w with 16-byte
 // loads, and compares each boxcar sum S_w = P[t+w] - P[t] with the smallest
-// sum reaching the threshold.  Hot cells get their best S/N and width; the
-// four-cell nibbles of eight lanes form one word of the row's hot bitmask.
+// sum reaching the threshold.  That exact test runs only in warps where a bound
+// for a lane's four cells says that one may be hot (mf_may_be_hot4), which takes
+// a third of its operations and a quarter of its words: a gulp of 1500 x 131072
+// with 15 % hot cells 572 us before the bound, 462 now (1.65 GB to read and
+// write, 250 us; the rest are the hot cells' S/N over 11 widths).  Hot cells get
+// their best S/N and width; the four-cell nibbles of eight lanes form one word
+// of the row's hot bitmask.
 constexpr int kMfSpan = kMfTile + 1024;       // samples loaded per tile (tile + widest boxcar)
 constexpr int kMfSeg = kMfSpan / kMfThreads;  // samples per thread in the scan
 static_assert(kMfSeg % 4 == 0 && kMfSeg * kMfThreads == kMfSpan, "scan segments of whole int4s");
@@ -735,6 +740,31 @@ __device__ __forceinline__ void mf_test4(const int32_t *P, int t, int nrem, unsi
     }
 }
 
+// false: none of the four cells t..t+3 is hot (true: one may be).  Widths 1 and
+// 2 cell by cell, from the registers; for a wider one the four sums are at most
+// the largest of P[t+w..t+w+3] (p4[w / 4]) less the smallest of P[t..t+3]: one
+// operation and one word for four cells, and noise hardly ever reaches T with
+// it (at w = 4 the bound covers 7 samples, T is 6 sigma of 4).
+template <bool ALLW>
+__device__ __forceinline__ bool mf_may_be_hot4(const int32_t *p4, unsigned wmask, const int32_t (&tm)[kPows], int4 p0,
+                                               int2 p45) {
+    int32_t a = -1, wide = -0x7fffffff - 1;
+    if (ALLW || (wmask & 1u)) {
+        a &= (p0.y - p0.x - tm[0]) & (p0.z - p0.y - tm[0]);
+        a &= (p0.w - p0.z - tm[0]) & (p45.x - p0.w - tm[0]);
+    }
+    if (ALLW || (wmask & 2u)) {
+        a &= (p0.z - p0.x - tm[1]) & (p0.w - p0.y - tm[1]);
+        a &= (p45.x - p0.z - tm[1]) & (p45.y - p0.w - tm[1]);
+    }
+#pragma unroll
+    for (int j = 2; j < kPows; ++j) {
+        if (!ALLW && !((wmask >> j) & 1u)) continue;
+        wide = max(wide, p4[(1 << j) / 4] - tm[j]);
+    }
+    return a >= 0 || wide >= min(min(p0.x, p0.y), min(p0.z, p0.w));
+}
+
 template <bool ALLW>
 __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__restrict__ y, long long ld_y, long long n,
                                                         const unsigned long long *__restrict__ sumsq,
@@ -745,6 +775,7 @@ __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__rest
                                                         int ntiles, const float *__restrict__ den_all,
                                                         const int32_t *__restrict__ tmin_all, int full_map) {
     __shared__ __align__(16) int32_t P[kMfSpan];  // exclusive prefix of the tile's samples
+    __shared__ int32_t P4[kMfSpan / 4];           // largest of each four
     // per-width values indexed by log2(width)
     __shared__ float s_den[kPows];
     __shared__ float s_rcp[kPows];  // 1/den rounded to nearest
@@ -818,8 +849,11 @@ __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__rest
     for (int w2 = 0; w2 < warp; ++w2) off += s_warp[w2];
 #pragma unroll
     for (int q = 0; q < kMfSeg / 4; ++q)
-        *reinterpret_cast<int4 *>(P + tid * kMfSeg + 4 * q) =
-            make_int4(v[q].x + off, v[q].y + off, v[q].z + off, v[q].w + off);
+    {
+        const int4 w = make_int4(v[q].x + off, v[q].y + off, v[q].z + off, v[q].w + off);
+        *reinterpret_cast<int4 *>(P + tid * kMfSeg + 4 * q) = w;
+        P4[tid * (kMfSeg / 4) + q] = max(max(w.x, w.y), max(w.z, w.w));
+    }
     __syncthreads();
 
     int32_t tm[kPows];
@@ -836,12 +870,24 @@ __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__rest
         const int t = warp * (kMfTile / (kMfThreads / 32)) + j * 128 + lane * 4;  // first of this lane's 4 cells
         const int4 p0 = *reinterpret_cast<const int4 *>(P + t);
         const int2 p45 = *reinterpret_cast<const int2 *>(P + t + 4);
+        if (t + 3 < nrem && ((cbase + t) & 3) == 0) {
+            *reinterpret_cast<int4 *>(pre + cbase + t) = p0;  // pre comes from cudaMalloc: 16-byte aligned rows of 4
+        } else {
+            const int32_t pc[4] = {p0.x, p0.y, p0.z, p0.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (t + i < nrem) pre[cbase + t + i] = pc[i];
+        }
+        const long long tw = t0 + t;  // first cell of the word for lanes 0, 8, 16, 24
+        if (!full_map && !__any_sync(0xffffffffu, mf_may_be_hot4<ALLW>(P4 + t / 4, wmask, tm, p0, p45))) {
+            if ((lane & 7) == 0 && tw < n) hotbits[(long long)d * nwr + tw / 32] = 0u;
+            continue;
+        }
         bool h0 = false, h1 = false, h2 = false, h3 = false;
         if (inside)
             mf_test4<true, ALLW>(P, t, nrem, wmask, tm, p0, p45, h0, h1, h2, h3);
         else
             mf_test4<false, ALLW>(P, t, nrem, wmask, tm, p0, p45, h0, h1, h2, h3);
-        const int32_t pc[4] = {p0.x, p0.y, p0.z, p0.w};
         const bool hc[4] = {h0, h1, h2, h3};
         uint32_t nib = 0, live = 0;
 #pragma unroll
@@ -849,13 +895,6 @@ __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__rest
             const bool lv = t + i < nrem;
             live |= (uint32_t)lv << i;
             nib |= (uint32_t)(lv && hc[i]) << i;
-        }
-        if (live == 0xFu && ((cbase + t) & 3) == 0) {
-            *reinterpret_cast<int4 *>(pre + cbase + t) = p0;  // pre comes from cudaMalloc: 16-byte aligned rows of 4
-        } else {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if ((live >> i) & 1u) pre[cbase + t + i] = pc[i];
         }
         // cells whose S/N is computed (hot ones, or all with full_map) join
         // the tile's list, warp by warp in cell order
@@ -880,7 +919,6 @@ __global__ void __launch_bounds__(kMfThreads) dd_mf_kernel(const int32_t *__rest
         word |= __shfl_xor_sync(0xffffffffu, word, 1);
         word |= __shfl_xor_sync(0xffffffffu, word, 2);
         word |= __shfl_xor_sync(0xffffffffu, word, 4);
-        const long long tw = t0 + t;  // first cell of the word for lanes 0, 8, 16, 24
         if ((lane & 7) == 0 && tw < n) {
             hotbits[(long long)d * nwr + tw / 32] = word;
             if (word) atomicAdd(&s_nhot, (unsigned)__popc(word));

@@ -399,3 +399,36 @@ def test_mean_baseline_ragged_rows(P):
         y, ss, _, _ = s.buffers()
         np.testing.assert_array_equal(y.cpu().numpy(), oracle.baseline_mean(x, half))
         s.close()
+
+
+@pytest.mark.parametrize("widths", [WIDTHS, (1,), (2, 1024), (4, 8, 64), (1, 4)])
+@pytest.mark.parametrize("n", [4097, 6003, 8192 + 1024])
+def test_hot_cells_at_the_threshold(P, n, widths):
+    """Cells whose S/N lies just at, above and below the cut, alone in quiet
+    rows, at every position of a group of four and at tile and row ends: the
+    hot cells are those whose best S/N in the oracle's map reaches it."""
+    import torch
+
+    rng = np.random.default_rng(n + len(widths))
+    ndm, thresh = 24, 6.0
+    x = 1000 + rng.integers(-1, 2, (ndm, n))
+    for d in range(1, ndm):
+        w = widths[d % len(widths)]
+        sigma = np.sqrt(2.0 / 3.0)
+        t0 = [0, 4096 - w, 4096, n - w, n // 2][d % 5] + d % 4
+        t0 = max(0, min(t0, n - w))
+        lift = thresh * sigma * np.sqrt(w) / w
+        x[d, t0:t0 + w] += int(round(lift)) + d % 3 - 1
+    x = x.astype(np.uint32)
+    s = P.Search(ndm, n, nchan=1024, half_window=700, widths=widths, thresh=thresh, max_cands=4096)
+    s.run(torch.from_numpy(x.view(np.int32)).cuda(), ndm, n)
+    hot = s.result()["nhot"]
+    y_or = oracle.baseline(x, 700)
+    best, _ = oracle.best_snr(y_or, widths)
+    full = P.Search(ndm, n, nchan=1024, half_window=700, widths=widths, thresh=thresh, max_cands=4096, full_map=True)
+    full.run(torch.from_numpy(x.view(np.int32)).cuda(), ndm, n)
+    fb = full.buffers()[2].cpu().numpy()
+    np.testing.assert_array_equal(fb, best)
+    assert hot == int((best >= np.float32(thresh)).sum()) and full.result()["nhot"] == hot
+    a, b = s.candidates(), full.candidates()
+    np.testing.assert_array_equal(a, b)
