@@ -80,6 +80,7 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     bool gsum_off = false;
     if (cache_lookup(p, nsamp_in, &cached, &gsum_off) && ensure_shape_table(p, cached) == DD_OK) {
         p->shape = cached;
+        p->narrow_sms = 0;
         p->gs.off = gsum_off;
         if (best_ms) *best_ms = 0.0f;
         return DD_OK;
@@ -141,6 +142,7 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     if (out) cudaFree(out);
     if (st != DD_OK) return st;
     p->shape = best_shape;
+    p->narrow_sms = 0;  // the tuned shape, for every gulp
     // keep only the chosen shape's tables, unless a batch still points at some
     // of them (they are then freed with the plan)
     for (auto it = p->tables.begin(); it != p->tables.end() && p->live_batches == 0;) {

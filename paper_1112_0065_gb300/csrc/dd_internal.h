@@ -33,6 +33,10 @@ struct TiledShape {
     int chan_chunk = 64;    // channels per shared-memory stage (one CSA group)
 };
 
+// Shape for gulps of so few tiles that an SM gets one at most: half the work of
+// the default one in a tile.
+constexpr TiledShape kNarrowShape{1, 3, 64};
+
 // Map key of a shape's tables in Plan::tables.
 inline int shape_key(const TiledShape &s) { return s.chan_chunk * 10000 + s.dms_per_warp * 100 + s.words_per_lane; }
 
@@ -68,6 +72,7 @@ struct Plan {
     int device = 0;
     int kernel = DD_KERNEL_AUTO;
     TiledShape shape;
+    int narrow_sms = 0;                 // SMs when short gulps take kNarrowShape, else 0
     std::map<int, ShapeTable> tables;   // keyed by shape_key()
     GsumTable gs;                       // channel-group tables (automatic plans only)
     int live_batches = 0;               // batches whose descriptors point at these tables

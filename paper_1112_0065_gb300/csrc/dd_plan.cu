@@ -103,7 +103,15 @@ static dd_status run(const Plan *p, const uint8_t *d_in, size_t ld_in_bytes, siz
     if (p->kernel == DD_KERNEL_SIMPLE) return launch_simple(p, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
     if (takes_gsum(p, nsamp_in))
         return launch_gsum(p, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
-    return launch_tiled(p, p->shape, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
+    // A tile of the default shape takes 1.4 to 1.6 times as long as one of the
+    // narrow shape with an SM to itself, which loses as soon as two have to share
+    // one: default / narrow, in us, 64 channels x 64 trials x 6208 outputs 14.3 /
+    // 10.2, 1024 x 64 x 20000 63.5 / 40.9, 1024 x 64 x 40000 (216 narrow tiles)
+    // 63.5 / 67.6.
+    const long long nout = (long long)nsamp_in - p->maxdelay;
+    const long long narrow_tiles = (nout + 1535) / 1536 * ((p->ndm + 7) / 8);
+    const TiledShape &shape = narrow_tiles <= p->narrow_sms ? kNarrowShape : p->shape;
+    return launch_tiled(p, shape, d_in, ld_in_bytes, nsamp_in, d_out, ld_out, stream);
 }
 
 }  // namespace dd
@@ -202,8 +210,16 @@ dd_status dd_plan_create(dd_plan **out, int nchan, const double *freqs_mhz, doub
             p->kernel = DD_KERNEL_SIMPLE;  // delay spread beyond the tiled kernel's shared memory
         }
     }
-    // the channel-group kernel for automatic plans (a given shape asks for the tiled kernel)
-    if (p->kernel == DD_KERNEL_AUTO && !(o.dms_per_block || o.words_per_thread || o.chan_chunk)) build_gsum(p);
+    // the channel-group kernel and the narrow shape for automatic plans (a given
+    // shape asks for that one); with more than 304 trials only gulps of 6000
+    // outputs and fewer would be narrow, not worth the tables
+    if (p->kernel == DD_KERNEL_AUTO && !(o.dms_per_block || o.words_per_thread || o.chan_chunk)) {
+        build_gsum(p);
+        if (ndm <= 304 && ensure_shape_table(p, kNarrowShape) == DD_OK &&
+            cudaDeviceGetAttribute(&p->narrow_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess)
+            p->narrow_sms = 0;
+        cudaGetLastError();  // without memory for the tables the default shape serves
+    }
     *out = reinterpret_cast<dd_plan *>(p);
     return DD_OK;
 }

@@ -418,3 +418,21 @@ def test_channel_groups_equal_the_tiled_kernel(P, case):
     packed = np.ascontiguousarray(part[:, : P.row_bytes(n)].cpu().numpy())
     want = oracle.dedisperse(delays[trials], packed, n)[:, :first]
     np.testing.assert_array_equal(P.as_uint32(outs[0])[trials][:, :first], want)
+
+
+@pytest.mark.parametrize("nchan,ndm,nout", [(64, 64, 19 * 1536), (64, 64, 19 * 1536 + 1), (1, 8, 1), (65, 61, 1537),
+                                            (130, 9, 76 * 1536), (100, 304, 6144), (100, 305, 6144), (2050, 16, 3000)])
+def test_short_gulps_on_the_narrow_shape(P, nchan, ndm, nout):
+    """Gulps at the lines where an automatic plan leaves its default tile for
+    the one of half the trials (152 SMs), with one channel, partial stages and
+    partial blocks of trials: the oracle's sums."""
+    f = synth.band_freqs(nchan)
+    dms = synth.dm_list_linear(ndm, 90.0)
+    plan = P.Plan(f, 64e-6, dms)
+    nsamp = nout + plan.maxdelay
+    packed, _ = synth.make_gulp(nchan + nout, nchan, nsamp)
+    want = oracle.dedisperse(oracle.delay_table(f, 64e-6, dms), packed, nsamp)
+    np.testing.assert_array_equal(_run(P, plan, packed, nsamp), want)
+    if nchan < 2048:  # tuned, the plan runs its tuned shape for every gulp
+        plan.autotune(nsamp)
+        np.testing.assert_array_equal(_run(P, plan, packed, nsamp), want)
