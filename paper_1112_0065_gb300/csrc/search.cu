@@ -16,7 +16,7 @@
 //                    decides with integer thresholds whether some width reaches
 //                    the S/N cut; hot cells get their best S/N and width and a
 //                    bit in the row's hot bitmask.
-//  * runs/vunion/compress/ids/group_reduce kernels: 4-connected groups in
+//  * runs/vunion/compress/group_reduce kernels: 4-connected groups in
 //                    (DM, time) from runs of hot cells along time joined across
 //                    rows by union-find (roots = smallest run start, so the
 //                    result is deterministic); one record per group at its best
@@ -1046,15 +1046,6 @@ __global__ void __launch_bounds__(512) dd_runs_kernel(const uint32_t *__restrict
     }
 }
 
-__device__ __forceinline__ int32_t find_root(const int32_t *L, int32_t x) {
-    int32_t p = __ldcg(L + x);
-    while (p != x) {
-        x = p;
-        p = __ldcg(L + x);
-    }
-    return x;
-}
-
 // find with path halving: each visited node is pointed at its grandparent.
 // Labels only ever move to smaller indices of the same group, so a plain
 // store of an ancestor is safe against concurrent links (a linker that loses
@@ -1112,44 +1103,43 @@ __global__ void dd_vunion_kernel(const uint32_t *__restrict__ hotbits, int nwr, 
     }
 }
 
-// Every run start points straight at its root.
-__global__ void dd_compress_kernel(const uint32_t *__restrict__ hotbits, int nwr, int ndm, long long n, int32_t *L) {
+// Every run start points straight at its root; roots get compact ids, stored in
+// place as -(id + 2), where a search that meets one ends (two passes over the
+// bitmask, one for the roots and one for the ids, took 56 us for 1500 x 131072,
+// this one 31).
+__global__ void dd_compress_kernel(const uint32_t *__restrict__ hotbits, int nwr, int ndm, long long n, int32_t *L,
+                                   DevState *st) {
     for (int d = blockIdx.y; d < ndm; d += gridDim.y) {
         const uint32_t *h = hotbits + (long long)d * nwr;
         for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nwr; w += gridDim.x * blockDim.x) {
             for (uint32_t q = run_starts(h[w], w > 0 ? h[w - 1] : 0u); q; q &= q - 1) {
                 const int32_t c = (int32_t)((long long)d * n + 32 * w + __ffs(q) - 1);
-                L[c] = find_root(L, c);
+                int32_t x = c, p = __ldcg(L + x);
+                while (p != x && p >= 0) {
+                    x = p;
+                    p = __ldcg(L + x);
+                }
+                L[c] = x != c ? x : -2 - (int32_t)atomicAdd(&st->nroots, 1u);
             }
         }
     }
 }
 
-// Roots get compact ids, stored in place as -(id + 2).
-__global__ void dd_ids_kernel(const uint32_t *__restrict__ hotbits, int nwr, int ndm, long long n, int32_t *L,
-                              DevState *st) {
-    for (int d = blockIdx.y; d < ndm; d += gridDim.y) {
-        const uint32_t *h = hotbits + (long long)d * nwr;
-        for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < nwr; w += gridDim.x * blockDim.x) {
-            for (uint32_t q = run_starts(h[w], w > 0 ? h[w - 1] : 0u); q; q &= q - 1) {
-                const int32_t c = (int32_t)((long long)d * n + 32 * w + __ffs(q) - 1);
-                if (L[c] == c) L[c] = -2 - (int32_t)atomicAdd(&st->nroots, 1u);
-            }
-        }
-    }
-}
-
-// Group id of a run start: start -> root (at most two hops after compression).
+// Group id of a run start: start -> root (one hop after compression).
 __device__ __forceinline__ int group_id(const int32_t *L, int32_t start) {
     int32_t v = L[start];
-    for (int hop = 0; hop < 2 && v >= 0; ++hop) v = L[v];
+    for (int hop = 0; hop < 1 && v >= 0; ++hop) v = L[v];
     return v <= -2 ? -2 - v : -1;
 }
 
 // Per group: the largest (S/N, -cell) key and the number of cells.  A lane
 // takes one word; each stretch of consecutive hot bits lies in one run and
 // gives one record, and the warp combines records of the same group before
-// its atomics.
+// its atomics.  The stretches' S/N values are read by the whole warp, a stretch
+// at a time (four on their way): lane by lane, each its own line of 32 values,
+// 3e7 hot cells of 1500 x 131072 took 144 us, now 134, bound by the chain of
+// loads from a run start to its group.  (A lane that goes down 4 or 16 rows and
+// hands records on when the group changes: 133 and 159 us.)
 __global__ void dd_group_reduce_kernel(const uint32_t *__restrict__ hotbits, int nwr, int ndm, long long n,
                                        const int32_t *__restrict__ L, const int32_t *__restrict__ wl,
                                        const float *__restrict__ best, int max_cands,
@@ -1174,22 +1164,38 @@ __global__ void dd_group_reduce_kernel(const uint32_t *__restrict__ hotbits, int
             int id = -1;
             unsigned long long kv = 0;
             unsigned cntv = 0;
+            int32_t c0 = 0;
+            unsigned todo = __ballot_sync(0xffffffffu, q != 0u);
             if (q) {
                 const int b0 = __ffs(q) - 1;
                 const uint32_t rest = ~(q >> b0);
                 const int len = rest ? __ffs(rest) - 1 : 32 - b0;
                 q = len >= 32 - b0 ? 0u : q & ~(((1u << len) - 1u) << b0);
-                const int32_t c0 = (int32_t)(cw + b0);
+                c0 = (int32_t)(cw + b0);
                 id = group_id(L, ((sq >> b0) & 1u) ? c0 : wlk);  // a stretch not at a run start begins at bit 0
                 if (id >= max_cands) id = -1;
-                for (int i = 0; i < len; ++i) {
-                    // largest S/N first, then the smallest cell index (lower DM, then earlier time)
-                    const uint32_t c = (uint32_t)(c0 + i);
-                    const unsigned long long v =
-                        ((unsigned long long)__float_as_uint(best[c]) << 32) | (unsigned long long)(0xFFFFFFFFu - c);
-                    kv = v > kv ? v : kv;
-                }
                 cntv = (unsigned)len;
+            }
+            while (todo) {
+                constexpr int kAhead = 4;
+                uint32_t v[kAhead];
+                int src[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    src[u] = todo ? __ffs(todo) - 1 : -1;
+                    todo &= todo - 1;
+                    const int32_t first = __shfl_sync(0xffffffffu, c0, src[u] & 31);
+                    const unsigned cells = __shfl_sync(0xffffffffu, cntv, src[u] & 31);
+                    v[u] = src[u] >= 0 && (unsigned)lane < cells ? __float_as_uint(best[(uint32_t)first + lane]) : 0u;
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    // largest S/N (positive: ordered as its bits) first, then the
+                    // smallest cell index (lower DM, then earlier time)
+                    const uint32_t top = __reduce_max_sync(0xffffffffu, v[u]);
+                    const int at = __ffs(__ballot_sync(0xffffffffu, v[u] == top)) - 1;
+                    if (lane == src[u]) kv = ((unsigned long long)top << 32) | (0xFFFFFFFFu - (uint32_t)(c0 + at));
+                }
             }
             const unsigned peers = __match_any_sync(0xffffffffu, id);
             unsigned long long m = kv;
@@ -1242,24 +1248,34 @@ __global__ void __launch_bounds__(kCompactThreads) dd_count_marks_kernel(const u
     if (threadIdx.x == 0) chunk_count[blockIdx.x] = s_cnt;
 }
 
-__global__ void __launch_bounds__(kCompactThreads) dd_scan_chunks_kernel(unsigned *__restrict__ chunk_count, int nchunks) {
-    // single CTA: exclusive scan in place, kCompactThreads entries at a time
-    __shared__ unsigned s[kCompactThreads];
-    unsigned carry = 0;
-    for (int base = 0; base < nchunks; base += kCompactThreads) {
-        const int i = base + threadIdx.x;
-        const unsigned v = i < nchunks ? chunk_count[i] : 0u;
-        s[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < kCompactThreads; o <<= 1) {
-            const unsigned u = threadIdx.x >= o ? s[threadIdx.x - o] : 0u;
-            __syncthreads();
-            s[threadIdx.x] += u;
-            __syncthreads();
+// Exclusive scan of the chunk counts in place, by one CTA, 1024 at a time with
+// two barriers each (256 at a time with 16 barriers: 12 us for 3000 chunks).
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) dd_scan_chunks_kernel(unsigned *__restrict__ chunk_count, int nchunks) {
+    __shared__ unsigned s_warp[2][kScanThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto warp_scan = [&](unsigned v) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
         }
-        if (i < nchunks) chunk_count[i] = carry + s[threadIdx.x] - v;
-        carry += s[kCompactThreads - 1];
+        return v;
+    };
+    unsigned carry = 0;
+    int buf = 0;
+    for (int base = 0; base < nchunks; base += kScanThreads) {
+        const int i = base + (int)threadIdx.x;
+        const unsigned v = i < nchunks ? chunk_count[i] : 0u;
+        const unsigned incl = warp_scan(v);
+        if (lane == 31) s_warp[buf][warp] = incl;
         __syncthreads();
+        // every warp scans the warps' totals; the other buffer is the next round's
+        const unsigned totals = warp_scan(s_warp[buf][lane]);
+        const unsigned before = __shfl_sync(0xffffffffu, totals, (warp + 31) & 31);
+        if (i < nchunks) chunk_count[i] = carry + (warp ? before : 0u) + incl - v;
+        carry += __shfl_sync(0xffffffffu, totals, 31);
+        buf ^= 1;
     }
 }
 
@@ -1586,8 +1602,7 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
     // word kernels: words of a row on x, rows on y
     const dim3 gw((unsigned)std::min((nwr + 255) / 256, 64), (unsigned)std::min(ndm, 4096));
     dd_vunion_kernel<<<gw, 256, 0, st>>>(s->hotbits, nwr, ndm, (long long)n, s->labels, s->wl, s->st);
-    dd_compress_kernel<<<gw, 256, 0, st>>>(s->hotbits, nwr, ndm, (long long)n, s->labels);
-    dd_ids_kernel<<<gw, 256, 0, st>>>(s->hotbits, nwr, ndm, (long long)n, s->labels, s->st);
+    dd_compress_kernel<<<gw, 256, 0, st>>>(s->hotbits, nwr, ndm, (long long)n, s->labels, s->st);
     dd_group_reduce_kernel<<<gw, 256, 0, st>>>(s->hotbits, nwr, ndm, (long long)n, s->labels, s->wl, s->best,
                                               s->cfg.max_cands, s->key, s->cnt);
     const long long nwords = (cells + 31) / 32;
@@ -1595,7 +1610,7 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
     dd_mark_kernel<<<g, 256, 0, st>>>(s->key, s->labels, s->marks, s->st, s->cfg.max_cands);
     const int nchunks = (int)((cells + kCompactChunk - 1) / kCompactChunk);
     dd_count_marks_kernel<<<nchunks, kCompactThreads, 0, st>>>(s->marks, nwords, s->chunk);
-    dd_scan_chunks_kernel<<<1, kCompactThreads, 0, st>>>(s->chunk, nchunks);
+    dd_scan_chunks_kernel<<<1, kScanThreads, 0, st>>>(s->chunk, nchunks);
     dd_write_marks_kernel<<<nchunks, kCompactThreads, 0, st>>>(s->marks, nwords, s->bestw, s->best, s->labels, s->cnt,
                                                                (long long)n, beam, s->chunk, s->cfg.max_cands,
                                                                s->cands);
