@@ -8,9 +8,8 @@
 //                    [t-half, t+half) of its own row segment, 32 outputs at a
 //                    time; writes y = x - median and adds sum(y^2) to the row
 //                    total (int64).
-//  * dd_xprefix_kernel, dd_mean_apply_kernel  the paper's running mean instead
-//                    (an option): row prefix sums, then x minus the window mean
-//                    rounded half up.
+//  * dd_mean_kernel  the paper's running mean instead (an option): x minus the
+//                    window mean rounded half up.
 //  * dd_mf_kernel       a CTA loads a tile of y plus the widest boxcar's halo,
 //                    prefix-sums it in shared memory, and for every sample
 //                    decides with integer thresholds whether some width reaches
@@ -93,6 +92,38 @@ __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_gr
 template <int N>
 __device__ __forceinline__ void copy_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Every output of the group of steps from t has its whole window [t - h, t + h)
+// in the row, and is one of those up to stop.
+__device__ __forceinline__ bool group_inside(unsigned t, unsigned h, unsigned n, unsigned stop) {
+    return t >= h && t + 32 * kMwGroup + h <= n && t + 32 * kMwGroup <= stop;
+}
+
+// Start copying the values of kMwGroup steps of 32 outputs: x[t], x[t + h] and
+// x[t - h] of the lane's outputs, into words 0, 32 and 64 of each step's 96 (a
+// lane reads only what it copied itself; values outside the row are not copied).
+__device__ __forceinline__ void fetch_group(uint32_t *to, const uint32_t *row, unsigned tg, int lane, unsigned h,
+                                            unsigned n, unsigned stop) {
+    const unsigned t = tg + (unsigned)lane;
+    const uint32_t *p = row + t;
+    if (group_inside(tg, h, n, stop)) {
+#pragma unroll
+        for (int j = 0; j < (int)kMwGroup; ++j) {
+            copy_async4(to + 96 * j, p + 32 * j);
+            copy_async4(to + 96 * j + 32, p + h + 32 * j);
+            copy_async4(to + 96 * j + 64, p - h + 32 * j);
+        }
+    } else {
+#pragma unroll 1
+        for (unsigned j = 0; j < kMwGroup; ++j)
+            if (t + 32 * j < stop) {
+                copy_async4(to + 96 * j, p + 32 * j);
+                if (t + 32 * j + h < n) copy_async4(to + 96 * j + 32, p + h + 32 * j);
+                if (t + 32 * j >= h) copy_async4(to + 96 * j + 64, row + (t + 32 * j - h));
+            }
+    }
+    copy_commit();
 }
 
 // H[bin] += by, if the bin is one.
@@ -213,32 +244,9 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
 #pragma unroll 1
     while (t0 < t_end) {
         const unsigned start = t0, stop = singles ? t0 + 1 : t_end;
-        // the values of kMwGroup steps: x[t], x[t + h], x[t - h] of the lane's
-        // outputs (each lane reads only what it copied itself)
-        auto inside = [&](unsigned t) {  // every output has its whole window in the row, and is of this go
-            return t >= h && t + 32 * kMwGroup + h <= n && t + 32 * kMwGroup <= stop;
-        };
-        auto fetch = [&](unsigned tg, int half) {
-            uint32_t *to = &s_ring[wid][half][0][0][lane];
-            const unsigned t = tg + (unsigned)lane;
-            const uint32_t *p = row + t;
-            if (inside(tg)) {
-#pragma unroll
-                for (int j = 0; j < (int)kMwGroup; ++j) {
-                    copy_async4(to + 96 * j, p + 32 * j);
-                    copy_async4(to + 96 * j + 32, p + h + 32 * j);
-                    copy_async4(to + 96 * j + 64, p - h + 32 * j);
-                }
-            } else {
-#pragma unroll 1
-                for (unsigned j = 0; j < kMwGroup; ++j)
-                    if (t + 32 * j < stop) {
-                        copy_async4(to + 96 * j, p + 32 * j);
-                        if (t + 32 * j + h < n) copy_async4(to + 96 * j + 32, p + h + 32 * j);
-                        if (t + 32 * j >= h) copy_async4(to + 96 * j + 64, row + (t + 32 * j - h));
-                    }
-            }
-            copy_commit();
+        auto inside = [&](unsigned t) { return group_inside(t, h, n, stop); };
+        auto fetch = [&](unsigned t, int half) {
+            fetch_group(&s_ring[wid][half][0][0][lane], row, t, lane, h, n, stop);
         };
         fetch(t0, 0);
         fetch(t0 + 32 * kMwGroup, 1);
@@ -397,17 +405,18 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
     if (most > top) atomicOr(&st->err, 1u);
 }
 
-// Outputs per segment.  A segment counts its first window (2 h values, 0.15 of a
-// step per 32 values), so long ones are cheaper, but the warps have to fill the
+// Outputs per segment.  A segment takes in its first window at the cost of `first`
+// outputs (the medians' histogram 0.15 of one per value, the means' sum 0.05), so
+// long ones are cheaper, but the warps have to fill the
 // device (32 per SM, half a segment's time lost at the end).  Measured for whole
 // searches of 1500 x 131072, h 4096, segments of 2048 / 4096 / 8192 (chosen):
 // 2718 / 2576 / 2504 us (40 warps per SM then); 16 x 100000, segments of 256 (chosen) / 4096: 142 / 167.
-unsigned median_segment(int ndm, long long n, long long h) {
+unsigned row_segment(int ndm, long long n, double first) {
     unsigned best = 0;
     double least = 0;
     for (unsigned seg = 256; seg <= 32768; seg *= 2) {
         const double warps = (double)ndm * (double)((n + seg - 1) / seg);
-        const double cost = (std::max(warps / (152.0 * kMwBlocks * kMwWarps), 1.0) + 0.5) * (0.3 * (double)h + seg);
+        const double cost = (std::max(warps / (152.0 * kMwBlocks * kMwWarps), 1.0) + 0.5) * (first + seg);
         if (!best || cost < least) {
             best = seg;
             least = cost;
@@ -417,221 +426,118 @@ unsigned median_segment(int ndm, long long n, long long h) {
 }
 
 // ---------------------------------------------------------------------------
-// baseline, paper form: running mean (rounded half up) from row prefix sums
+// baseline, paper form: running mean (rounded half up)
 // ---------------------------------------------------------------------------
 
-// Tile-local exclusive prefix of x (values clipped to top) and the tile's
-// total: a CTA stages kMfTile samples, each thread sums 16 consecutive ones,
-// a block scan of the thread totals gives its offset.
-__global__ void __launch_bounds__(256) dd_xprefix_kernel(const uint32_t *__restrict__ x, long long ld_x, long long n,
-                                                         uint32_t top, int32_t *__restrict__ pre,
-                                                         long long *__restrict__ tile_sum, int ntiles,
-                                                         DevState *st) {
-    // element i at i + i/16: a thread's 16 consecutive elements start at 17*tid,
-    // so the scan's reads and writes hit 32 distinct banks
-    __shared__ uint32_t xs[kMfTile + kMfTile / 16];
-    __shared__ int32_t s_warp[8];
-    const int d = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long t0 = (long long)blockIdx.x * kMfTile;
-    const uint32_t *row = x + (long long)d * ld_x;
-    bool over = false;
-    for (int i = tid; i < kMfTile; i += 256) {
-        uint32_t v = 0;
-        if (t0 + i < n) {
-            v = __ldg(row + t0 + i);
-            over |= v > top;
-            v = min(v, top);
-        }
-        xs[i + (i >> 4)] = v;
-    }
-    if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(&st->err, 1u);
-    __syncthreads();
-    int32_t loc[16];
-    int32_t tot = 0;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-        loc[q] = tot;
-        tot += (int32_t)xs[17 * tid + q];
-    }
-    int32_t incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += u;
-    }
-    if (lane == 31) s_warp[warp] = incl;
-    __syncthreads();
-    int32_t off = incl - tot;
-    for (int w = 0; w < warp; ++w) off += s_warp[w];
-    if (tid == 255) tile_sum[(long long)d * ntiles + blockIdx.x] = off + tot;
-    __syncthreads();
-    // back through shared memory for coalesced stores
-#pragma unroll
-    for (int q = 0; q < 16; ++q) xs[17 * tid + q] = (uint32_t)(loc[q] + off);
-    __syncthreads();
-    int32_t *prow = pre + (long long)d * n;
-    for (int i = tid; i < kMfTile; i += 256)
-        if (t0 + i < n) prow[t0 + i] = (int32_t)xs[i + (i >> 4)];
-}
-
-// floor(a / m) for a < 2^32 and 1 <= m < 2^16 from rm = 1/m rounded to
-// nearest: the float estimate a*rm is within 2^-6 of a/m (three roundings
-// of at most 2^-23 relative each, a/m < 2^16), so its truncation is off by
-// at most one, which one exact integer remainder corrects.
-__device__ __forceinline__ uint32_t udiv_small(uint32_t a, uint32_t m, float rm) {
-    uint32_t q = __float2uint_rz(__uint2float_rz(a) * rm);
-    const long long r = (long long)a - (long long)q * m;
-    if (r < 0) --q;
-    else if (r >= (long long)m) ++q;
-    return q;
+// floor(a / m) from inv = floor((2^32 - 1) / m), for a < 2^32 and 1 <= m < 2^17:
+// 2^32 / m exceeds inv by 1 at most, so the product's high word is the quotient
+// or one less, and the remainder tells.
+__device__ __forceinline__ uint32_t udiv_by(uint32_t a, uint32_t m, uint32_t inv) {
+    const uint32_t q = __umulhi(a, inv);
+    return q + (a - q * m >= m ? 1u : 0u);
 }
 
 // y[t] = x[t] - floor((S + floor(m/2)) / m) for the window sum S of its m
 // values (= the mean rounded half up; S < 2^32 since m <= 65534 and x <=
-// 65532), and the row's sum of y^2.  A block takes kMeanCells consecutive
-// outputs of a row, a thread every 256th.  Prefix values are used modulo 2^32:
-// a window sum is below 2^32, so the difference of the low words is exact.
-constexpr int kMeanCells = 2048;
-__global__ void __launch_bounds__(256) dd_mean_apply_kernel(const uint32_t *__restrict__ x, long long ld_x, long long n,
-                                                            long long h, uint32_t top,
-                                                            const int32_t *__restrict__ pre,
-                                                            const long long *__restrict__ tile_off,
-                                                            const long long *__restrict__ tile_sum, int ntiles,
-                                                            int32_t *__restrict__ y, long long ld_y,
-                                                            unsigned long long *__restrict__ sumsq) {
-    const int d = blockIdx.y;
-    const int32_t *prow = pre + (long long)d * n;
-    const long long *orow = tile_off + (long long)d * ntiles;
-    const uint32_t *xrow = x + (long long)d * ld_x;
-    int32_t *yrow = y + (long long)d * ld_y;
-    const int ni = (int)n, hi32 = (int)h;  // n < 2^31 (cells are int32 indices)
-    const uint32_t p_end = (uint32_t)(orow[ntiles - 1] + tile_sum[(long long)d * ntiles + ntiles - 1]);
-    const uint32_t m_full = (uint32_t)min(2LL * h, n);
-    const float rm_full = __frcp_rn((float)m_full);
-    unsigned long long sq = 0;
-    const int t0 = blockIdx.x * kMeanCells + threadIdx.x;
-#pragma unroll 4
-    for (int j = 0; j < kMeanCells / 256; ++j) {
-        const int t = t0 + 256 * j;
-        if (t >= ni) break;
-        const int lo = max(0, t - hi32), hi = min(ni, t + hi32);
-        const uint32_t p_hi = hi == ni ? p_end : (uint32_t)orow[hi / kMfTile] + (uint32_t)prow[hi];
-        const uint32_t p_lo = (uint32_t)orow[lo / kMfTile] + (uint32_t)prow[lo];
-        const uint32_t S = p_hi - p_lo;
-        const uint32_t m = (uint32_t)(hi - lo);
-        const float rm = m == m_full ? rm_full : __frcp_rn((float)m);
-        const uint32_t mean = udiv_small(S + m / 2, m, rm);
-        const int32_t yv = (int32_t)min(__ldg(xrow + t), top) - (int32_t)mean;
-        yrow[t] = yv;
-        sq += (unsigned long long)((long long)yv * yv);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if ((threadIdx.x & 31) == 0 && sq) atomicAdd(sumsq + d, sq);
-}
+// 65532), and the row's sum of y^2.  A warp takes a row segment as in the median
+// kernel, one lane per output: S moves by the difference of the value that
+// enters and the one that leaves, scanned over the warp.  Nothing but x is read
+// and nothing but y written; a block that staged 8192 outputs with both windows'
+// values and scanned them in shared memory (what this replaces) read and added
+// every value twice: 253 us for 700 x 100003 with window 8192, now 204 (0.56 GB,
+// 82 us; bound by instruction issue, the scan and the division).
+__global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_mean_kernel(
+    const uint32_t *__restrict__ x, long long ld_x, int ndm, unsigned n, unsigned h, unsigned seg, unsigned nseg,
+    uint32_t top, int32_t *__restrict__ y, long long ld_y, unsigned long long *__restrict__ sumsq, DevState *st) {
+    __shared__ uint32_t s_ring[kMwWarps][2][kMwGroup][3][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long g = (long long)blockIdx.x * kMwWarps + wid;
+    const int d = (int)(g / nseg);
+    if (d >= ndm) return;
+    unsigned t0 = (unsigned)(g % nseg) * seg;
+    const unsigned t_end = min(n, t0 + seg);
+    const uint32_t *const row = x + (long long)d * ld_x;
+    int32_t *const yrow = y + (long long)d * ld_y;
+    fetch_group(&s_ring[wid][0][0][0][lane], row, t0, lane, h, n, t_end);
+    fetch_group(&s_ring[wid][1][0][0][lane], row, t0 + 32 * kMwGroup, lane, h, n, t_end);
 
-// Fused form of the same baseline, used when a tile's window span fits in
-// shared memory: a CTA takes kMeanTile consecutive outputs of a row, stages
-// the row's values over [t0 - h, t0 + kMeanTile + h) (clipped to the row and
-// to top), forms their exclusive prefix P in shared memory (32 values per
-// thread per pass, one padding word per 32 so the passes are free of bank
-// conflicts), and writes y[t] = x[t] - floor((S + floor(m/2)) / m) with
-// S = P[hi] - P[lo] for the window [lo, hi) of t and x[t] = P[t+1] - P[t], and
-// the row's sum of y^2.  No row-wide prefix goes through memory.
-constexpr int kMeanTile = 8192;
-constexpr int kMeanThreads = 512;
-constexpr int kMeanPass = 32 * kMeanThreads;  // span values per scan pass
-__host__ __device__ constexpr int mean_pad(int i) { return i + (i >> 5); }
-inline size_t mean_fused_smem(long long h) {
-    const long long span = kMeanTile + 2 * h;
-    return (size_t)(mean_pad((int)span) + 1) * 4;
-}
-constexpr size_t kMeanFusedSmemMax = 200 * 1024;
-
-__global__ void __launch_bounds__(kMeanThreads) dd_mean_fused_kernel(const uint32_t *__restrict__ x, long long ld_x,
-                                                                     long long n, long long h, uint32_t top,
-                                                                     int32_t *__restrict__ y, long long ld_y,
-                                                                     unsigned long long *__restrict__ sumsq,
-                                                                     DevState *st) {
-    extern __shared__ __align__(16) uint32_t Pm[];
-    __shared__ uint32_t s_warp[kMeanThreads / 32];
-    __shared__ uint32_t s_carry;
-    const int d = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const long long t0 = (long long)blockIdx.x * kMeanTile;
-    const long long lo0 = max(0LL, t0 - h), hi0 = min(n, t0 + kMeanTile + h);
-    const int L = (int)(hi0 - lo0);
-    const uint32_t *row = x + (long long)d * ld_x + lo0;
-    bool over = false;
-    // 16-byte loads when the span starts on a 16-byte boundary (4 values at
-    // i..i+3 never straddle a padding word), then the ragged rest one by one
-    const int L4 = (reinterpret_cast<uintptr_t>(row) & 15u) == 0 ? L / 4 : 0;
-    for (int q = tid; q < L4; q += kMeanThreads) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(row) + q);
-        over |= v.x > top || v.y > top || v.z > top || v.w > top;
-        uint32_t *dst = Pm + mean_pad(4 * q);
-        dst[0] = min(v.x, top);
-        dst[1] = min(v.y, top);
-        dst[2] = min(v.z, top);
-        dst[3] = min(v.w, top);
-    }
-    for (int i = 4 * L4 + tid; i < L; i += kMeanThreads) {
-        const uint32_t v = __ldg(row + i);
-        over |= v > top;
-        Pm[mean_pad(i)] = min(v, top);
-    }
-    if (__any_sync(0xffffffffu, over) && lane == 0) atomicOr(&st->err, 1u);
-    if (tid == 0) s_carry = 0u;
-    __syncthreads();
-    for (int c0 = 0; c0 < L; c0 += kMeanPass) {
-        const int b = c0 + 32 * tid;
-        uint32_t v[32];
-        uint32_t tot = 0;
+    // sum of the first window
+    uint32_t sum = 0;
+    {
+        unsigned i = t0 - min(t0, h) + (unsigned)lane;
+        const unsigned hi = min(n, t0 + h);
+        for (; i + 7 * 32 < hi; i += 8 * 32) {
+            uint32_t v[8];
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            v[q] = b + q < L ? Pm[mean_pad(b + q)] : 0u;
-            const uint32_t e = tot;
-            tot += v[q];
-            v[q] = e;
+            for (int u = 0; u < 8; ++u) v[u] = __ldg(row + i + 32 * u);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) sum += min(v[u], top);
         }
-        uint32_t incl = tot;
+        for (; i < hi; i += 32) sum += min(__ldg(row + i), top);
+        sum = __reduce_add_sync(0xffffffffu, sum);  // below 2^32
+    }
+    const uint32_t m_full = 2 * h, inv_full = 0xffffffffu / m_full;
+    unsigned long long ssq = 0;
+    uint32_t most = 0;
+    // the outputs of one group; FULL: an inside one
+    auto group = [&](auto is_full, const uint32_t *from) {
+        constexpr bool FULL = decltype(is_full)::value;
+        uint32_t cur[kMwGroup], incl[kMwGroup], own[kMwGroup];
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += u;
+        for (int j = 0; j < (int)kMwGroup; ++j) {
+            const unsigned t = t0 + 32 * j + (unsigned)lane;
+            const bool act = FULL || t < t_end;
+            cur[j] = act ? from[96 * j] : 0u;
+            own[j] = (FULL || (act && t + h < n) ? min(from[96 * j + 32], top) : 0u) -
+                     (FULL || (act && t >= h) ? min(from[96 * j + 64], top) : 0u);
+            incl[j] = own[j];
         }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        uint32_t off = s_carry + incl - tot;
-        for (int w = 0; w < warp; ++w) off += s_warp[w];
 #pragma unroll
-        for (int q = 0; q < 32; ++q)
-            if (b + q < L) Pm[mean_pad(b + q)] = v[q] + off;
-        __syncthreads();
-        if (tid == kMeanThreads - 1) s_carry = off + tot;
-        __syncthreads();
-    }
-    if (tid == 0) Pm[mean_pad(L)] = s_carry;
-    __syncthreads();
-    const long long m_full = min(2LL * h, n);
-    const float rm_full = __frcp_rn((float)m_full);
-    const int nt = (int)min((long long)kMeanTile, n - t0);
-    int32_t *yrow = y + (long long)d * ld_y + t0;
-    unsigned long long sq = 0;
-    for (int j = tid; j < nt; j += kMeanThreads) {
-        const long long t = t0 + j;
-        const int lo = (int)(max(0LL, t - h) - lo0), hi = (int)(min(n, t + h) - lo0), c = (int)(t - lo0);
-        const uint32_t S = Pm[mean_pad(hi)] - Pm[mean_pad(lo)];
-        const uint32_t m = (uint32_t)(hi - lo);
-        const float rm = m == (uint32_t)m_full ? rm_full : __frcp_rn((float)m);
-        const uint32_t mean = udiv_small(S + m / 2, m, rm);
-        const int32_t xv = (int32_t)(Pm[mean_pad(c + 1)] - Pm[mean_pad(c)]);
-        const int32_t yv = xv - (int32_t)mean;
-        yrow[j] = yv;
-        sq += (unsigned long long)((long long)yv * yv);
-    }
+        for (int o = 1; o < 32; o <<= 1) {  // the four steps' moves, scanned over the warp
+            const bool add = lane >= o;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane == 0 && sq) atomicAdd(sumsq + d, sq);
+            for (int j = 0; j < (int)kMwGroup; ++j) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, incl[j], o);
+                if (add) incl[j] += u;
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < (int)kMwGroup; ++j) {
+            const unsigned t = t0 + 32 * j + (unsigned)lane;
+            const uint32_t S = sum + incl[j] - own[j];
+            uint32_t mean;
+            if (FULL) {
+                mean = udiv_by(S + h, m_full, inv_full);
+            } else {
+                const uint32_t m = t < t_end ? min(n, t + h) - (t - min(t, h)) : 1u;
+                mean = udiv_by(S + m / 2, m, 0xffffffffu / m);
+            }
+            most = max(most, cur[j]);
+            const int32_t yv = (int32_t)min(cur[j], top) - (int32_t)mean;
+            if (FULL || t < t_end) {
+                yrow[t] = yv;
+                ssq += (unsigned long long)((long long)yv * yv);
+            }
+            sum += __shfl_sync(0xffffffffu, incl[j], 31);
+        }
+    };
+    int half = 0;
+#pragma unroll 1
+    for (; t0 < t_end; t0 += 32 * kMwGroup) {
+        copy_wait<1>();
+        const uint32_t *from = &s_ring[wid][half][0][0][lane];
+        if (group_inside(t0, h, n, t_end))
+            group(std::true_type(), from);
+        else
+            group(std::false_type(), from);
+        fetch_group(&s_ring[wid][half][0][0][lane], row, t0 + 64 * kMwGroup, lane, h, n, t_end);
+        half ^= 1;
+    }
+    copy_wait<0>();
+#pragma unroll
+    for (int o = 16; o; o >>= 1) ssq += __shfl_down_sync(0xffffffffu, ssq, o);
+    if (lane == 0 && ssq) atomicAdd(sumsq + d, ssq);
+    if (most > top) atomicOr(&st->err, 1u);
 }
 
 // ---------------------------------------------------------------------------
@@ -1553,26 +1459,14 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
     // baseline
     const long long h = s->cfg.half_window;
     s->ntiles = (int)((n + kMfTile - 1) / kMfTile);
-    if (s->cfg.baseline == 1 && mean_fused_smem(h) <= kMeanFusedSmemMax) {
-        const size_t sm = mean_fused_smem(h);
-        static thread_local size_t configured = 0;
-        if (sm > 48 * 1024 && sm > configured) {
-            DD_CUDA_TRY(cudaFuncSetAttribute(dd_mean_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            configured = sm;
-        }
-        dd_mean_fused_kernel<<<dim3((unsigned)(((long long)n + kMeanTile - 1) / kMeanTile), (unsigned)ndm), kMeanThreads,
-                               sm, st>>>(d_x, (long long)ld_x, (long long)n, h, (uint32_t)(s->nbins - 1), s->y, s->ld_y,
-                                         s->sumsq, s->st);
-    } else if (s->cfg.baseline == 1) {
-        dd_xprefix_kernel<<<dim3((unsigned)s->ntiles, (unsigned)ndm), 256, 0, st>>>(
-            d_x, (long long)ld_x, (long long)n, (uint32_t)(s->nbins - 1), s->pre, s->tile_sum, s->ntiles, s->st);
-        dd_tile_scan_kernel<<<(ndm + 127) / 128, 128, 0, st>>>(s->tile_sum, s->tile_off, ndm, s->ntiles);
-        dd_mean_apply_kernel<<<dim3((unsigned)(((long long)n + kMeanCells - 1) / kMeanCells), (unsigned)ndm), 256, 0,
-                               st>>>(
-            d_x, (long long)ld_x, (long long)n, h, (uint32_t)(s->nbins - 1), s->pre, s->tile_off, s->tile_sum,
-            s->ntiles, s->y, s->ld_y, s->sumsq);
+    if (s->cfg.baseline == 1) {
+        const unsigned seg = row_segment(ndm, (long long)n, 0.1 * (double)h);
+        const unsigned nseg = (unsigned)(((long long)n + seg - 1) / seg);
+        dd_mean_kernel<<<(unsigned)(((long long)ndm * nseg + kMwWarps - 1) / kMwWarps), 32 * kMwWarps, 0, st>>>(
+            d_x, (long long)ld_x, ndm, (unsigned)n, (unsigned)h, seg, nseg, (uint32_t)(s->nbins - 1), s->y, s->ld_y,
+            s->sumsq, s->st);
     } else {
-        const unsigned seg = median_segment(ndm, (long long)n, h);
+        const unsigned seg = row_segment(ndm, (long long)n, 0.3 * (double)h);
         const unsigned nseg = (unsigned)(((long long)n + seg - 1) / seg);
         dd_median_kernel<<<(unsigned)(((long long)ndm * nseg + kMwWarps - 1) / kMwWarps), 32 * kMwWarps, 0, st>>>(
             d_x, (long long)ld_x, ndm, (unsigned)n, (unsigned)h, seg, nseg, (uint32_t)(s->nbins - 1), s->y, s->ld_y,

@@ -432,3 +432,30 @@ def test_hot_cells_at_the_threshold(P, n, widths):
     assert hot == int((best >= np.float32(thresh)).sum()) and full.result()["nhot"] == hot
     a, b = s.candidates(), full.candidates()
     np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("ndm,n,half", [(3, 127, 20), (3, 128, 64), (3, 129, 65), (5, 255, 1), (5, 385, 128),
+                                        (700, 4609, 1024), (1600, 4230, 96), (2, 70001, 32767)])
+def test_mean_baseline_segment_edges(P, ndm, n, half):
+    """The running mean at the lengths and windows around a warp's segments and
+    groups of steps, rows at odd offsets, the largest sums and windows: y and
+    sum y^2 equal the oracle's; values above the largest sum are flagged."""
+    import torch
+
+    rng = np.random.default_rng(ndm * n + half)
+    top = 3 * 21844
+    x = rng.integers(0, top + 1, (ndm, n)).astype(np.uint32)
+    x[1] = top
+    wide = np.full((ndm, n + 5), 0xFFFFFFFF, dtype=np.uint32)
+    wide[:, 3:n + 3] = x
+    for flagged in (False, True):
+        if flagged:
+            wide[0, 3 + n // 2] = top + 1
+        s = P.Search(ndm, n, nchan=21844, half_window=half, widths=(1,), thresh=50.0, max_cands=64, baseline="mean")
+        s.run(torch.from_numpy(wide.view(np.int32)).cuda()[:, 3:n + 3], ndm, n)
+        assert s.result()["flags"] & 1 == int(flagged)
+        y, ss, _, _ = s.buffers()
+        y_or = oracle.baseline_mean(np.minimum(wide[:, 3:n + 3], top), half)
+        np.testing.assert_array_equal(y.cpu().numpy(), y_or)
+        np.testing.assert_array_equal(ss.cpu().numpy(), [oracle.sumsq(r) for r in y_or])
+        s.close()
