@@ -7,6 +7,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
+#include <numeric>
+#include <thread>
 #include <vector>
 
 #include "dd_internal.h"
@@ -135,6 +138,24 @@ Encode gsum_encoder() {
 // Dynamic shared memory of a CTA, for every plan: all there is.
 size_t gsum_smem() { return 227 * 1024; }
 
+// f(b) for every DM block, on a few threads (1500 trials x 1024 channels: the
+// tables took 6 ms of a plan's creation on one); f does not throw.
+template <class F>
+static void each_block(int n, F f) {
+    const int want = std::min({8, (int)std::thread::hardware_concurrency(), n / 4});
+    std::atomic<int> next{0};
+    auto work = [&] {
+        for (int b = next++; b < n; b = next++) f(b);
+    };
+    std::vector<std::thread> threads;
+    try {
+        for (int k = 1; k < want; ++k) threads.emplace_back(work);
+    } catch (...) {  // no more threads: those there are do the work
+    }
+    work();
+    for (std::thread &t : threads) t.join();
+}
+
 // Sizes and host tables of a plan; t.ok stays false when the plan does not suit.
 static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab, std::vector<int32_t> &ws) {
     if (p->nchan < kChunkChans || 3 * p->nchan >= 1 << 14) return;
@@ -143,14 +164,18 @@ static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab,
     t.nchunks = ((ngroups + kCG - 1) / kCG + 1) / 2 * 2;
     std::vector<Group> groups((size_t)t.n_dmb * t.nchunks * kCG);
     std::vector<int> from_word((size_t)t.n_dmb * t.nchunks * kParts);  // first staged word of each part
-    int most = 0;
-    for (int b = 0; b < t.n_dmb; ++b)
-        for (int s = 0; s < t.nchunks * kParts; ++s) {
+    std::vector<int> most(t.n_dmb, 0);
+    std::atomic<bool> suits{true};
+    each_block(t.n_dmb, [&](int b) {
+        for (int s = 0; s < t.nchunks * kParts && suits; ++s) {
             const size_t k = (size_t)b * t.nchunks * kParts + s;
             int lo = 0x7fffffff, end = 0;
             for (int g = 0; g < kHalfCG && s * kHalfCG + g < ngroups; ++g) {
                 Group &x = groups[k * kHalfCG + g];
-                if (!make_group(p, b * kD, (s * kHalfCG + g) * kG, x)) return;
+                if (!make_group(p, b * kD, (s * kHalfCG + g) * kG, x)) {
+                    suits = false;
+                    return;
+                }
                 for (int i = 0; i < x.nchan; ++i) {
                     lo = std::min(lo, x.start[i] >> 4);
                     end = std::max(end, (x.start[i] >> 4) + x.words);
@@ -158,9 +183,11 @@ static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab,
             }
             if (s * kHalfCG >= ngroups) continue;
             from_word[k] = lo & ~3;
-            most = std::max(most, end - from_word[k]);
+            most[b] = std::max(most[b], end - from_word[k]);
         }
-    t.slot = (most + kHalfWords + 2 + 3) / 4 * 4;
+    });
+    if (!suits) return;
+    t.slot = (*std::max_element(most.begin(), most.end()) + kHalfWords + 2 + 3) / 4 * 4;
     if (t.slot > 256) return;  // a tensor map's box
     tab.assign((size_t)t.n_dmb * t.nchunks * kRecWords, 0u);
     ws.assign((size_t)t.n_dmb * 2 * kParts, 0);
@@ -222,9 +249,14 @@ static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab,
         }
         if (!fits) return;
     }
-    double alu = 0;  // ALU instructions of all DM blocks' tiles, per warp
-    int turn = 0;  // items go round the warps
-    for (int b = 0; b < t.n_dmb; ++b) {
+    std::vector<int> turn(need.size());  // items go round the warps
+    for (size_t n = 0, items = 0; n < need.size(); ++n) {
+        turn[n] = (int)(items % kWarps);
+        items += (size_t)(kHalfCG * need[n] + 31) / 32;
+    }
+    std::vector<double> alus(t.n_dmb, 0.0);  // ALU instructions of a tile of each DM block
+    each_block(t.n_dmb, [&](int b) {
+        double alu = 0;
         for (int q = 0; q < 2 * kParts; ++q) ws[(size_t)b * 2 * kParts + q] = from_word[(size_t)b * nparts + q];
         for (int s = 0; s < t.nchunks; ++s) {
             const size_t k = (size_t)b * t.nchunks + s;
@@ -238,8 +270,7 @@ static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab,
                 r[0] = (uint32_t)half[n];
                 r[1] = (uint32_t)need[n];
                 r[3] = s + 2 < t.nchunks ? (uint32_t)from_word[(k + 2) * kParts + part] : 0u;
-                r[2] = (uint32_t)units | (uint32_t)(turn % kWarps) << 8 | (uint32_t)keep[k] << 16;
-                turn += units;
+                r[2] = (uint32_t)units | (uint32_t)turn[n] << 8 | (uint32_t)keep[k] << 16;
                 uint32_t at = (uint32_t)(vec_at(t.slot) + place[n]);
                 double vwork = 0;
                 for (int g = 0; g < kHalfCG; ++g) {
@@ -276,10 +307,11 @@ static void gsum_tables(const Plan *p, GsumTable &t, std::vector<uint32_t> &tab,
                 alu += kWarps * kDT * kHalfCG * 31.0 + units * (70 + vwork / kHalfCG);
             }
         }
-    }
+        alus[b] = alu;
+    });
     if (pool < kWarps * kHalf * 4) return;  // the finished sums pass through the pool's place
     // two of the ALU's warp instructions a cycle at the 80 % that the kernel reaches
-    t.tile_cycles = 0.615 * alu / t.n_dmb + 14400;
+    t.tile_cycles = 0.615 * std::accumulate(alus.begin(), alus.end(), 0.0) / t.n_dmb + 14400;
     t.ok = true;
 }
 
@@ -287,7 +319,11 @@ void build_gsum(Plan *p) {
     GsumTable &t = p->gs;
     std::vector<uint32_t> tab;
     std::vector<int32_t> ws;
-    gsum_tables(p, t, tab, ws);
+    try {
+        gsum_tables(p, t, tab, ws);
+    } catch (...) {  // no host memory for them: the tiled kernel serves the plan
+        t.ok = false;
+    }
     if (!t.ok || !gsum_encoder()) return free_gsum(p);
     cudaError_t e = cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, p->device);
     if (e == cudaSuccess) e = cudaMalloc(&t.tab, tab.size() * 4);
