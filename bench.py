@@ -326,10 +326,10 @@ class GulpPipeline:
         if ev:
             ev[4].record(s)
         self.last_n = n
-        # kernels launched: dedispersion 1, search 13 (median, thresholds, matched filter, tile scan, runs,
-        # row joins, compress, ids, group reduce, marks, count, scan, write), snippets (if any),
+        # kernels launched: dedispersion 1, search 12 (median, thresholds, matched filter, tile scan, runs,
+        # row joins, compress, group reduce, marks, count, scan, write), snippets (if any),
         # classifier 6 per chunk (4 convolutions, fc1, fc2)
-        return 1 + 13 + (1 if n else 0) + 6 * ((n + CLF_BATCH - 1) // CLF_BATCH)
+        return 1 + 12 + (1 if n else 0) + 6 * ((n + CLF_BATCH - 1) // CLF_BATCH)
 
     def baseline_variants(self, reps=3):
         """The search stage on the last gulp's dedispersed rows with the running
@@ -891,7 +891,7 @@ def launch_table(path: str) -> int:
         if k in tiled:
             if k == chosen:
                 rows[k] = (t / n, 1.0)
-        elif not (k.startswith("probe_kernel") or "elementwise" in k or "distribution" in k):
+        elif not ("probe_kernel" in k or k.startswith("fp_check") or "elementwise" in k or "distribution" in k):
             rows[k] = (t / steps, n / steps)
     tot = sum(v[0] for v in rows.values())
     print("| kernel | launches per step | ms per step | share |\n|---|---|---|---|")
