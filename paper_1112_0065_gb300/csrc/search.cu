@@ -74,9 +74,10 @@ constexpr int kPows = 11;  // possible widths 2^0 .. 2^10
 // output's bookkeeping was one dependency chain, 8192 outputs and counts long,
 // with too few lanes to hide it.  Measured, window 8192: the search of a
 // dedispersed gulp of 1500 x 131072 with pulses and interference 2606 us before,
-// 1875 now (the medians 1496 of 2780 before); searches of noise rows, 700 x 100003:
+// 1875 now (the medians alone 1496 and 750); searches of noise rows, 700 x 100003:
 // 1800 before, 999 now, 16 x 100000: 1126 and 116; 1500 x 40000 with window
-// 1000: 1009 and 889.  A bound on the counts by one warp sum before the ballots
+// 1000: 1009 and 904; 300 x 20000 with window 128 and steps in the rows: 254 and
+// 205.  A bound on the counts by one warp sum before the ballots
 // settled two steps in three at window 8192 and cost more than it saved.
 constexpr int kMwWarps = 4;    // warps per block, each on its own row segment
 constexpr int kMwBins = 256;   // values base .. base + 255 are counted
@@ -235,18 +236,16 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
     unsigned long long ssq = 0;
     uint32_t most = 0;
     unsigned builds = 0;
-    int singles = 0;  // outputs to take one by one
 
     // One go: the histogram from the window of t0, then steps of 32 outputs
-    // until the segment ends or a median lies beyond the bins; the next go has
-    // its bins around the present median.  Where that one fails at once, the 32
-    // medians lie too far apart for any bins and 32 goes take one output each.
+    // until the segment ends or a median lies beyond the bins; the next go
+    // starts at that output, with its bins around the median before it (its
+    // first output's median is then within the bins).
 #pragma unroll 1
     while (t0 < t_end) {
-        const unsigned start = t0, stop = singles ? t0 + 1 : t_end;
-        auto inside = [&](unsigned t) { return group_inside(t, h, n, stop); };
+        auto inside = [&](unsigned t) { return group_inside(t, h, n, t_end); };
         auto fetch = [&](unsigned t, int half) {
-            fetch_group(&s_ring[wid][half][0][0][lane], row, t, lane, h, n, stop);
+            fetch_group(&s_ring[wid][half][0][0][lane], row, t, lane, h, n, t_end);
         };
         fetch(t0, 0);
         fetch(t0 + 32 * kMwGroup, 1);
@@ -279,11 +278,12 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
             ++builds;
         }
 
-        // 32 outputs; FULL: of an inside group.  false: a median lies beyond the bins.
+        // 32 outputs; FULL: of an inside group.  Returns those before the first
+        // whose median lies beyond the bins.
         auto step = [&](auto is_full, unsigned ts, const uint32_t *from) {
             constexpr bool FULL = decltype(is_full)::value;
             const unsigned t = ts + (unsigned)lane;
-            const bool act = FULL || t < stop;
+            const bool act = FULL || t < t_end;
             const uint32_t nc = from[0];
             int vi = (int)min(from[32], top), vo = (int)min(from[64], top);
             if (!FULL) {  // past the row: above every median
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
             // m is the median of all 32?  (Of a window of 8192 noise values nine
             // times in ten.)
             const int c0 = b0 + __popc(i0 & lt) - __popc(o0 & lt), c1 = b1 + __popc(i1 & lt) - __popc(o1 & lt);
-            int med = m, to = m;
+            int med = m, to = m, done = 32;
             if (__any_sync(0xffffffffu, act && (c0 > r || c1 <= r))) {
                 // values of the window of output t that are below v: (those of
                 // the window of ts) + (entered since) - (left since)
@@ -309,9 +309,13 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
                 };
                 __syncwarp();
                 int v = m + 1, b = b1, c = c1;
+                unsigned left;  // lanes whose median is v or above it, below
 #pragma unroll 1
-                while (__any_sync(0xffffffffu, act && c <= r)) {
-                    if (v - base >= kMwBins) return false;
+                while ((left = __ballot_sync(0xffffffffu, act && c <= r))) {
+                    if (v - base >= kMwBins) {
+                        done = __ffs(left) - 1;
+                        break;
+                    }
                     if (c <= r) med = v;
                     b += (int)H[v - base];
                     ++v;
@@ -319,9 +323,12 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
                 }
                 v = m, b = b0, c = c0;
 #pragma unroll 1
-                while (__any_sync(0xffffffffu, act && c > r)) {
+                while ((left = __ballot_sync(0xffffffffu, act && c > r))) {
                     --v;
-                    if (v < base) return false;
+                    if (v < base) {
+                        done = min(done, __ffs(left) - 1);
+                        break;
+                    }
                     if (c > r) med = v;
                     b -= (int)H[v - base];
                     c = b + since(v);
@@ -329,11 +336,15 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
                 to = __shfl_sync(0xffffffffu, med, 31);
                 __syncwarp();
             }
-            if (act) {
+            if (act && lane < done) {
                 most = max(most, nc);
                 const int yv = (int)min(nc, top) - med;
                 yrow[t] = yv;
                 ssq += (unsigned long long)((long long)yv * yv);
+            }
+            if (done < 32) {
+                if (done) m = __shfl_sync(0xffffffffu, med, done - 1);
+                return done;
             }
             // the window moves on by 32
             mw_bump(h_addr, vi - base, 1u);
@@ -354,29 +365,31 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
                 }
                 __syncwarp();
             }
-            return true;
+            return done;
         };
         int half = 0;
         bool far = false;
 #pragma unroll 1
-        while (t0 < stop) {
+        while (t0 < t_end) {
             copy_wait<1>();
             const uint32_t *from = &s_ring[wid][half][0][0][lane];
             if (inside(t0)) {
 #pragma unroll kMwUnroll
                 for (unsigned j = 0; j < kMwGroup; ++j) {
-                    far = !step(std::true_type(), t0 + 32 * j, from + 96 * j);
-                    if (far) {
-                        t0 += 32 * j;
+                    const int done = step(std::true_type(), t0 + 32 * j, from + 96 * j);
+                    if (done < 32) {
+                        t0 += 32 * j + (unsigned)done;
+                        far = true;
                         break;
                     }
                 }
             } else {
 #pragma unroll 1
-                for (unsigned j = 0; j < kMwGroup && t0 + 32 * j < stop; ++j) {
-                    far = !step(std::false_type(), t0 + 32 * j, from + 96 * j);
-                    if (far) {
-                        t0 += 32 * j;
+                for (unsigned j = 0; j < kMwGroup && t0 + 32 * j < t_end; ++j) {
+                    const int done = step(std::false_type(), t0 + 32 * j, from + 96 * j);
+                    if (done < 32) {
+                        t0 += 32 * j + (unsigned)done;
+                        far = true;
                         break;
                     }
                 }
@@ -389,12 +402,6 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
         copy_wait<0>();
         __syncwarp();
         guess = m;
-        if (singles) {
-            --singles;
-            t0 = start + 1;
-        } else if (far && t0 == start) {
-            singles = 32;
-        }
     }
 #pragma unroll
     for (int o = 16; o; o >>= 1) ssq += __shfl_down_sync(0xffffffffu, ssq, o);
