@@ -56,6 +56,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         a.map = &desc->map[b];
         const long long local = g - desc->tile_start[b];
         if (!gsum_tile<NP>(a, (int)(local % a.n_dmb), local / a.n_dmb, gsum_smem, phase)) break;
+        // the next tile's beam may have another layout, whose copies land where
+        // this tile's threads wrote (zero slot, output rows)
+        tc::fence_async_smem();
         __syncthreads();
     }
 }

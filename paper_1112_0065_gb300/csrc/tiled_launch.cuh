@@ -44,6 +44,9 @@ __global__ void __launch_bounds__(kThreads, TileOcc<DT, W, NP>::value)
         const TiledArgs a = desc->beam[b];
         const long long local = g - desc->tile_start[b];
         if (!dd_tile<DT, W, NP, G>(a, (int)(local % a.n_dmb), local / a.n_dmb, smem, phase)) break;
+        // the next tile's beam may have another layout, whose copies land where
+        // this tile's threads wrote (zero slots, window bases)
+        tc::fence_async_smem();
         __syncthreads();
     }
 }

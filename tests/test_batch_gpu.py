@@ -260,3 +260,38 @@ def test_batch_changes_kernels_with_its_beams(P, use_graph):
         captured.replay() if captured is not None else b.launch()
         _check(P, beams, want)
     b.close()
+
+
+@pytest.mark.parametrize("tiled", [False, True])
+def test_neighbouring_tiles_of_different_layouts(P, tiled):
+    """Beams whose shared-memory layouts differ (the windows of their DM ranges
+    are 156, 188 and 180 words long in the channel-group kernel) in turn, some
+    fifty tiles per CTA: what one tile's threads wrote lies where the next
+    tile's copies land, and every sum equals the tiled kernel's single-gulp
+    one.  (No order of the two can be forced; the fence between them is checked
+    in the source, on the CPU.)"""
+    import torch
+
+    f = synth.band_freqs(1024)
+    kernel = P.KERNEL_TILED if tiled else P.KERNEL_AUTO
+    plans = {m: (P.Plan(f, 64e-6, synth.dm_list_piecewise(m), kernel=kernel),
+                 P.Plan(f, 64e-6, synth.dm_list_piecewise(m), kernel=P.KERNEL_TILED)) for m in (250.0, 1000.0, 500.0)}
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    items, wants = [], []
+    for i, m in enumerate((250.0, 1000.0, 500.0, 1000.0, 250.0, 500.0)):
+        plan, alone = plans[m]
+        nout = 65537 + 640 * i
+        nsamp = nout + plan.maxdelay
+        d_in = torch.randint(0, 256, (1024, P.row_bytes(nsamp)), dtype=torch.uint8, device="cuda", generator=gen)
+        items.append((plan, d_in, nsamp, torch.empty((plan.ndm, P.out_stride(nout)), dtype=torch.int32, device="cuda")))
+        wants.append(alone.execute(d_in, nsamp)[:, :nout])
+        assert plan.uses_channel_groups(nsamp) == (not tiled)
+    b = P.Batch(items, use_graph=True)
+    for _ in range(5):
+        for _, _, _, out in items:
+            out.fill_(-1)
+        b.launch()
+        for (_, _, _, out), want in zip(items, wants):
+            assert bool((out[:, : want.shape[1]] == want).all())
+    b.close()
+    assert P.dedisp_status() == 0
