@@ -38,7 +38,7 @@ METRIC = "dedispersion Gsamp/s (nchan*ndm*nsamp)"
 KERNEL_SRCS = [os.path.join(ROOT, "paper_1112_0065_gb300", "csrc", f)
                for f in ("dedisp_kernels.cu", "tiled_tile.cuh", "tiled_launch.cuh", "tiled_g64.cu", "tc.cuh")]
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "dd_tiled_kernel_htru_1024x1500.md")
-GROUP_SRCS = [os.path.join(ROOT, "paper_1112_0065_gb300", "csrc", f) for f in ("gsum.cu", "gsum.cuh", "tma.cuh", "tc.cuh")]
+GROUP_SRCS = [os.path.join(ROOT, "paper_1112_0065_gb300", "csrc", f) for f in ("gsum.cu", "gsum.cuh", "gsum_tables.h", "tma.cuh", "tc.cuh")]
 GROUP_PROFILE = os.path.join(ROOT, "profiles", "dd_gsum_kernel_htru_1024x1500.md")
 WIDTHS = tuple(1 << k for k in range(11))
 CLF_BATCH = 32768  # snippets per classifier launch (a gulp's candidates in one launch chain)

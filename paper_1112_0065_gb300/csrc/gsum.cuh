@@ -100,9 +100,10 @@ struct Args {
 
 constexpr int kBRing = 4;  // B parts, and intervals, that warps may be apart in
 
-// Shared-memory layout in bytes: mbarriers (and the persistent kernel's tile), the two stages' channel windows, a
-// zero slot, their A parts, the B parts, the pool of vectors.
-constexpr int kTileWord = 112;
+// Shared-memory layout in bytes: mbarriers (beside them the persistent kernel's
+// tile and the number of stages issued), the two stages' channel windows, a zero
+// slot, their A parts, the B parts, the pool of vectors.
+constexpr int kTileWord = 112, kStagedWord = 120;
 static_assert((2 + 2 * kBRing) * 8 <= kTileWord, "mbarriers");
 __host__ __device__ constexpr int raw_bytes(int slot) { return (kPartChans * 4 * slot + 127) / 128 * 128; }
 __host__ __device__ constexpr int raw_at(int slot, int b) { return 128 + b * kParts * raw_bytes(slot); }
@@ -124,8 +125,8 @@ __device__ __forceinline__ uint32_t add_into(uint32_t &p, uint32_t a, uint32_t b
 // group's common start (words j and j + 1 of each), then per vector the
 // channels' extra delays and the sum of five 2-bit numbers as four planes.
 // Vectors are ordered so that neighbours often share channels 1 and 2, whose
-// part of the sum is then kept.  Called by whole warps; lanes with store =
-// false only keep in step.
+// part of the sum is then kept.  Lanes with store = false form nothing; no lane
+// needs another here.
 __device__ __forceinline__ void vectors_word(unsigned char *smem, const uint32_t *rec, int j, uint32_t half, bool store) {
     uint32_t lo[kG][2], hi[kG][2];
 #pragma unroll
@@ -142,9 +143,7 @@ __device__ __forceinline__ void vectors_word(unsigned char *smem, const uint32_t
             hi[c][i] = tiled::lop3<0xCA>(0x55555555u, x[i] >> 1, y[i]);
         }
     }
-    // a lane's own count bounds its stores, the warp's largest the loop, so that
-    // the lanes of an item that spans two groups stay together
-    const int nv = store ? (int)rec[6] : 0, most = (int)__reduce_max_sync(0xffffffffu, (unsigned)nv);
+    const int nv = store ? (int)rec[6] : 0;  // a lane's own count: those of an item may belong to two groups
     unsigned char *dst = smem + rec[5] + 16u * ((uint32_t)(j >> 1) + ((j & 1) ? half : 0u));
     half *= 32u;
     uint32_t s1 = 0, k1 = 0, s2 = 0, k2 = 0;
@@ -162,9 +161,9 @@ __device__ __forceinline__ void vectors_word(unsigned char *smem, const uint32_t
     };
     const uint4 *vec = reinterpret_cast<const uint4 *>(rec + 8);
 #pragma unroll 1
-    for (int v = 0; v < most; v += 2) {  // a pair past the last vector reads unused words of the record
+    for (int v = 0; v < nv; v += 2) {  // a pair past the last vector reads unused words of the record
         const uint4 e = vec[v >> 1];
-        one(e.x, e.y, v < nv, dst);
+        one(e.x, e.y, true, dst);
         one(e.z, e.w, v + 1 < nv, dst + half);
         dst += 2u * half;
     }
@@ -229,11 +228,12 @@ __device__ __forceinline__ void init_bars(unsigned char *smem) {
 }
 
 // One output tile: DM block dmb x time tile tt.  false (in every thread) when a
-// wait ran out of polls: the outputs are then not written and the error word
-// has bit 0 set.
+// wait ran out of polls: the outputs are then not written, the error word has
+// bit 0 set, and the mbarriers serve no further tile.
 template <int NP>
 __device__ __forceinline__ bool gsum_tile(const Args &a, int dmb, long long tt, unsigned char *smem, Phases &ph) {
     uint64_t *const full = reinterpret_cast<uint64_t *>(smem), *const formed = full + 2, *const spent = formed + kBRing;
+    volatile int &staged = *reinterpret_cast<volatile int *>(smem + kStagedWord);  // stages that the tile has issued
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const long long t0 = tt * kTile;
     const int tw0 = (int)(t0 >> 4);
@@ -256,10 +256,20 @@ __device__ __forceinline__ bool gsum_tile(const Args &a, int dmb, long long tt, 
         const uint32_t *rec = gtab + (long long)s * kRecWords;
         tc::bulk_copy_g2s(smem + a_at(a.slot, b), rec, kAWords * 4, &full[b]);
         tc::bulk_copy_g2s(smem + b_at(a.slot, s % kBRing), rec + kAWords, kBWords * 4, &full[b]);
+        staged = s + 1;
     };
-    bool ok = true;
+    // A lane whose wait runs out of polls waits no more and skips the work that
+    // follows (its sums, and the tile, are then void), but keeps step with its
+    // warp.  Lane 0 arrives for the warp, and nowhere any more once it gave up: a
+    // phase completes only when every warp's lane 0 came through its waits, so
+    // nothing is refilled while another warp reads it, no arrival counts for a
+    // later phase, and the other warps run out of polls in their turn.  (The
+    // whole warp voting after each wait: 2424 us instead of 2372 for 1024
+    // channels x 1500 trials x 131072 outputs.)
+    bool ok = true, leader = lane == 0;
     auto wait = [&](uint64_t *bar, uint32_t phase) {
         if (ok) ok = tc::mbar_wait(bar, phase & 1u, a.poll_limit);
+        leader = leader && ok;
     };
     // chunk (interval) s of this tile in the sets of kBRing
     auto number = [&](int s) { return ph.chunks + (uint32_t)s; };
@@ -288,7 +298,7 @@ __device__ __forceinline__ bool gsum_tile(const Args &a, int dmb, long long tt, 
             }
         }
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&formed[number(s) % kBRing]);
+        if (leader) tc::mbar_arrive(&formed[number(s) % kBRing]);
     };
 
     if (tid == 0)
@@ -311,9 +321,9 @@ __device__ __forceinline__ bool gsum_tile(const Args &a, int dmb, long long tt, 
     for (int k = 0; k < a.nchunks; ++k) {
         if (k + 1 < a.nchunks) form(k + 1);
         wait(&formed[number(k) % kBRing], number(k) / kBRing);
-        if (tid == 32 * (k % kWarps) && ok && k + 2 < a.nchunks)
-            stage(k + 2, reinterpret_cast<const uint32_t *>(smem + a_at(a.slot, k & 1)) + 3, kPartWords);
         if (ok) {
+            if (tid == 32 * (k % kWarps) && k + 2 < a.nchunks)
+                stage(k + 2, reinterpret_cast<const uint32_t *>(smem + a_at(a.slot, k & 1)) + 3, kPartWords);
             // the chunk's four groups in a carry-save tree; the trees of two
             // chunks are joined and rippled into the upper planes
             const uint4 *bt = reinterpret_cast<const uint4 *>(smem + b_at(a.slot, k % kBRing)) + warp;
@@ -360,15 +370,17 @@ __device__ __forceinline__ bool gsum_tile(const Args &a, int dmb, long long tt, 
             }
         }
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(&spent[number(k) % kBRing]);
+        if (leader) tc::mbar_arrive(&spent[number(k) % kBRing]);
     }
+    const uint32_t first = ph.chunks;
     ph.chunks += (uint32_t)a.nchunks;
     if (__syncthreads_or(!ok)) {
-        // a stage or an interval never completed: record it, give the stages'
-        // last copies one more short bounded wait, and leave the outputs alone
+        // a stage or an interval never completed: record it, give the last two
+        // stages' copies one more short bounded wait, and leave the outputs alone
         if (tid == 0) atomicOr(a.err, 1u);
         const uint32_t last = a.poll_limit / 64 + 1;
-        for (int b = 0; b < 2; ++b) tc::mbar_wait(&full[b], (ph.chunks / 2 - 1) & 1u, last);
+        for (int s = staged - 2; s < staged; ++s)
+            tc::mbar_wait(&full[s & 1], ((first >> 1) + ((uint32_t)s >> 1)) & 1u, last);
         return false;
     }
 

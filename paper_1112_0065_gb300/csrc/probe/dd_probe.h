@@ -70,6 +70,21 @@ dd_status dd_probe_wait_giveup(unsigned poll_limit, unsigned *h_status);
  */
 dd_status dd_probe_tile_giveup(unsigned poll_limit, unsigned *h_err, long long *h_written);
 
+/*
+ * The give-up paths of the channel-group tile's bounded waits, likewise: one
+ * CTA dedisperses a 64-channel, 32-trial, 2048-sample tile (its delays give 20
+ * vectors per group, so that a chunk waits for the place of the chunk two
+ * before it).  withheld: 1 the mbarriers of the stages, 2 of the chunks formed,
+ * 3 of the chunks spent expect one arrival more than is made, so that no such
+ * phase completes; 0 none does, and the tile runs to its end.  Every wait stops
+ * after poll_limit polls (1..2^20).  h_in (64 rows of 528 bytes) is the packed
+ * input, h_delays (32 x 64) receives the delays and h_out (32 x 2048) the
+ * output, preset to 0xFFFFFFFF; *h_err the tile's error word.  Synchronous;
+ * DD_ERR_TIMEOUT when the tile gave up, DD_OK when it did not.
+ */
+dd_status dd_probe_group_tile(int withheld, unsigned poll_limit, const uint8_t *h_in, int32_t *h_delays,
+                              uint32_t *h_out, unsigned *h_err);
+
 /* Message of the calling thread's last failed probe call ("" if none). */
 const char *dd_probe_last_error(void);
 

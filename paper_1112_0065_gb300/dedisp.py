@@ -137,9 +137,9 @@ class Plan:
 
 
 def dedisp_status() -> int:
-    """Device error flags of the tiled dedispersion kernels on the current
-    device, read and cleared (bit 0: a tile stopped waiting for its staged
-    input and left its outputs unwritten).  Synchronises the device."""
+    """Device error flags of the dedispersion kernels (tiled and channel-group)
+    on the current device, read and cleared (bit 0: a tile stopped waiting for
+    its staged input or its warps' shares and left its outputs unwritten).  Synchronises the device."""
     L = _lib.load()
     f = ctypes.c_uint()
     _lib.check(L.dd_dedisp_status(ctypes.byref(f)), "dd_dedisp_status")

@@ -27,6 +27,7 @@ SIGNATURES = {
     "dd_probe_tc_gemm": (_I, [_P, _P, _P, _I, _I]),
     "dd_probe_wait_giveup": (_I, [ctypes.c_uint, ctypes.POINTER(ctypes.c_uint)]),
     "dd_probe_tile_giveup": (_I, [ctypes.c_uint, ctypes.POINTER(ctypes.c_uint), ctypes.POINTER(ctypes.c_longlong)]),
+    "dd_probe_group_tile": (_I, [_I, ctypes.c_uint, _P, _P, _P, ctypes.POINTER(ctypes.c_uint)]),
     "dd_probe_last_error": (ctypes.c_char_p, []),
 }
 
@@ -103,3 +104,23 @@ def tile_giveup(poll_limit: int = 1000):
     st = L.dd_probe_tile_giveup(int(poll_limit), ctypes.byref(err), ctypes.byref(written))
     msg = L.dd_probe_last_error()
     return st, err.value, written.value, msg.decode() if msg else ""
+
+
+GROUP_TILE_BYTES = 528  # bytes of a row of group_tile's input (2048 samples and 15 of delay, in 16-byte groups)
+
+
+def group_tile(packed, withheld: int = 0, poll_limit: int = 1000):
+    """Run one channel-group tile on packed input (uint8 [64, GROUP_TILE_BYTES])
+    with the completions of its stages (1), formed chunks (2), spent chunks (3)
+    or of nothing (0) withheld: -> (status code, the tile's error word, its
+    delays [32, 64], its output [32, 2048], message)."""
+    packed = np.ascontiguousarray(packed, dtype=np.uint8)
+    assert packed.shape == (64, GROUP_TILE_BYTES)
+    delays = np.empty((32, 64), dtype=np.int32)
+    out = np.empty((32, 2048), dtype=np.uint32)
+    err = ctypes.c_uint()
+    L = load()
+    st = L.dd_probe_group_tile(int(withheld), int(poll_limit), packed.ctypes.data, delays.ctypes.data, out.ctypes.data,
+                               ctypes.byref(err))
+    msg = L.dd_probe_last_error()
+    return st, err.value, delays, out, msg.decode() if msg else ""

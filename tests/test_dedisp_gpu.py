@@ -376,6 +376,32 @@ def test_tile_gives_up_without_fault(P):
     plan.close()
 
 
+@pytest.mark.parametrize("withheld", [1, 2, 3, 0])
+def test_group_tile_gives_up_without_fault(P, withheld):
+    """The give-up paths of the channel-group tile's three kinds of waits (a
+    stage that arrived, a chunk that all have formed, a place that all have
+    spent), run without any fault: with one arrival of the kind withheld the
+    tile ends within its polls, sets bit 0 of its error word and writes no
+    output; with none withheld the same tile gives the oracle's sums, and so
+    does a dedispersion afterwards, the library's own error word clear."""
+    from paper_1112_0065_gb300 import probes
+
+    rng = np.random.default_rng(withheld)
+    packed = rng.integers(0, 256, (64, probes.GROUP_TILE_BYTES), dtype=np.uint8)
+    st, err, delays, out, msg = probes.group_tile(packed, withheld)
+    if withheld:
+        assert st == -5 and err == 1 and "gave up" in msg, (st, err, msg)
+        assert bool((out == 0xFFFFFFFF).all())
+    else:
+        assert st == 0 and err == 0, (st, err, msg)
+        np.testing.assert_array_equal(out, oracle.dedisperse(delays, packed, 2048 + 15))
+    assert P.dedisp_status() == 0
+    f, dms, delays, packed, nsamp = tiny_config()
+    plan = P.Plan(f, 64e-6, dms)
+    np.testing.assert_array_equal(_run(P, plan, packed, nsamp), oracle.dedisperse(delays, packed, nsamp))
+    plan.close()
+
+
 # gulps long enough for the automatic choice to leave the tiled kernel:
 # (nchan, trials, last DM, outputs): partial groups and chunks of channels,
 # blocks of trials (32) and tiles (2048 outputs), the last channel counts of
