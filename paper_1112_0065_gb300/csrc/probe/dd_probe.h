@@ -60,15 +60,17 @@ dd_status dd_probe_wait_giveup(unsigned poll_limit, unsigned *h_status);
 
 /*
  * The give-up path of the dedispersion tile's bounded stage waits, run
- * without any fault (no paper counterpart): one CTA dedisperses a 64-channel,
- * 16-trial, 1536-sample tile whose stage mbarriers expect one arrival more
- * than the stage copies make, so no stage ever completes; every wait stops
- * after poll_limit polls (1..2^20).  *h_err receives the tile's error word
+ * without any fault (no paper counterpart): one CTA dedisperses a 192-channel,
+ * 16-trial, 1536-sample tile in three stages whose mbarriers expect one arrival
+ * more than the stage copies make, so no stage ever completes; the first wait
+ * stops after poll_limit polls (1..2^20).  *h_err receives the tile's error word
  * (bit 0: gave up), *h_written the number of output words the tile wrote
- * (expected 0).  Synchronous; DD_ERR_TIMEOUT when the tile gave up (always, by
- * construction), DD_ERR_INVALID_ARG for bad arguments.
+ * (expected 0), *h_restaged 1 if the third stage was copied over the first,
+ * which never counted as arrived (expected 0).  Synchronous; DD_ERR_TIMEOUT
+ * when the tile gave up (always, by construction), DD_ERR_INVALID_ARG for bad
+ * arguments.
  */
-dd_status dd_probe_tile_giveup(unsigned poll_limit, unsigned *h_err, long long *h_written);
+dd_status dd_probe_tile_giveup(unsigned poll_limit, unsigned *h_err, long long *h_written, int *h_restaged);
 
 /*
  * The give-up paths of the channel-group tile's bounded waits, likewise: one

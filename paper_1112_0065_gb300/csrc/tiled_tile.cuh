@@ -201,9 +201,10 @@ __device__ __forceinline__ void tile_init_bars(uint32_t *smem) {
 // tile_smem_bytes() with its mbarriers initialised by tile_init_bars; bit b
 // of `phase` is the parity of stage buffer b's next completion and carries
 // over to the CTA's next tile.  Returns false (in every thread) when a stage
-// never arrived within the poll limit; the tile's outputs are then not
-// written and the error word has bit 0 set.  The caller synchronises the
-// block before reusing the shared memory.
+// never arrived within the poll limit; no further stage is then copied, the
+// tile's outputs are not written, the error word has bit 0 set and the
+// mbarriers serve no further tile.  The caller synchronises the block before
+// reusing the shared memory.
 template <int DT, int W, int NP, int G>
 __device__ __forceinline__ bool dd_tile(const TiledArgs &a, int dmb, long long tt, uint32_t *smem, uint32_t &phase) {
     constexpr int D = kWarps * DT;
@@ -274,39 +275,41 @@ __device__ __forceinline__ bool dd_tile(const TiledArgs &a, int dmb, long long t
 #pragma unroll
             for (int k = 0; k < NP; ++k) P[jj][i][k] = 0u;
 
-    bool ok = true;
     stage(0, 0);
     for (int k = 0; k < nchunks; ++k) {
         if (k + 1 < nchunks) stage(k + 1, (k + 1) & 1);
-        // stage k is in once its mbarrier completes the phase of this use
+        // stage k is in once its mbarrier completes the phase of this use; a
+        // stage that is not in is not read (its table's offsets could be anything)
         const int b = k & 1;
-        if (ok) ok = tc::mbar_wait(&s_bar[b], (phase >> b) & 1u, a.poll_limit);
+        const bool in = tc::mbar_wait(&s_bar[b], (phase >> b) & 1u, a.poll_limit);
         phase ^= 1u << b;
-        Ctx<DT, W> x{reinterpret_cast<const char *>(s_win0 + (k & 1) * stage_words + LaneWords<W>::first(lane)),
-                     s_tab0 + (k & 1) * (G * D), warp * DT};
-        uint32_t cg[DT][W];
-        hs<LG>(x, P, cg, 0);
-        // ripple the weight-G carry into the upper planes
+        if (in) {
+            Ctx<DT, W> x{reinterpret_cast<const char *>(s_win0 + (k & 1) * stage_words + LaneWords<W>::first(lane)),
+                         s_tab0 + (k & 1) * (G * D), warp * DT};
+            uint32_t cg[DT][W];
+            hs<LG>(x, P, cg, 0);
+            // ripple the weight-G carry into the upper planes
 #pragma unroll
-        for (int jj = 0; jj < DT; ++jj)
+            for (int jj = 0; jj < DT; ++jj)
 #pragma unroll
-            for (int i = 0; i < W; ++i) {
-                uint32_t c = cg[jj][i];
+                for (int i = 0; i < W; ++i) {
+                    uint32_t c = cg[jj][i];
 #pragma unroll
-                for (int l = LG; l < NP; ++l) {
-                    const uint32_t s = P[jj][i][l] ^ c;
-                    c &= P[jj][i][l];
-                    P[jj][i][l] = s;
+                    for (int l = LG; l < NP; ++l) {
+                        const uint32_t s = P[jj][i][l] ^ c;
+                        c &= P[jj][i][l];
+                        P[jj][i][l] = s;
+                    }
                 }
-            }
-        __syncthreads();
-    }
-    if (__syncthreads_or(!ok)) {
-        // a stage never arrived: record it, give both buffers' last copies
-        // one more short bounded wait, and leave the outputs alone
+        }
+        if (!__syncthreads_or(!in)) continue;
+        // a stage never arrived: record it, give the copies on their way (this
+        // stage's and the next one's) one more short bounded wait, and leave the
+        // outputs alone
         if (threadIdx.x == 0) atomicOr(a.err, 1u);
         const uint32_t last = a.poll_limit / 64 + 1;
-        for (int b = 0; b < 2; ++b) tc::mbar_wait(&s_bar[b], ((phase >> b) & 1u) ^ 1u, last);
+        tc::mbar_wait(&s_bar[b], ((phase >> b) & 1u) ^ 1u, last);
+        if (k + 1 < nchunks) tc::mbar_wait(&s_bar[b ^ 1], (phase >> (b ^ 1)) & 1u, last);
         return false;
     }
 

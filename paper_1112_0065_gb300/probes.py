@@ -26,7 +26,8 @@ SIGNATURES = {
     "dd_probe_fp_rates": (_I, [_P, _P]),
     "dd_probe_tc_gemm": (_I, [_P, _P, _P, _I, _I]),
     "dd_probe_wait_giveup": (_I, [ctypes.c_uint, ctypes.POINTER(ctypes.c_uint)]),
-    "dd_probe_tile_giveup": (_I, [ctypes.c_uint, ctypes.POINTER(ctypes.c_uint), ctypes.POINTER(ctypes.c_longlong)]),
+    "dd_probe_tile_giveup": (_I, [ctypes.c_uint, ctypes.POINTER(ctypes.c_uint), ctypes.POINTER(ctypes.c_longlong),
+                                  ctypes.POINTER(_I)]),
     "dd_probe_group_tile": (_I, [_I, ctypes.c_uint, _P, _P, _P, ctypes.POINTER(ctypes.c_uint)]),
     "dd_probe_last_error": (ctypes.c_char_p, []),
 }
@@ -95,15 +96,26 @@ def wait_giveup(poll_limit: int = 1000):
     return st, flags.value, msg.decode() if msg else ""
 
 
+def _tile_giveup(poll_limit):
+    err = ctypes.c_uint()
+    written = ctypes.c_longlong()
+    restaged = ctypes.c_int()
+    L = load()
+    st = L.dd_probe_tile_giveup(int(poll_limit), ctypes.byref(err), ctypes.byref(written), ctypes.byref(restaged))
+    msg = L.dd_probe_last_error()
+    return st, err.value, written.value, restaged.value, msg.decode() if msg else ""
+
+
 def tile_giveup(poll_limit: int = 1000):
     """Run the dedispersion tile with stage waits that cannot complete: ->
     (status code, the tile's error word, output words it wrote, message)."""
-    err = ctypes.c_uint()
-    written = ctypes.c_longlong()
-    L = load()
-    st = L.dd_probe_tile_giveup(int(poll_limit), ctypes.byref(err), ctypes.byref(written))
-    msg = L.dd_probe_last_error()
-    return st, err.value, written.value, msg.decode() if msg else ""
+    st, err, written, _, msg = _tile_giveup(poll_limit)
+    return st, err, written, msg
+
+
+def tile_restages(poll_limit: int = 1000) -> bool:
+    """Whether that tile copies a stage over one that never counted as arrived."""
+    return bool(_tile_giveup(poll_limit)[3])
 
 
 GROUP_TILE_BYTES = 528  # bytes of a row of group_tile's input (2048 samples and 15 of delay, in 16-byte groups)

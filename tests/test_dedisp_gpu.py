@@ -376,6 +376,16 @@ def test_tile_gives_up_without_fault(P):
     plan.close()
 
 
+def test_tile_stages_nothing_after_giving_up(P):
+    """A tile whose first of three stages never counts as arrived stops there:
+    the third stage is not copied over it (nor is the stage read, whose table of
+    shared-memory offsets is not known to be there)."""
+    from paper_1112_0065_gb300 import probes
+
+    assert not probes.tile_restages(1000)
+    assert P.dedisp_status() == 0
+
+
 @pytest.mark.parametrize("withheld", [1, 2, 3, 0])
 def test_group_tile_gives_up_without_fault(P, withheld):
     """The give-up paths of the channel-group tile's three kinds of waits (a
