@@ -957,8 +957,10 @@ __global__ void __launch_bounds__(256) fc1_bwd_x_kernel(const float *__restrict_
 }
 
 // Gradient of a convolution's pooled output routed to the one position of
-// each 2x2 window that pooling kept (0 elsewhere, and 0 where the ReLU cut).
-__device__ __forceinline__ float live_grad(float d, uint16_t pooled) { return bf2f(pooled) > 0.0f ? d : 0.0f; }
+// each 2x2 window that pooling kept (0 elsewhere, and 0 where the ReLU cut: a
+// dead window).
+__device__ __forceinline__ bool live(uint16_t pooled) { return bf2f(pooled) > 0.0f; }
+__device__ __forceinline__ float live_grad(float d, uint16_t pooled) { return live(pooled) ? d : 0.0f; }
 
 // Input gradient of a 3x3 convolution: din[n][ci] = sum over (co, taps) of the
 // routed output gradient times the flipped weights, a convolution over CO
@@ -1118,7 +1120,9 @@ __global__ void __launch_bounds__((ConvBwdXCfg<CI, CO, H>::THREADS))
 // that pooling kept and the 3x3 input patch around it: a quarter of the dense
 // multiply-adds.  A sample's input sits in shared memory channel-last with a
 // zero border (a lane's 4 channels are one 8-byte load, the lanes of one
-// output channel consecutive), its (gradient, patch offset) pairs beside it.
+// output channel consecutive), its (gradient, patch offset) pairs beside it.  A
+// dead window's patch is one of zeros past the bottom border: its gradient of 0
+// times an infinite or NaN input would be NaN.
 // A block walks samples blockIdx.x, + gridDim.x, ...; its sums (SL window
 // slices joined in order) are one partial, and conv_bwd_w_sum_kernel adds the
 // partials in order, so the result is deterministic.  Issue-bound: about 64
@@ -1132,7 +1136,8 @@ struct ConvBwdWCfg {
     static constexpr int THREADS = SL * COB * CQ;
     static constexpr int GS = NWIN + 1;              // padded row of (gradient, offset) pairs
     static constexpr int PIX = CI * 2;               // bytes of a pixel
-    static constexpr int IN_BYTES = (H + 2) * (H + 2) * PIX;
+    static constexpr int ZERO_PATCH = (H + 1) * (H + 2) * PIX;  // rows H+1 (the border) .. H+3, 3 pixels each
+    static constexpr int IN_BYTES = (((H + 3) * (H + 2) + 3) * PIX + 15) / 16 * 16;
     static constexpr int RED_BYTES = SL > 1 ? (SL - 1) * COB * CQ * 37 * 4 : 0;  // slices' sums, in the pairs' place
     static constexpr int GP_BYTES = COB * GS * 8;
     static constexpr size_t SMEM = (size_t)IN_BYTES + (GP_BYTES > RED_BYTES ? GP_BYTES : RED_BYTES);
@@ -1179,9 +1184,11 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
             const int k = e % C::NWIN, c = e / C::NWIN;
             const long long o = ((long long)n * CO + co0 + c) * C::NWIN + k;
             const int a = __ldg(arg + o);
+            const bool on = live(__ldg(pooled + o));
             // patch around (2 yo + a/2, 2 xo + a%2): its corner in padded coordinates is that position
             const int off = ((2 * (k / HO) + (a >> 1)) * (H + 2) + 2 * (k % HO) + (a & 1)) * C::PIX;
-            gp[c * C::GS + k] = make_uint2(__float_as_uint(live_grad(__ldg(dpool + o), __ldg(pooled + o))), (uint32_t)off);
+            const float d = __ldg(dpool + o);
+            gp[c * C::GS + k] = make_uint2(on ? __float_as_uint(d) : 0u, (uint32_t)(on ? off : C::ZERO_PATCH));
         }
         __syncthreads();
         const uint2 *g = gp + co * C::GS + sl * (C::NWIN / SL);
@@ -1235,16 +1242,17 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
 
 // The first layer (one input channel): warp w owns output channel w, its lanes
 // the windows of a row, 9 sums each; the sample's image sits in shared memory
-// as float with a zero border.
+// as float with a zero border, past it the zeros that dead windows read (as
+// conv_bwd_w_kernel).
 __global__ void __launch_bounds__(512) conv0_bwd_w_kernel(const float *__restrict__ dpool,
                                                           const uint16_t *__restrict__ pooled,
                                                           const uint8_t *__restrict__ arg,
                                                           const uint16_t *__restrict__ in, int N,
                                                           float *__restrict__ partial) {
     constexpr int H = 64, HO = 32, CO = 16, RS = H + 2;
-    __shared__ float img[RS * RS];
+    __shared__ float img[(RS + 1) * RS + 3];  // rows H+1 (the border) .. H+3 of zeros, 3 pixels in the last
     const int tid = threadIdx.x, co = tid >> 5, lane = tid & 31;
-    for (int i = tid; i < RS * RS; i += 512) img[i] = 0.0f;
+    for (int i = tid; i < (RS + 1) * RS + 3; i += 512) img[i] = 0.0f;
     float acc[10] = {};  // 9 taps and the bias
 #pragma unroll 1
     for (int n = blockIdx.x; n < N; n += gridDim.x) {
@@ -1262,8 +1270,9 @@ __global__ void __launch_bounds__(512) conv0_bwd_w_kernel(const float *__restric
 #pragma unroll 4
         for (int yo = 0; yo < HO; ++yo) {
             const int a = __ldg(arg + o + yo * HO);
-            const float g = live_grad(__ldg(dpool + o + yo * HO), __ldg(pooled + o + yo * HO));
-            const float *px = img + (2 * yo + (a >> 1)) * RS + 2 * lane + (a & 1);
+            const bool on = live(__ldg(pooled + o + yo * HO));
+            const float d = __ldg(dpool + o + yo * HO), g = on ? d : 0.0f;
+            const float *px = img + (on ? (2 * yo + (a >> 1)) * RS + 2 * lane + (a & 1) : (H + 1) * RS);
 #pragma unroll
             for (int t = 0; t < 9; ++t) acc[t] = fmaf(g, px[(t / 3) * RS + t % 3], acc[t]);
             acc[9] += g;

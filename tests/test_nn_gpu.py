@@ -282,3 +282,29 @@ def test_backward_of_a_batch_is_the_mean_of_its_halves(P):
         got.append(c.grads().astype(np.float64))
     want = 0.5 * (got[1] + got[2])
     assert float(np.abs(got[0] - want).max()) <= 1e-5 * float(np.abs(want).max())
+
+
+@pytest.mark.parametrize("value", [float("nan"), float("inf"), -float("inf")])
+def test_backward_with_a_bad_pixel(P, value):
+    """A pixel that is not a finite number kills the windows over it (the ReLU of
+    a NaN is 0), and dead windows contribute nothing: the weight gradients are
+    finite where the oracle's are, and equal to them there as everywhere else."""
+    import torch
+
+    n = 6
+    p = params_with_biases(P, 4)
+    x = snippets(31, n).copy()
+    bits = np.float32(value).view(np.uint32) >> 16
+    x[1, 20, 33] = bits
+    x[4, 0, 63] = bits
+    y = (np.arange(n) % 2).astype(np.float32)
+    c = P.Classifier(max_batch=n, params=p)
+    c.backward(to_dev(x), torch.from_numpy(y).cuda())
+    loss_or, g_or, _ = oracle.nn_backward(p, x, y, round_bf16=True)
+    got = c.grads()
+    finite = np.isfinite(g_or)
+    assert bool(finite.all()) == np.isnan(value)
+    np.testing.assert_array_equal(np.isfinite(got), finite)
+    np.testing.assert_array_equal(got[~finite], g_or[~finite])
+    assert float(np.abs(got - g_or)[finite].max()) <= 1e-4 * float(np.abs(g_or[finite]).max())
+    assert abs(c.loss() - loss_or) <= 1e-6 * max(1.0, abs(loss_or))
