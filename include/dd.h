@@ -124,7 +124,9 @@ dd_status dd_plan_kernel_shape(const dd_plan *plan, int *kernel, int *dms_per_bl
  * candidate tile shapes -- DM trials per CTA x 16-sample words per thread (8
  * pairs) x channels per shared-memory stage (32, 64, 128) -- on `stream` with
  * scratch buffers it allocates and frees, keeps the fastest, and writes it to
- * opt->tune_cache_path if one was given at plan creation.  The tables of the
+ * opt->tune_cache_path if one was given at plan creation.  Where the plan would
+ * take the channel-group kernel it is timed beside them; if it loses, gulps of
+ * this length and shorter ones run the tiled kernel.  The tables of the
  * other shapes are freed, unless a batch built on this plan still points at
  * them (they then live until dd_destroy).  Synchronous.  Returns the best
  * time in *best_ms (0 when the shape came from the cache).

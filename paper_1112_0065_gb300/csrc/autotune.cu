@@ -30,7 +30,7 @@ static std::string cache_key(const Plan *p, size_t nsamp_in) {
     return key;
 }
 
-static bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out, bool *gsum_off) {
+static bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out, bool *tiled_won) {
     if (p->tune_cache.empty()) return false;
     std::lock_guard<std::mutex> g(g_cache_mutex);
     FILE *f = fopen(p->tune_cache.c_str(), "r");
@@ -44,11 +44,11 @@ static bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out, bool *
         *bar = 0;
         if (key == line) {
             TiledShape s;
-            int tiled_won = 0;  // absent in files written before the channel-group kernel
-            if (sscanf(bar + 1, "%d %d %d %d", &s.dms_per_warp, &s.words_per_lane, &s.chan_chunk, &tiled_won) >= 3 &&
+            int won = 0;  // absent in files written before the channel-group kernel
+            if (sscanf(bar + 1, "%d %d %d %d", &s.dms_per_warp, &s.words_per_lane, &s.chan_chunk, &won) >= 3 &&
                 tiled_shape_supported(s)) {
                 *out = s;
-                *gsum_off = tiled_won != 0;
+                *tiled_won = won != 0;
                 found = true;
             }
         }
@@ -57,13 +57,13 @@ static bool cache_lookup(const Plan *p, size_t nsamp_in, TiledShape *out, bool *
     return found;
 }
 
-static void cache_store(const Plan *p, size_t nsamp_in, const TiledShape &s, bool gsum_off) {
+static void cache_store(const Plan *p, size_t nsamp_in, const TiledShape &s, bool tiled_won) {
     if (p->tune_cache.empty()) return;
     std::lock_guard<std::mutex> g(g_cache_mutex);
     FILE *f = fopen(p->tune_cache.c_str(), "a");
     if (!f) return;
     fprintf(f, "%s|%d %d %d %d\n", cache_key(p, nsamp_in).c_str(), s.dms_per_warp, s.words_per_lane, s.chan_chunk,
-            gsum_off ? 1 : 0);
+            tiled_won ? 1 : 0);
     fclose(f);
 }
 
@@ -77,11 +77,11 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     if (nsamp_in <= (size_t)p->maxdelay) return fail(DD_ERR_TOO_SHORT, "gulp shorter than the maximum delay");
     if (p->kernel == DD_KERNEL_SIMPLE) return fail(DD_ERR_INVALID_ARG, "plan uses the simple kernel");
     TiledShape cached;
-    bool gsum_off = false;
-    if (cache_lookup(p, nsamp_in, &cached, &gsum_off) && ensure_shape_table(p, cached) == DD_OK) {
+    bool tiled_won = false;
+    if (cache_lookup(p, nsamp_in, &cached, &tiled_won) && ensure_shape_table(p, cached) == DD_OK) {
         p->shape = cached;
         p->narrow_sms = 0;
-        p->gs.off = gsum_off;
+        p->gs.tiled_to = tiled_won ? (long long)nsamp_in - p->maxdelay : 0;
         if (best_ms) *best_ms = 0.0f;
         return DD_OK;
     }
@@ -127,15 +127,16 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
     // the channel-group kernel, where the plan would take it for this gulp
     const Plan *self = p;
     const long long outputs = (long long)nout;
-    const bool was_off = p->gs.off;
-    p->gs.off = false;
+    const long long tiled_before = p->gs.tiled_to;
+    p->gs.tiled_to = 0;
     if (st == DD_OK && use_gsum(&self, &outputs, 1)) {
         float ms = 0.f;
         st = timed([&] { return launch_gsum(p, in, ld_in, nsamp_in, out, ld_out, s); }, ms);
-        p->gs.off = st == DD_OK && ms > best;
+        tiled_won = st == DD_OK && ms > best;
+        if (tiled_won) p->gs.tiled_to = outputs;
         if (st == DD_OK && ms < best) best = ms;
     }
-    if (st != DD_OK) p->gs.off = was_off;
+    if (st != DD_OK) p->gs.tiled_to = tiled_before;
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (in) cudaFree(in);
@@ -154,7 +155,7 @@ extern "C" dd_status dd_plan_autotune(dd_plan *plan, size_t nsamp_in, void *stre
             ++it;
         }
     }
-    cache_store(p, nsamp_in, best_shape, p->gs.off);
+    cache_store(p, nsamp_in, best_shape, tiled_won);
     if (best_ms) *best_ms = best;
     return DD_OK;
 }

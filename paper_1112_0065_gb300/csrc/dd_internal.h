@@ -53,7 +53,7 @@ struct ShapeTable {
 // suit it (few distinct combinations, everything fits in shared memory).
 struct GsumTable {
     bool ok = false;
-    bool off = false;        // the autotuner measured the tiled kernel faster
+    long long tiled_to = 0;  // the autotuner measured the tiled kernel faster on a gulp of so many outputs
     uint32_t *tab = nullptr;
     int32_t *ws = nullptr;
     int n_dmb = 0, nchunks = 0, slot = 0, sms = 0;

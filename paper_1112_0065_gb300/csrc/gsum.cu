@@ -91,7 +91,8 @@ void free_gsum(Plan *p) {
 // 4 % over 20 to 2048 channels, 24 to 1500 trials and 2000 to 131072 outputs,
 // and what they leave out, some 8 us of launch and first copies, is the same.
 // A gulp too short to fill the waves stays on the tiled kernel, whose tiles are
-// smaller.  Measured, tiled / here, in us: 1024 channels x 1500 trials x 6208
+// smaller; so does one no longer than a gulp on which the autotuner measured the
+// tiled kernel faster (longer ones fill the waves better and keep to the rule).  Measured, tiled / here, in us: 1024 channels x 1500 trials x 6208
 // outputs 214 / 236, x 10000 267 / 243, x 131072 2778 / 2372; 1024 x 64 x 40000
 // 64 / 111, x 131072 165 / 111; 2048 x 700 x 131072 2783 / 2069; 1024 x 1000
 // linear trials to DM 1000 (many vectors) x 20000 320 / 390, x 131072 1861 /
@@ -101,7 +102,7 @@ bool use_gsum(const Plan *const *p, const long long *nout, int n) {
     double tiles = 0, work = 0, tiles16 = 0, work16 = 0;
     for (int i = 0; i < n; ++i) {
         const GsumTable &t = p[i]->gs;
-        if (!t.ok || t.off || gsum_big(p[i]) != gsum_big(p[0])) return false;
+        if (!t.ok || nout[i] <= t.tiled_to || gsum_big(p[i]) != gsum_big(p[0])) return false;
         const double m = (double)((nout[i] + kTile - 1) / kTile) * t.n_dmb;
         tiles += m;
         work += m * t.tile_cycles;

@@ -343,6 +343,35 @@ def test_autotune_cache_round_trip(P, tmp_path):
     np.testing.assert_array_equal(_run(P, b, packed, nsamp), oracle.dedisperse(delays, packed, nsamp))
 
 
+def test_lost_tuning_race_holds_for_that_length_only(P, tmp_path):
+    """A cache line that says the tiled kernel won (its fourth number) keeps
+    gulps of that length and shorter ones on the tiled kernel; longer ones stay
+    with the channel-group kernel, and both give the same sums."""
+    import torch
+
+    f = synth.band_freqs(96)
+    dms = synth.dm_list_linear(1500, 60.0)
+    cache = str(tmp_path / "tune.txt")
+    first = P.Plan(f, 64e-6, dms, tune_cache=cache)
+    short, long = 20000 + first.maxdelay, 60000 + first.maxdelay
+    assert first.uses_channel_groups(short) and first.uses_channel_groups(long)
+    first.autotune(short)
+    with open(cache) as fh:
+        key, choice = fh.read().strip().split("|")
+    with open(cache, "w") as fh:
+        fh.write(f"{key}|{' '.join(choice.split()[:3])} 1\n")
+    plan = P.Plan(f, 64e-6, dms, tune_cache=cache)
+    assert plan.autotune(short) == 0.0
+    assert not plan.uses_channel_groups(short) and not plan.uses_channel_groups(short - 1000)
+    assert plan.uses_channel_groups(long) and plan.uses_channel_groups(short + 2048)
+    tiled = P.Plan(f, 64e-6, dms, kernel=P.KERNEL_TILED)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randint(0, 256, (96, P.row_bytes(long)), dtype=torch.uint8, device="cuda", generator=gen)
+    for nsamp in (short, long):
+        n = plan.nout(nsamp)
+        assert bool((plan.execute(x, nsamp)[:, :n] == tiled.execute(x, nsamp)[:, :n]).all())
+
+
 def test_stage_waits_report_no_error(P):
     """The tiled kernels stage each channel window by a bulk copy whose
     completion every thread waits for with a bounded poll: after this
