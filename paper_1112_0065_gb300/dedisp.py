@@ -18,11 +18,15 @@ def _f64(a):
 
 def _stream_handle(stream):
     if stream is None:
-        # the current stream's handle without the Stream object around it,
-        # which took 2.8 us of a short gulp's 13 on the Grace host
         import torch
 
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        # the current stream's handle without the Stream object around it,
+        # which took 2.8 us of a short gulp's 13 on the Grace host; PyTorch
+        # promises only the object
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return torch.cuda.current_stream().cuda_stream
+        return raw(torch.cuda.current_device())
     return stream.cuda_stream
 
 
