@@ -211,13 +211,14 @@ dd_status dd_plan_create(dd_plan **out, int nchan, const double *freqs_mhz, doub
         }
     }
     // the channel-group kernel and the narrow shape for automatic plans (a given
-    // shape asks for that one); with more than 304 trials only gulps of 6000
-    // outputs and fewer would be narrow, not worth the tables
+    // shape asks for that one); with more than two trials per SM (304) only gulps
+    // of four tiles (6000 outputs) and fewer would be narrow, not worth the tables
     if (p->kernel == DD_KERNEL_AUTO && !(o.dms_per_block || o.words_per_thread || o.chan_chunk)) {
         build_gsum(p);
-        if (ndm <= 304 && ensure_shape_table(p, kNarrowShape) == DD_OK &&
-            cudaDeviceGetAttribute(&p->narrow_sms, cudaDevAttrMultiProcessorCount, p->device) != cudaSuccess)
-            p->narrow_sms = 0;
+        int sms = 0;
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device) == cudaSuccess && ndm <= 2 * sms &&
+            ensure_shape_table(p, kNarrowShape) == DD_OK)
+            p->narrow_sms = sms;
         cudaGetLastError();  // without memory for the tables the default shape serves
     }
     *out = reinterpret_cast<dd_plan *>(p);

@@ -36,7 +36,9 @@ constexpr int kCin[kConvLayers] = {1, 16, 32, 64};
 constexpr int kCout[kConvLayers] = {16, 32, 64, 64};
 constexpr int kHin[kConvLayers] = {64, 32, 16, 8};
 constexpr int kFcIn = 1024, kFcHid = 128;
-constexpr int kMaxPartials = 304;  // blocks (= partials) of a convolution's weight gradient: two per SM
+// Blocks (= partials) of a convolution's weight gradient: two per SM of a GB300.
+// A fixed number, so that the order of the sums is the same on every device.
+constexpr int kMaxPartials = 304;
 
 struct Layout {
     long long cw[kConvLayers], cb[kConvLayers], f1w, f1b, f2w, f2b, total;

@@ -227,7 +227,7 @@ __global__ void __launch_bounds__(256) dd_rfi_apply_kernel(const BeamPtrs beams,
 }
 
 struct Rfi {
-    int nbeams_max = 0, nchan = 0;
+    int nbeams_max = 0, nchan = 0, sms = 0;
     long long nsamp_max = 0, ldz = 0;
     uint32_t *z = nullptr;                // [nbeams_max][ldz] zero-DM series
     unsigned long long *stats = nullptr;  // [nbeams_max][2]: sum z, sum z^2; then the masked count and the list length
@@ -265,7 +265,10 @@ dd_status dd_rfi_create(dd_rfi **out, int nbeams_max, int nchan, size_t nsamp_ma
     r->nchan = nchan;
     r->nsamp_max = (long long)nsamp_max;
     r->ldz = ((long long)nsamp_max + 15) / 16 * 16;
-    cudaError_t e = cudaMalloc(&r->z, (size_t)nbeams_max * r->ldz * 4);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&r->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMalloc(&r->z, (size_t)nbeams_max * r->ldz * 4);
     if (e == cudaSuccess) e = cudaMalloc(&r->stats, ((size_t)2 * nbeams_max + 2) * 8);
     if (e == cudaSuccess) e = cudaMalloc(&r->mask, (size_t)r->ldz);
     if (e == cudaSuccess) e = cudaMalloc(&r->list, (size_t)(r->ldz / 16) * sizeof(uint2));
@@ -305,7 +308,7 @@ dd_status dd_rfi_run(dd_rfi *rfi, uint8_t *const *d_in, int nbeams, size_t ld_in
         r->z, r->ldz, nbeams, (long long)nsamp, r->stats, k_sigma, min_beams, r->mask, r->stats + 2 * nbeams,
         r->stats + 2 * nbeams + 1, r->list);
     if (apply)
-        dd_rfi_apply_kernel<<<152 * 4, 256, 0, st>>>(bp, nbeams, (long long)ld_in_bytes, r->nchan,
+        dd_rfi_apply_kernel<<<4 * r->sms, 256, 0, st>>>(bp, nbeams, (long long)ld_in_bytes, r->nchan,
                                                      r->stats + 2 * nbeams + 1, r->list);
     return cuda_fail(cudaGetLastError(), "RFI kernels");
 }

@@ -418,12 +418,12 @@ __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_median_kernel(
 // device (32 per SM, half a segment's time lost at the end).  Measured for whole
 // searches of 1500 x 131072, h 4096, segments of 2048 / 4096 / 8192 (chosen):
 // 2718 / 2576 / 2504 us (40 warps per SM then); 16 x 100000, segments of 256 (chosen) / 4096: 142 / 167.
-unsigned row_segment(int ndm, long long n, double first) {
+unsigned row_segment(int sms, int ndm, long long n, double first) {
     unsigned best = 0;
     double least = 0;
     for (unsigned seg = 256; seg <= 32768; seg *= 2) {
         const double warps = (double)ndm * (double)((n + seg - 1) / seg);
-        const double cost = (std::max(warps / (152.0 * kMwBlocks * kMwWarps), 1.0) + 0.5) * (first + seg);
+        const double cost = (std::max(warps / ((double)sms * kMwBlocks * kMwWarps), 1.0) + 0.5) * (first + seg);
         if (!best || cost < least) {
             best = seg;
             least = cost;
@@ -1341,6 +1341,7 @@ struct Search {
     dd_search_config cfg;
     SearchCfgDev dcfg;
     int nbins = 0;
+    int sms = 0;
     int32_t *y = nullptr;
     unsigned long long *sumsq = nullptr;
     float *best = nullptr;
@@ -1419,7 +1420,10 @@ dd_status dd_search_create(dd_search **out, const dd_search_config *cfg) {
     for (int k = 0; k < c.nwidths; ++k) s->dcfg.wmask |= (unsigned)c.widths[k];
     s->nbins = 3 * c.nchan + 1;
     const size_t cells = (size_t)c.ndm_max * c.n_max;
-    cudaError_t e = cudaMalloc(&s->y, cells * 4);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaMalloc(&s->y, cells * 4);
     if (e == cudaSuccess) e = cudaMalloc(&s->sumsq, (size_t)c.ndm_max * 8);
     if (e == cudaSuccess) e = cudaMalloc(&s->best, cells * 4);
     if (e == cudaSuccess) e = cudaMalloc(&s->bestw, cells * 2);
@@ -1467,13 +1471,13 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
     const long long h = s->cfg.half_window;
     s->ntiles = (int)((n + kMfTile - 1) / kMfTile);
     if (s->cfg.baseline == 1) {
-        const unsigned seg = row_segment(ndm, (long long)n, 0.1 * (double)h);
+        const unsigned seg = row_segment(s->sms, ndm, (long long)n, 0.1 * (double)h);
         const unsigned nseg = (unsigned)(((long long)n + seg - 1) / seg);
         dd_mean_kernel<<<(unsigned)(((long long)ndm * nseg + kMwWarps - 1) / kMwWarps), 32 * kMwWarps, 0, st>>>(
             d_x, (long long)ld_x, ndm, (unsigned)n, (unsigned)h, seg, nseg, (uint32_t)(s->nbins - 1), s->y, s->ld_y,
             s->sumsq, s->st);
     } else {
-        const unsigned seg = row_segment(ndm, (long long)n, 0.3 * (double)h);
+        const unsigned seg = row_segment(s->sms, ndm, (long long)n, 0.3 * (double)h);
         const unsigned nseg = (unsigned)(((long long)n + seg - 1) / seg);
         dd_median_kernel<<<(unsigned)(((long long)ndm * nseg + kMwWarps - 1) / kMwWarps), 32 * kMwWarps, 0, st>>>(
             d_x, (long long)ld_x, ndm, (unsigned)n, (unsigned)h, seg, nseg, (uint32_t)(s->nbins - 1), s->y, s->ld_y,
@@ -1497,7 +1501,7 @@ dd_status dd_search_run(dd_search *search, const uint32_t *d_x, size_t ld_x, int
     DD_CUDA_TRY(cudaGetLastError());
     dd_tile_scan_kernel<<<(ndm + 127) / 128, 128, 0, st>>>(s->tile_sum, s->tile_off, ndm, s->ntiles);
     // grouping
-    const int g = 152 * 8;
+    const int g = s->sms * 8;
     const long long cells = (long long)ndm * (long long)n;
     dd_runs_kernel<<<ndm, 512, 0, st>>>(s->hotbits, nwr, (long long)n, s->labels, s->wl);
     // word kernels: words of a row on x, rows on y

@@ -27,3 +27,10 @@ def test_persistent_tiles_fence_before_the_next_tile():
             assert tile, path
             assert re.match(r"\s*tc::fence_async_smem\(\);\s*__syncthreads\(\);\s*}", rest[tile.end():]), path
     assert sorted(loops) == ["gsum.cu", "tiled_launch.cuh"]
+
+
+def test_no_multiprocessor_count_in_the_code():
+    """Grids and rules ask the device how many multiprocessors it has (the weight
+    gradients' number of partial sums is fixed: it sets their order)."""
+    for path in sorted(glob.glob(os.path.join(CSRC, "**", "*.cu*"), recursive=True)):
+        assert not re.search(r"\b(152|304)\b", re.sub(r"kMaxPartials = 304", "", _code(path))), path
