@@ -125,7 +125,6 @@ dd_status gsum_args(const Plan *p, size_t nsamp_in, uint32_t *d_out, size_t ld_o
     a.map = nullptr;
     a.tab = t.tab;
     a.ws = t.ws;
-    a.nchan = p->nchan;
     a.nchunks = t.nchunks;
     a.ndm = p->ndm;
     a.n_dmb = t.n_dmb;

@@ -86,7 +86,6 @@ struct Args {
     const CUtensorMap *map;  // the packed input as 32-bit words, [channel][word]
     const uint32_t *tab;  // [n_dmb][nchunks][kRecWords]
     const int32_t *ws;    // [n_dmb][2][kParts] first staged words of the first two chunks
-    int nchan;
     int nchunks;          // even; groups past the band are empty
     int ndm;
     int n_dmb;
@@ -442,7 +441,6 @@ struct BatchDesc {
     long long tile_start[DD_BATCH_MAX_BEAMS + 1];
     long long ntiles;
     int nbeams;
-    int pad;
 };
 
 }  // namespace gsum

@@ -124,15 +124,17 @@ struct ConvFwdCfg {
 // Float images of the layers' weights in the staged order, refreshed whenever
 // the parameters change: dst[cb][ci][tap][co] = w[cb*COB + co][ci][tap] for
 // every output-channel block cb, once for the wide and once for the narrow
-// blocks' COB.  A third image (cob 0) is the tensor-core kernels' bfloat16
-// operand: K-major over k = tap * ci + channel, 9 taps padded to 16 when ci = 1.
+// blocks' COB (the first layer has no narrow blocks).  A third image (cob 0) is
+// the tensor-core kernels' bfloat16 operand: K-major over k = tap * ci + channel,
+// 9 taps padded to 16 when ci = 1.
 struct WPrepLayer {
     const uint16_t *w;
     float *dst;
     int ci, cob, count;
 };
 constexpr int kImages = 3;  // wide, narrow, tensor cores
-constexpr int kImageCob[kImages][kConvLayers] = {{16, 32, 64, 64}, {16, 16, 16, 16}, {0, 0, 0, 0}};
+constexpr int kNoImage = -1;
+constexpr int kImageCob[kImages][kConvLayers] = {{16, 32, 64, 64}, {kNoImage, 16, 16, 16}, {0, 0, 0, 0}};
 constexpr int kNarrowGroups = 512;  // snippet groups of a wide launch up to which the narrow blocks run
 struct WPrepArgs {
     WPrepLayer l[kImages * kConvLayers];
@@ -1383,14 +1385,15 @@ static void free_nn(NN *p) {
 // Refresh the convolutions' float weight images from the bfloat16 parameters.
 static void refresh_images(NN *p, cudaStream_t s) {
     WPrepArgs a;
-    int most = 0;
+    int most = 0, images = 0;
     for (int i = 0; i < kImages; ++i)
         for (int l = 0; l < kConvLayers; ++l) {
+            if (kImageCob[i][l] == kNoImage) continue;
             const int count = (kImageCob[i][l] == 0 && kCin[l] == 1 ? 16 : 9 * kCin[l]) * kCout[l];
-            a.l[i * kConvLayers + l] = {p->bf + p->L.cw[l], p->wprep + p->wprep_off[i][l], kCin[l], kImageCob[i][l], count};
+            a.l[images++] = {p->bf + p->L.cw[l], p->wprep + p->wprep_off[i][l], kCin[l], kImageCob[i][l], count};
             most = std::max(most, count);
         }
-    conv_wprep_kernel<<<dim3((unsigned)((most + 255) / 256), kImages * kConvLayers), 256, 0, s>>>(a);
+    conv_wprep_kernel<<<dim3((unsigned)((most + 255) / 256), (unsigned)images), 256, 0, s>>>(a);
 }
 
 // One convolution layer in the fixed order with the tile parameters given.
@@ -1528,7 +1531,7 @@ dd_status dd_nn_create(dd_nn **out, int max_batch) {
     for (int i = 0; i < kImages; ++i)
         for (int l = 0; l < kConvLayers; ++l) {
             p->wprep_off[i][l] = wtot;
-            wtot += std::max(kCin[l] * 9, 16) * kCout[l];
+            if (kImageCob[i][l] != kNoImage) wtot += std::max(kCin[l] * 9, 16) * kCout[l];
         }
     if (e == cudaSuccess) e = cudaMalloc(&p->wprep, (size_t)wtot * 4);
     if (e == cudaSuccess) e = cudaMemset(p->wprep, 0, (size_t)wtot * 4);

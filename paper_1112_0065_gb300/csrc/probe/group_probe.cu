@@ -81,7 +81,6 @@ extern "C" dd_status dd_probe_group_tile(int withheld, unsigned poll_limit, cons
     Args a = {};
     a.tab = reinterpret_cast<uint32_t *>(buf + tab_at);
     a.ws = reinterpret_cast<int32_t *>(buf + ws_at);
-    a.nchan = kProbeChan;
     a.nchunks = t.nchunks;
     a.ndm = kD;
     a.n_dmb = 1;
