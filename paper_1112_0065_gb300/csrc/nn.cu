@@ -44,8 +44,8 @@ struct Layout {
     long long cw[kConvLayers], cb[kConvLayers], f1w, f1b, f2w, f2b, total;
 };
 
-Layout make_layout() {
-    Layout L;
+constexpr Layout make_layout() {
+    Layout L{};
     long long o = 0;
     for (int l = 0; l < kConvLayers; ++l) {
         L.cw[l] = o;
@@ -64,6 +64,8 @@ Layout make_layout() {
     L.total = o;
     return L;
 }
+// fc1's weights (bfloat16) are read, and their gradients (float) written, 16 bytes at a time
+static_assert(make_layout().f1w % 8 == 0 && kFcIn % 8 == 0, "16-byte rows of fc1");
 
 __device__ __forceinline__ float bf2f(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
 __device__ __forceinline__ uint16_t f2bf(float f) {
@@ -917,9 +919,8 @@ __global__ void __launch_bounds__(256) fc1_bwd_w_kernel(const float *__restrict_
             acc[3] = fmaf(d, f.w, acc[3]);
         }
     }
-    float *dst = g_w1 + (long long)(o0 + o) * kFcIn + i0 + iq;  // 4-byte aligned only: the flat vector is unpadded
-#pragma unroll
-    for (int k = 0; k < 4; ++k) dst[k] = acc[k];
+    *reinterpret_cast<float4 *>(g_w1 + (long long)(o0 + o) * kFcIn + i0 + iq) =
+        make_float4(acc[0], acc[1], acc[2], acc[3]);
 }
 
 // fc1 input gradient: a block owns 16 samples x 64 inputs.
