@@ -1125,9 +1125,11 @@ __global__ void __launch_bounds__((ConvBwdXCfg<CI, CO, H>::THREADS))
 // that pooling kept and the 3x3 input patch around it: a quarter of the dense
 // multiply-adds.  A sample's input sits in shared memory channel-last with a
 // zero border (a lane's 4 channels are one 8-byte load, the lanes of one
-// output channel consecutive), its (gradient, patch offset) pairs beside it.  A
-// dead window's patch is one of zeros past the bottom border: its gradient of 0
-// times an infinite or NaN input would be NaN.
+// output channel consecutive), its (gradient, patch offset) pairs beside it.  In
+// a sample with an infinite or NaN input the patch of a dead window is one of
+// zeros past the bottom border, since its gradient of 0 times such a value would
+// be NaN (in every sample: 46 instead of 41 us for the 16 -> 32 layer at 256
+// snippets, by bank conflicts).
 // A block walks samples blockIdx.x, + gridDim.x, ...; its sums (SL window
 // slices joined in order) are one partial, and conv_bwd_w_sum_kernel adds the
 // partials in order, so the result is deterministic.  Issue-bound: about 64
@@ -1170,6 +1172,7 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
 #pragma unroll 1
     for (int n = blockIdx.x; n < N; n += gridDim.x) {
         __syncthreads();  // zeros written; the previous sample consumed
+        uint32_t odd = 0;  // some input is infinite or NaN
         // input, channel-last: two neighbouring pixels of 4 channels at a time
 #pragma unroll 4
         for (int e = tid; e < C::CQ * H * (H / 2); e += T) {
@@ -1179,6 +1182,8 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
             for (int c = 0; c < 4; ++c)
                 v[c] = __ldg(reinterpret_cast<const uint32_t *>(in + (((long long)n * CI + 4 * q + c) * H + y) * H +
                                                                  2 * x2));
+#pragma unroll
+            for (int c = 0; c < 4; ++c) odd |= ((v[c] & 0x7F807F80u) + 0x00800080u) & 0x80008000u;  // exponent of ones
             unsigned char *dst = xin + ((y + 1) * (H + 2) + 2 * x2 + 1) * C::PIX + 8 * q;
             *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410));
             *reinterpret_cast<uint2 *>(dst + C::PIX) =
@@ -1189,13 +1194,16 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
             const int k = e % C::NWIN, c = e / C::NWIN;
             const long long o = ((long long)n * CO + co0 + c) * C::NWIN + k;
             const int a = __ldg(arg + o);
-            const bool on = live(__ldg(pooled + o));
             // patch around (2 yo + a/2, 2 xo + a%2): its corner in padded coordinates is that position
             const int off = ((2 * (k / HO) + (a >> 1)) * (H + 2) + 2 * (k % HO) + (a & 1)) * C::PIX;
-            const float d = __ldg(dpool + o);
-            gp[c * C::GS + k] = make_uint2(on ? __float_as_uint(d) : 0u, (uint32_t)(on ? off : C::ZERO_PATCH));
+            gp[c * C::GS + k] = make_uint2(__float_as_uint(live_grad(__ldg(dpool + o), __ldg(pooled + o))), (uint32_t)off);
         }
-        __syncthreads();
+        if (__syncthreads_or(odd != 0)) {
+            for (int e = tid; e < COB * C::NWIN; e += T)
+                if (!live(__ldg(pooled + ((long long)n * CO + co0) * C::NWIN + e)))
+                    gp[e / C::NWIN * C::GS + e % C::NWIN].y = C::ZERO_PATCH;
+            __syncthreads();
+        }
         const uint2 *g = gp + co * C::GS + sl * (C::NWIN / SL);
         const unsigned char *xb = xin + 8 * cq;
 #pragma unroll 2
@@ -1247,8 +1255,8 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
 
 // The first layer (one input channel): warp w owns output channel w, its lanes
 // the windows of a row, 9 sums each; the sample's image sits in shared memory
-// as float with a zero border, past it the zeros that dead windows read (as
-// conv_bwd_w_kernel).
+// as float with a zero border, past it the zeros that dead windows read (always:
+// 22 us at 256 snippets, 25 with their own patches).
 __global__ void __launch_bounds__(512) conv0_bwd_w_kernel(const float *__restrict__ dpool,
                                                           const uint16_t *__restrict__ pooled,
                                                           const uint8_t *__restrict__ arg,
