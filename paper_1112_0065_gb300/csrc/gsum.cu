@@ -33,8 +33,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     long long &s_tile = *reinterpret_cast<long long *>(gsum_smem + kTileWord);
     const long long ntiles = desc->ntiles;
     init_bars(gsum_smem);
-    // the maps lie in global memory, which the host writes between launches
-    if ((int)threadIdx.x < desc->nbeams) tc::fence_tensormap(&desc->map[threadIdx.x]);
+    // the maps lie in global memory, which the host writes between launches: each
+    // thread that issues copies (lane 0 of every warp) fences for itself
+    if ((threadIdx.x & 31) == 0)
+        for (int b = 0; b < desc->nbeams; ++b) tc::fence_tensormap(&desc->map[b]);
     Phases phase;
     for (;;) {
         if (threadIdx.x == 0) s_tile = (long long)atomicAdd(counter, 1ULL);

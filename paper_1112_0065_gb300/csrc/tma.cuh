@@ -22,10 +22,10 @@ __device__ __forceinline__ void tensor_copy_g2s(void *dst, const void *map, int 
         : "memory");
 }
 
-// A tensor map in global memory that was written before this kernel becomes
-// visible to the copies issued after the block's next barrier.
+// A tensor map in global memory that the host wrote before this kernel becomes
+// visible to the copies that this thread issues from here on.
 __device__ __forceinline__ void fence_tensormap(const void *map) {
-    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(map) : "memory");
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
 }
 
 }  // namespace tc

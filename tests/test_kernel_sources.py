@@ -34,3 +34,12 @@ def test_no_multiprocessor_count_in_the_code():
     gradients' number of partial sums is fixed: it sets their order)."""
     for path in sorted(glob.glob(os.path.join(CSRC, "**", "*.cu*"), recursive=True)):
         assert not re.search(r"\b(152|304)\b", re.sub(r"kMaxPartials = 304", "", _code(path))), path
+
+
+def test_tensor_maps_in_memory_are_fenced_by_the_threads_that_use_them():
+    """Tensor maps that the host copied to global memory: the acquiring fence has
+    system scope and is the issuing thread's own (lane 0 of each warp)."""
+    assert "fence.proxy.tensormap::generic.acquire.sys" in _code(os.path.join(CSRC, "tma.cuh"))
+    kernel = _code(os.path.join(CSRC, "gsum.cu")).split("dd_gsum_batch_kernel(")[1]
+    assert re.search(r"if \(\(threadIdx\.x & 31\) == 0\)\s*for \(int b = 0; b < desc->nbeams; \+\+b\) "
+                     r"tc::fence_tensormap\(&desc->map\[b\]\);", kernel)
