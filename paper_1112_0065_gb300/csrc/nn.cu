@@ -1126,10 +1126,11 @@ __global__ void __launch_bounds__((ConvBwdXCfg<CI, CO, H>::THREADS))
 // multiply-adds.  A sample's input sits in shared memory channel-last with a
 // zero border (a lane's 4 channels are one 8-byte load, the lanes of one
 // output channel consecutive), its (gradient, patch offset) pairs beside it.  In
-// a sample with an infinite or NaN input the patch of a dead window is one of
-// zeros past the bottom border, since its gradient of 0 times such a value would
-// be NaN (in every sample: 46 instead of 41 us for the 16 -> 32 layer at 256
-// snippets, by bank conflicts).
+// a sample with an infinite input (after a ReLU there is no NaN) the patch of a
+// dead window is one of zeros past the bottom border, since its gradient of 0
+// times infinity would be NaN.  (The 16 -> 32 layer at 256 snippets: 41 us
+// without, 42.5 so, 46 with every sample's dead windows there, by bank
+// conflicts.)
 // A block walks samples blockIdx.x, + gridDim.x, ...; its sums (SL window
 // slices joined in order) are one partial, and conv_bwd_w_sum_kernel adds the
 // partials in order, so the result is deterministic.  Issue-bound: about 64
@@ -1172,7 +1173,7 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
 #pragma unroll 1
     for (int n = blockIdx.x; n < N; n += gridDim.x) {
         __syncthreads();  // zeros written; the previous sample consumed
-        uint32_t odd = 0;  // some input is infinite or NaN
+        uint32_t top = 0;  // largest inputs of even and odd pixels (after the ReLU: none negative)
         // input, channel-last: two neighbouring pixels of 4 channels at a time
 #pragma unroll 4
         for (int e = tid; e < C::CQ * H * (H / 2); e += T) {
@@ -1183,7 +1184,7 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
                 v[c] = __ldg(reinterpret_cast<const uint32_t *>(in + (((long long)n * CI + 4 * q + c) * H + y) * H +
                                                                  2 * x2));
 #pragma unroll
-            for (int c = 0; c < 4; ++c) odd |= ((v[c] & 0x7F807F80u) + 0x00800080u) & 0x80008000u;  // exponent of ones
+            for (int c = 0; c < 4; ++c) top = __vmaxu2(top, v[c]);
             unsigned char *dst = xin + ((y + 1) * (H + 2) + 2 * x2 + 1) * C::PIX + 8 * q;
             *reinterpret_cast<uint2 *>(dst) = make_uint2(__byte_perm(v[0], v[1], 0x5410), __byte_perm(v[2], v[3], 0x5410));
             *reinterpret_cast<uint2 *>(dst + C::PIX) =
@@ -1198,7 +1199,7 @@ __global__ void __launch_bounds__((ConvBwdWCfg<CI, CO, H, COB, SL>::THREADS), 2)
             const int off = ((2 * (k / HO) + (a >> 1)) * (H + 2) + 2 * (k % HO) + (a & 1)) * C::PIX;
             gp[c * C::GS + k] = make_uint2(__float_as_uint(live_grad(__ldg(dpool + o), __ldg(pooled + o))), (uint32_t)off);
         }
-        if (__syncthreads_or(odd != 0)) {
+        if (__syncthreads_or((top & 0xFFFFu) >= 0x7F80u || top >= 0x7F800000u)) {
             for (int e = tid; e < COB * C::NWIN; e += T)
                 if (!live(__ldg(pooled + ((long long)n * CO + co0) * C::NWIN + e)))
                     gp[e / C::NWIN * C::GS + e % C::NWIN].y = C::ZERO_PATCH;

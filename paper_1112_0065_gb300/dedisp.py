@@ -23,8 +23,9 @@ def _stream_handle(stream):
         # the current stream's handle without the Stream object around it,
         # which took 2.8 us of a short gulp's 13 on the Grace host; PyTorch
         # promises only the object
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-        if raw is None:
+        try:
+            raw = torch._C._cuda_getCurrentRawStream
+        except AttributeError:
             return torch.cuda.current_stream().cuda_stream
         return raw(torch.cuda.current_device())
     return stream.cuda_stream
