@@ -211,12 +211,16 @@ typedef struct dd_batch dd_batch;
 #define DD_BATCH_MAX_BEAMS 64
 
 /*
- * Create a batch for nbeams (1..DD_BATCH_MAX_BEAMS) beams.  All beams run the
- * tiled kernel with one tile shape (the first beam's plan's shape).  With
- * use_graph != 0 the launch (work-counter reset + persistent kernel) is
+ * Create a batch for nbeams (1..DD_BATCH_MAX_BEAMS) beams.  All beams run one
+ * kernel: the channel-group one where the plans and the sum of the beams suit
+ * it, else the tiled one with one tile shape (the first beam's plan's).  A batch
+ * created on beams of the channel-group kernel launches both, one of them with
+ * an empty work list, and so takes beams of either kind from dd_batch_set; one
+ * created on beams of the tiled kernel stays with that kernel.  With
+ * use_graph != 0 the launch (work-counter reset + persistent kernels) is
  * captured once in a CUDA graph and replayed by dd_batch_launch.  The beam
  * descriptors are uploaded synchronously.  The batch owns its device
- * descriptor block and work counter; its descriptors point at the plans'
+ * descriptor blocks and work counters; its descriptors point at the plans'
  * tables, so every plan of the batch must outlive it (dd_plan_autotune on
  * such a plan keeps those tables).  The input and output buffers belong to
  * the caller and must stay valid while launches may run.

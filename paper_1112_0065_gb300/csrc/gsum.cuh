@@ -19,8 +19,8 @@
 // words of the packed 2-bit input become the low and the high plane with four
 // operations and no transpose.
 //
-// Bound by the ALU pipe, which the logic ops and the shifts share: 77 % busy at
-// 1024 channels x 1500 trials x 131072 outputs, 2378 us against 2775 us for the
+// Bound by the ALU pipe, which the logic ops and the shifts share: 78 % busy at
+// 1024 channels x 1500 trials x 131072 outputs, 2373 us against 2780 us for the
 // tiled kernel (1.12e9 ALU warp instructions against 1.52e9 at 88 %); the rest
 // is the warps' waiting for one another's shares of a chunk.  A barrier a chunk
 // took 2739 us, two chunks of slack and smaller chunks 2390, vectors copied

@@ -34,10 +34,12 @@ struct BeamPtrs {
 // Five channels (at most 15) are added in nibbles, even and odd samples apart,
 // then widened into byte lanes: acc[4*kw + i] byte j sums sample 16kw + 4j + i
 // of the group.  That is 7 integer operations per 16-sample word against 12
-// when every word is widened at once, which kept the kernel at 5.3 TB/s (13
-// beams of 1024 channels x 151536 samples, 504 MB: 95 us of the 109 us run,
-// which takes 102 us now); ten loads are in flight per thread, and CTAs of 512
-// samples leave a shorter last wave than 1024 (104 us).  The slices' byte sums meet in shared memory, where thread r
+// when every word is widened at once (13 beams of 1024 channels x 151536
+// samples, 504 MB: 95 us of the 109 us run then, 91 of 102 now); ten loads are in
+// flight per thread, and CTAs of 512 samples leave a shorter last wave than 1024
+// (104 us).  Bound by how fast DRAM answers: 5.5 TB/s of the copy's 6.8, warps
+// wait for loads in 19 of 25 cycles per issue, the ALU pipe is 49 % busy and issue
+// slots 29 %; a CTA reads 128 bytes of each row, rows 38 KB apart.  The slices' byte sums meet in shared memory, where thread r
 // (group r/16, word kw, lane i) adds its four samples over the slices in
 // 16-bit lanes (at most 3 * 21844 < 2^16), then sum z and sum z^2.
 constexpr int kZdSlices = 16;  // channel slices per pass (64 channels each)

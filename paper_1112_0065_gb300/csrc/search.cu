@@ -452,7 +452,9 @@ __device__ __forceinline__ uint32_t udiv_by(uint32_t a, uint32_t m, uint32_t inv
 // and nothing but y written; a block that staged 8192 outputs with both windows'
 // values and scanned them in shared memory (what this replaces) read and added
 // every value twice: 253 us for 700 x 100003 with window 8192, now 204 (0.56 GB,
-// 82 us; bound by instruction issue, the scan and the division).
+// 82 us).  Issue slots are 62 % taken, 64 thread instructions per output; the
+// rest is the latency of the scan's five steps, of which a warp has four side by
+// side, with 28 warps on an SM.
 __global__ void __launch_bounds__(32 * kMwWarps, kMwBlocks) dd_mean_kernel(
     const uint32_t *__restrict__ x, long long ld_x, int ndm, unsigned n, unsigned h, unsigned seg, unsigned nseg,
     uint32_t top, int32_t *__restrict__ y, long long ld_y, unsigned long long *__restrict__ sumsq, DevState *st) {
